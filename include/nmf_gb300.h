@@ -162,7 +162,8 @@ nmf_status nmf_nls_bpp_tune(const nmf_nls_desc *d, void *stream, int32_t *warps,
 /* Sets the launch shape of every later solve of this k in the process, as the
  * tuner would (an interface of this library): warps per CTA 1..16 (the FP64
  * solves use at most 8), right-hand sides per grab of the work counter
- * 1..1024, and the group-tile pass of FP32 half-steps (right-hand sides whose
+ * 1..1024 (fewer where the batch is too small to give every warp several
+ * grabs), and the group-tile pass of FP32 half-steps (right-hand sides whose
  * first candidate partition is all usable indices are solved together by
  * tile products with the preparation's inverse; the rest go to the per-warp
  * solves): group = 0 off, 1 on the SIMT pipes, 2 on the tensor cores (k <=

@@ -900,10 +900,12 @@ nmf_status launch_solve(const SolveParams &P, int list_pass, cudaStream_t s)
     int64_t blocks = (int64_t)per_sm * sm_count();
     // The second pass's size is known only on the device: launch it at full
     // width; it returns at once when nothing was deferred.
-    const int64_t need = list_pass ? blocks : cdiv(cdiv(P.nrhs, (int64_t)P.chunk), nwarps);
+    SolveParams Q = P;
+    Q.chunk = grab_size(P, blocks * nwarps);
+    const int64_t need = list_pass ? blocks : cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), nwarps);
     if (need < blocks)
         blocks = need < 1 ? 1 : need;
-    bpp_solve_kernel<KW, PT, MODE><<<(unsigned)blocks, nwarps * 32, smem, s>>>(P, pmax, LS,
+    bpp_solve_kernel<KW, PT, MODE><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, pmax, LS,
                                                                               staged, list_pass);
     NMF_LAUNCHED("bpp_solve_kernel");
     return NMF_OK;

@@ -858,10 +858,12 @@ nmf_status launch32(const SolveParams &P, cudaStream_t s)
     if (per_sm < 1)
         return NMF_ERR_INVALID_ARG;
     int64_t blocks = (int64_t)per_sm * sm_count();
-    const int64_t need = cdiv(cdiv(P.nrhs, (int64_t)P.chunk), nwarps);
+    SolveParams Q = P;
+    Q.chunk = grab_size(P, blocks * nwarps);
+    const int64_t need = cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), nwarps);
     if (need < blocks)
         blocks = need < 1 ? 1 : need;
-    bpp_solve32_kernel<KW, PM><<<(unsigned)blocks, nwarps * 32, smem, s>>>(P, pmax, LS);
+    bpp_solve32_kernel<KW, PM><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, pmax, LS);
     NMF_LAUNCHED("bpp_solve32_kernel");
     return NMF_OK;
 }

@@ -123,7 +123,7 @@ __host__ __device__ inline size_t group_smem(int k, int TR)
 }
 
 __global__ void __launch_bounds__(GT_THREADS)
-    bpp_group_kernel(const SolveParams P, int TR)
+    bpp_group_kernel(const SolveParams P, int TR, int SPT)
 {
     if (P.flags[0] != 0)
         return;   // not an FP32 half-step
@@ -175,11 +175,11 @@ __global__ void __launch_bounds__(GT_THREADS)
             pf[m] = e < TR * k4 && r < tnr && i < k ? P.B[(t0 + r) * k + i] : 0.0f;
         }
     };
-    // Tiles are taken in spans of SPT consecutive tiles (GT_THREADS
+    // Tiles are taken in spans of SPT consecutive tiles (at most GT_THREADS
     // right-hand sides). With a warm start the passive sets decide membership
     // without reading B: one thread per right-hand side of the span, one
     // round of loads for SPT tiles.
-    const int SPT = GT_THREADS / TR;
+    const int span = SPT * TR;
     const int64_t nspans = cdiv(ntiles, (int64_t)SPT);
     const bool pretest = P.pin || P.max_rounds < 1 || nU == 0;
     __shared__ int tcount[GT_THREADS / 32];   // members per tile of the span (SPT <= 16)
@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(GT_THREADS)
             if (tid < SPT)
                 tcount[tid] = 0;
             __syncthreads();
-            const int64_t j = sp * GT_THREADS + tid;
-            if (j < P.nrhs && nU > 0 && P.pin) {
+            const int64_t j = sp * span + tid;
+            if (tid < span && j < P.nrhs && nU > 0 && P.pin) {
                 memb = 1;
                 for (int w = 0; w < P.nwords; ++w)
                     if ((P.pin[j * P.nwords + w] & umask[w]) != umask[w])
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(GT_THREADS)
             const int min_members = (nr + 1) / 2;
             if (pretest && tcount[ts] < min_members) {
                 if (memb && tid / TR == ts)
-                    reinterpret_cast<uint32_t *>(P.X)[(sp * GT_THREADS + tid) * k] = GROUP_PENDING;
+                    reinterpret_cast<uint32_t *>(P.X)[(sp * span + tid) * k] = GROUP_PENDING;
                 if (tid == 0)
                     pending += nr;
                 continue;
@@ -362,8 +362,13 @@ __global__ void __launch_bounds__(GT_THREADS)
 
 nmf_status launch_group32(const SolveParams &P, cudaStream_t s)
 {
+    // 64-wide tiles where the shared memory allows them and the batch has one
+    // for every SM, else 32-wide ones: a CTA works through its tiles in turn,
+    // so a small batch takes as long as its longest span (k = 10, 2000
+    // right-hand sides: 55 us in spans of eight 64-wide tiles; k = 50, 16000:
+    // 120 us).
     int TR = 64;
-    if (group_smem(P.k, TR) > SMEM_LIMIT_GT)
+    if (group_smem(P.k, TR) > SMEM_LIMIT_GT || P.nrhs <= (int64_t)TR * sm_count())
         TR = 32;
     const size_t smem = group_smem(P.k, TR);
     if (smem > SMEM_LIMIT_GT)
@@ -376,10 +381,18 @@ nmf_status launch_group32(const SolveParams &P, cudaStream_t s)
     if (per_sm < 1)
         return NMF_ERR_INVALID_ARG;
     int64_t blocks = (int64_t)per_sm * sm_count();
-    const int64_t spans = cdiv(P.nrhs, (int64_t)GT_THREADS);   // GT_THREADS / TR tiles each
+    // Spans of up to GT_THREADS right-hand sides, shorter where that leaves
+    // CTAs without one.
+    const int64_t ntiles = cdiv(P.nrhs, (int64_t)TR);
+    int64_t spt = ntiles / blocks;
+    if (spt > GT_THREADS / TR)
+        spt = GT_THREADS / TR;
+    if (spt < 1)
+        spt = 1;
+    const int64_t spans = cdiv(ntiles, spt);
     if (spans < blocks)
         blocks = spans < 1 ? 1 : spans;
-    bpp_group_kernel<<<(unsigned)blocks, GT_THREADS, smem, s>>>(P, TR);
+    bpp_group_kernel<<<(unsigned)blocks, GT_THREADS, smem, s>>>(P, TR, (int)spt);
     NMF_LAUNCHED("bpp_group_kernel");
     return NMF_OK;
 }

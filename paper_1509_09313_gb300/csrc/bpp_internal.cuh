@@ -67,6 +67,17 @@ struct SolveParams {
     CsrGather gat;
 };
 
+// Right-hand sides per grab of the work counter: the shape's, less where the
+// batch would not give each of `warps` resident warps four grabs. A warp solves
+// a grab's right-hand sides one after the other, so in a small batch the grab
+// is the whole run time (1000 right-hand sides, k = 10: 45 us in grabs of
+// eight).
+inline int grab_size(const SolveParams &P, int64_t warps)
+{
+    const int64_t share = P.nrhs / (4 * warps);
+    return (int)(share < 1 ? 1 : share < P.chunk ? share : P.chunk);
+}
+
 __device__ __forceinline__ unsigned lanemask_lt(int lane) { return (1u << lane) - 1u; }
 
 template <typename T>
