@@ -49,6 +49,7 @@
 // (right-hand sides in, solutions out) plus bitmasks.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "bpp_internal.cuh"
@@ -564,34 +565,24 @@ __host__ __device__ inline size_t mats_bytes(int k, int mode)
     return (b + 15) & ~size_t(15);
 }
 
-// FP64 solves. KW = index slots per lane (k <= 32 KW); PT = compact-system
-// rows per lane (pmax <= 32 PT). The kernel of each MODE returns at once
-// unless the prep kernel chose that mode, so the host never waits for the
-// decision. With list_pass set (MODE 1 only) it is the second pass of mode 0:
-// it re-solves, from their starting partitions, the right-hand sides that the
-// FP32 kernel deferred (all of them if more than DEFER_CAP were).
+// How a mode's FP64 solves use the CTA: systems of up to pmax rows (row stride
+// LS), warps that solve (the others of the CTA return), G and M staged in
+// shared memory or not.
+struct Solve64Shape {
+    int pmax, LS, warps, staged;
+};
+
+// FP64 solves of one mode. KW = index slots per lane (k <= 32 KW); PT =
+// compact-system rows per lane (pmax <= 32 PT). The right-hand sides are pin's
+// batch, or, with use_list, those the FP32 kernel deferred.
 template <int KW, int PT, int MODE>
-__global__ void __launch_bounds__(BPP_THREADS, 2)
-    bpp_solve_kernel(const SolveParams P, int pmax, int LS, int staged, int list_pass)
+__device__ __forceinline__ void solve64(const SolveParams &P, const Solve64Shape &sh,
+                                        const uint64_t *__restrict__ pin, int64_t nwork,
+                                        bool use_list, unsigned long long *counter)
 {
     using T = double;
     constexpr bool HAVE_M = MODE != 2;
-    int64_t nwork = P.nrhs;
-    bool use_list = false;
-    unsigned long long *counter = &P.counters[CNT_WORK];
-    if (list_pass) {
-        if (P.flags[0] != 0)
-            return;
-        // Written by the FP32 kernel earlier in the same stream.
-        const unsigned long long nd = P.counters[CNT_DEFERRED];
-        if (nd == 0)
-            return;
-        use_list = nd <= (unsigned long long)DEFER_CAP;
-        nwork = use_list ? (int64_t)nd : P.nrhs;
-        counter = &P.counters[CNT_DEFER_WORK];
-    } else if (P.flags[0] != MODE) {
-        return;
-    }
+    const int pmax = sh.pmax, LS = sh.LS, staged = sh.staged;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = P.k;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -621,6 +612,8 @@ __global__ void __launch_bounds__(BPP_THREADS, 2)
     T *stage = invd + 128;
     T *Lw = stage + 128;
     __syncthreads();
+    if (warp >= sh.warps)
+        return;
 
     bool usable[KW];
     int nU = 0;
@@ -666,13 +659,13 @@ __global__ void __launch_bounds__(BPP_THREADS, 2)
                     x[s] = 0;
             } else {
                 // Starting partition: empty (cold) or the given bitmask (warm).
-                if (P.pin) {
+                if (pin) {
 #pragma unroll
                     for (int s = 0; s < KW; ++s) {
                         const int i = lane + 32 * s;
                         bool f = false;
                         if (i < k) {
-                            const uint64_t wv = P.pin[j * P.nwords + (i >> 6)];
+                            const uint64_t wv = pin[j * P.nwords + (i >> 6)];
                             f = (wv >> (i & 63)) & 1ull;
                         }
                         inF[s] = f && usable[s];
@@ -869,50 +862,96 @@ __global__ void __launch_bounds__(BPP_THREADS, 2)
     }
 }
 
-constexpr size_t SMEM_LIMIT = 227 * 1024;
+// One launch for every FP64 case, so that the host never waits for the mode the
+// preparation chose and an FP32 half-step pays for one kernel that returns at
+// once instead of three (2.4 us each): mode 1 (from the predicted partitions
+// where the FP32 kernel made them), mode 2, and, in mode 0, the second pass
+// that re-solves, from their starting partitions, the right-hand sides the FP32
+// kernel deferred (all of them if more than DEFER_CAP were).
+template <int KW>
+__global__ void __launch_bounds__(BPP_THREADS, 2)
+    bpp_solve_kernel(const SolveParams P, const Solve64Shape sh1, const Solve64Shape sh2)
+{
+    const int mode = P.flags[0];
+    if (mode == 2) {
+        solve64<KW, KW, 2>(P, sh2, P.pin, P.nrhs, false, &P.counters[CNT_WORK]);
+        return;
+    }
+    int64_t nwork = P.nrhs;
+    bool use_list = false;
+    const uint64_t *pin = P.pin;
+    unsigned long long *counter = &P.counters[CNT_WORK];
+    if (mode == 0) {
+        // Written by the FP32 kernel earlier in the same stream.
+        const unsigned long long nd = P.counters[CNT_DEFERRED];
+        if (nd == 0)
+            return;
+        use_list = nd <= (unsigned long long)DEFER_CAP;
+        nwork = use_list ? (int64_t)nd : P.nrhs;
+        counter = &P.counters[CNT_DEFER_WORK];
+    } else if (P.predict) {
+        pin = P.pout;
+    }
+    solve64<KW, (KW + 1) / 2, 1>(P, sh1, pin, nwork, use_list, counter);
+}
 
-template <int KW, int PT, int MODE>
-nmf_status launch_solve(const SolveParams &P, int list_pass, cudaStream_t s)
+constexpr size_t SMEM_LIMIT = 227 * 1024;
+constexpr size_t SMEM_HALF = 112 * 1024;   // two CTAs per SM
+
+template <int KW>
+nmf_status launch_solve64(const SolveParams &P, cudaStream_t s)
 {
     const int k = P.k;
-    int pmax = MODE == 2 ? k : k / 2;
-    if (pmax < 1)
-        pmax = 1;
-    const int LS = pmax | 1;   // odd row stride: conflict-free lane-per-row reads
-    int nwarps = P.warps < BPP_WARPS ? P.warps : BPP_WARPS;
-    // Stage G and M in shared memory when they leave room for >= 2 warps.
-    const int staged = MODE != 2 &&
-                       mats_bytes(k, MODE) + 2 * per_warp_bytes(pmax, LS) <= SMEM_LIMIT;
-    const size_t mats = staged ? mats_bytes(k, MODE) : 0;
-    auto bytes = [&](int nw) { return mats + (size_t)nw * per_warp_bytes(pmax, LS); };
-    while (nwarps > 1 && bytes(nwarps) > SMEM_LIMIT)
-        --nwarps;
-    const size_t smem = bytes(nwarps);
+    const int warps = P.warps < BPP_WARPS ? P.warps : BPP_WARPS;
+    Solve64Shape sh1, sh2;
+    sh1.pmax = k / 2 < 1 ? 1 : k / 2;
+    sh2.pmax = k;
+    sh1.LS = sh1.pmax | 1;   // odd row stride: conflict-free lane-per-row reads
+    sh2.LS = sh2.pmax | 1;
+    // Mode 1 stages G and M in shared memory when they leave room for >= 2
+    // warps.
+    const size_t pw1 = per_warp_bytes(sh1.pmax, sh1.LS), pw2 = per_warp_bytes(sh2.pmax, sh2.LS);
+    sh1.staged = mats_bytes(k, 1) + 2 * pw1 <= SMEM_LIMIT;
+    sh2.staged = 0;
+    const size_t mats = sh1.staged ? mats_bytes(k, 1) : 0;
+    sh1.warps = warps;
+    while (sh1.warps > 1 && mats + sh1.warps * pw1 > SMEM_LIMIT)
+        --sh1.warps;
+    size_t smem = mats + sh1.warps * pw1;
+    // Mode 2 (larger systems per warp) takes the warps that fit beside it, in
+    // at least half an SM's shared memory.
+    const size_t want2 = warps * pw2 < SMEM_HALF ? warps * pw2 : SMEM_HALF;
+    if (smem < want2)
+        smem = want2;
+    if (smem < pw2)
+        smem = pw2;
     if (smem > SMEM_LIMIT)
         return NMF_ERR_INVALID_ARG;
+    sh2.warps = (int)(smem / pw2) < warps ? (int)(smem / pw2) : warps;
+    const int nwarps = sh1.warps > sh2.warps ? sh1.warps : sh2.warps;
     static SmemOptIn opt_in;
-    NMF_TRY(ensure_smem(bpp_solve_kernel<KW, PT, MODE>, opt_in, smem));
+    NMF_TRY(ensure_smem(bpp_solve_kernel<KW>, opt_in, smem));
     int per_sm = 0;
-    NMF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, bpp_solve_kernel<KW, PT, MODE>, nwarps * 32, smem));
+    NMF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bpp_solve_kernel<KW>,
+                                                           nwarps * 32, smem));
     if (per_sm < 1)
         return NMF_ERR_INVALID_ARG;
     int64_t blocks = (int64_t)per_sm * sm_count();
-    // The second pass's size is known only on the device: launch it at full
-    // width; it returns at once when nothing was deferred.
     SolveParams Q = P;
     Q.chunk = grab_size(P, blocks * nwarps);
-    const int64_t need = list_pass ? blocks : cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), nwarps);
+    // As many CTAs as the batch has grabs for (the second pass's size is known
+    // only on the device).
+    const int64_t need =
+        cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), std::min(sh1.warps, sh2.warps));
     if (need < blocks)
         blocks = need < 1 ? 1 : need;
-    bpp_solve_kernel<KW, PT, MODE><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, pmax, LS,
-                                                                              staged, list_pass);
+    bpp_solve_kernel<KW><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, sh1, sh2);
     NMF_LAUNCHED("bpp_solve_kernel");
     return NMF_OK;
 }
 
 template <int KW>
-nmf_status launch_modes(const SolveParams &P, cudaStream_t s)
+nmf_status launch_modes(SolveParams P, cudaStream_t s)
 {
     // Mode 0 (FP32): the group-tile pass for the all-passive group first,
     // then the per-warp solves of what it left.
@@ -922,27 +961,18 @@ nmf_status launch_modes(const SolveParams &P, cudaStream_t s)
         else
             NMF_TRY(launch_group32(P, s));
     }
-    NMF_TRY(launch_solve32(P, s));
     if (P.fused) {
-        // FP64 half-step: the right-hand sides are formed here instead.
+        // FP64 half-step: the right-hand sides are formed here instead of
+        // inside the FP32 solves.
         NMF_TRY(launch_spmm_unless_fp32(P.gat.rowptr, P.gat.colidx, P.gat.vals, P.nrhs, P.gat.F,
                                         P.k, const_cast<float *>(P.B), P.flags, s));
     }
-    // Mode 1 (FP64): an FP32 pass first predicts each right-hand side's
+    // Mode 1 (FP64): the FP32 kernel first predicts each right-hand side's
     // partition into pout, and the FP64 solves start from it (their answer
     // does not depend on the start; they need fewer rounds).
-    SolveParams P1 = P;
-    if (P.pout && P.max_rounds >= 2 * PREDICT_ROUNDS) {   // (a tight cap keeps its meaning)
-        SolveParams Q = P;
-        Q.predict = 1;
-        Q.group = 0;
-        Q.fused = 0;
-        NMF_TRY(launch_solve32(Q, s));
-        P1.pin = P.pout;
-    }
-    NMF_TRY((launch_solve<KW, (KW + 1) / 2, 1>(P1, 0, s)));
-    NMF_TRY((launch_solve<KW, KW, 2>(P, 0, s)));
-    return launch_solve<KW, (KW + 1) / 2, 1>(P, 1, s);
+    P.predict = P.pout && P.max_rounds >= 2 * PREDICT_ROUNDS;   // (a tight cap keeps its meaning)
+    NMF_TRY(launch_solve32(P, s));
+    return launch_solve64<KW>(P, s);
 }
 
 }  // namespace

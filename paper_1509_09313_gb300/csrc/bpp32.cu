@@ -379,16 +379,18 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
 {
     constexpr int RS = 32 * KW;
     constexpr int PT = (KW + 1) / 2;
-    if (P.predict ? P.flags[0] != 1 : P.flags[0] != 0)
+    const int mode = P.flags[0];
+    const bool predict = mode == 1 && P.predict;
+    if (mode != 0 && !predict)
         return;
-    const bool fused = P.fused && !P.predict;
-    const bool group = P.group && !P.predict && !fused;   // no group-tile pass before fused solves
+    const bool fused = P.fused && !predict;   // (the SpMM has formed B for an FP64 half-step)
+    const bool group = P.group && !predict && !fused;   // no group-tile pass before fused solves
     if (group && P.counters[CNT_PENDING] == 0)
         return;   // the group-tile pass solved them all
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = P.k, k4 = (k + 3) & ~3;
-    const int max_rounds = P.predict ? PREDICT_ROUNDS : P.max_rounds;
-    unsigned long long *counter = &P.counters[P.predict ? CNT_PREDICT : CNT_WORK];
+    const int max_rounds = predict ? PREDICT_ROUNDS : P.max_rounds;
+    unsigned long long *counter = &P.counters[predict ? CNT_PREDICT : CNT_WORK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float *Gs = reinterpret_cast<float *>(smem_raw);
     float *Ms = Gs + k4 * RS;
@@ -751,7 +753,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         status = NMF_ERR_NONFINITE;
                 }
             }
-            if (P.predict) {
+            if (predict) {
                 // Only the partition reached seeds the FP64 solves; where the
                 // FP32 system was singular, the starting one (given or empty).
                 if (P.pout) {

@@ -51,9 +51,10 @@ struct SolveParams {
     unsigned long long *counters;  // CNT_WORDS words
     int64_t *defer;                // DEFER_CAP indices
     BppStats *stats;
-    // predict = 1: an FP64 (mode 1) half-step's FP32 pass that only writes
-    // passive sets (pout) for the FP64 solves to start from; no X, rounds,
-    // status or statistics, at most PREDICT_ROUNDS rounds, its own counter.
+    // predict = 1: in an FP64 (mode 1) half-step the FP32 kernel runs too, and
+    // only writes passive sets (pout) for the FP64 solves to start from; no X,
+    // rounds, status or statistics, at most PREDICT_ROUNDS rounds, its own
+    // counter.
     int predict;
     // group = 1: the group-tile pass ran first; the per-warp kernel solves
     // only the right-hand sides it marked GROUP_PENDING.
@@ -88,8 +89,8 @@ __device__ __forceinline__ T warp_max(T v)
     return v;
 }
 
-// FP32 solve kernel (mode 0): launched for every half-step, returns at once
-// unless the prep kernel chose mode 0.
+// FP32 solve kernel (mode 0; mode 1 where P.predict): launched for every
+// half-step, returns at once in the other modes.
 nmf_status launch_solve32(const SolveParams &P, cudaStream_t s);
 
 // Group-tile pass for the all-passive group (mode 0; returns at once
