@@ -599,7 +599,13 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
         if (ok) {
             fold();
             const int64_t p = p0 + row;
-            float *o = args.out + (int64_t)blockIdx.y * P * args.k + p * args.k + args.col0 + cbase;
+            const int64_t len = P * args.k;
+            // A split of the pass with the objective keeps its compensation too
+            // (two arrays per split), so that the sum over the splits rounds
+            // like the unsplit pass.
+            const bool pair = OBJ && gridDim.y > 1;
+            float *o = args.out + (int64_t)blockIdx.y * (pair ? 2 * len : len) + p * args.k +
+                       args.col0 + cbase;
 #pragma unroll
             for (int c0 = 0; c0 < NH; c0 += CH) {
                 float sm[CH], cm[CH];
@@ -608,8 +614,11 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
                 if (p < P) {
 #pragma unroll
                     for (int i = 0; i < CH; ++i)
-                        if (cbase + c0 + i < args.kc)
-                            o[c0 + i] = sm[i] - cm[i];
+                        if (cbase + c0 + i < args.kc) {
+                            o[c0 + i] = pair ? sm[i] : sm[i] - cm[i];
+                            if (pair)
+                                o[len + c0 + i] = -cm[i];
+                        }
                 }
             }
         }
@@ -625,7 +634,7 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
             double s = 0.0;
             for (int w = 0; w < 4; ++w)
                 s += red[w];
-            args.obj_partials[blockIdx.x] = s;
+            args.obj_partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
         }
     }
     if (warp == 1) {
@@ -759,7 +768,8 @@ __global__ void mm_tc_split_rows_kernel(const float *__restrict__ X, int64_t row
     lo[e] = __float2bfloat16_rn(v - __bfloat162float(h));
 }
 
-// out[p][col0 + c] = sum over splits of part[s][p][col0 + c], in split order.
+// out[p][col0 + c] = sum over the partial arrays of part[s][p][col0 + c], in
+// order.
 __global__ void mm_tc_reduce_kernel(const float *__restrict__ part, int splits, int64_t P, int k,
                                     int col0, int kc, float *__restrict__ out)
 {
@@ -829,7 +839,10 @@ struct TcWork {
 
 constexpr int TC_MAX_SPLITS = 16;   // tall-skinny A: few output tiles, a long contraction
 
-// Contraction splits that fill the last wave of CTAs better (1 CTA per SM).
+// Contraction splits that fill the last wave of CTAs better (1 CTA per SM),
+// with and without the objective (each split sums its own columns' residuals:
+// 24000 x 16000, k = 50 with the objective took 392 us in 188 CTAs, against
+// 243 us for the product alone in 752).
 int choose_splits(int64_t P, int64_t Q)
 {
     const int64_t tiles = cdiv(P, TC_BM), nkb = cdiv(Q, TC_BK);
@@ -864,12 +877,13 @@ TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj)
     if (obj)
         off += al(2 * sizeof(__nv_bfloat16) * (size_t)Pp * 64);
     w.part_off = off;
+    const int splits = choose_splits(P, Q);
     if (obj)
-        off += al(sizeof(double) * (size_t)(Pp / TC_BM));
+        off += al(sizeof(double) * (size_t)(Pp / TC_BM) * (size_t)splits);
     w.split_off = off;
-    const int splits = obj ? 1 : choose_splits(P, Q);
     if (splits > 1)
-        off += al(sizeof(float) * (size_t)splits * (size_t)(P > 0 ? P : 1) * (size_t)k);
+        off += al(sizeof(float) * (size_t)(obj ? 2 * splits : splits) *
+                  (size_t)(P > 0 ? P : 1) * (size_t)k);
     w.total = off;
     return w;
 }
@@ -982,9 +996,11 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
         a.col0 = col0;
         a.kc = kc;
         const bool fuse = obj && col0 == 0;
-        const int splits = fuse ? 1 : choose_splits(P, Q);
+        const int splits = choose_splits(P, Q);
         const int nkb = (int)cdiv(Q, TC_BK);
         a.kb_per_split = (int)cdiv(nkb, splits);
+        if (fuse)   // whole folds: the partial sums of the unsplit pass
+            a.kb_per_split = (int)cdiv(a.kb_per_split, TC_FOLD) * TC_FOLD;
         const int grid_y = (int)cdiv(nkb, a.kb_per_split);
         float *partial = reinterpret_cast<float *>(wb + wl.split_off);
         a.out = grid_y > 1 ? partial : out;
@@ -997,12 +1013,12 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
             st = presplit ? launch_tc_n<3, 0>(N, maps, a, s) : launch_tc_n<0, 0>(N, maps, a, s);
         NMF_TRY(st);
         if (grid_y > 1) {
-            mm_tc_reduce_kernel<<<(unsigned)cdiv(P * kc, 256), 256, 0, s>>>(partial, grid_y, P, k,
-                                                                            col0, kc, out);
+            mm_tc_reduce_kernel<<<(unsigned)cdiv(P * kc, 256), 256, 0, s>>>(
+                partial, fuse ? 2 * grid_y : grid_y, P, k, col0, kc, out);
             NMF_LAUNCHED("mm_tc_reduce_kernel");
         }
         if (fuse) {
-            obj_sum_kernel<<<1, 256, 0, s>>>(a.obj_partials, (int)(Pp / TC_BM), f_dev);
+            obj_sum_kernel<<<1, 256, 0, s>>>(a.obj_partials, (int)(Pp / TC_BM) * grid_y, f_dev);
             NMF_LAUNCHED("obj_sum_kernel");
         }
     }
