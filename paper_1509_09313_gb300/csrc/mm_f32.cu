@@ -385,7 +385,7 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
             double s = 0.0;
             for (int w = 0; w < NT / 32; ++w)
                 s += red[w];
-            obj_part[blockIdx.x] = s;
+            obj_part[blockIdx.z * gridDim.x + blockIdx.x] = s;
         }
     }
 }
@@ -475,7 +475,7 @@ struct F32Plan {
     size_t f_off, part_off, split_off, total;
 };
 
-F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool obj)
+F32Plan f32_plan(int64_t m, int64_t n, int k, int trans)
 {
     F32Plan w;
     w.P = trans ? n : m;
@@ -486,16 +486,18 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool obj)
     w.kpt = w.kp * w.nch;
     w.bp = 16 * (trans ? RPT1 : RPT0);
     w.ldf = trans ? w.kpt : cdiv(w.Q > 0 ? w.Q : 1, 4) * 4;
-    // A^T W splits its contraction (up to 16 ways, each split keeping at
-    // least 8 stages) so that its CTAs fill whole waves of two per SM: the
-    // fewest splits within 2% of the best wave efficiency. A H^T never
-    // splits, so that its products are the same with and without the fused
-    // objective.
+    // The contraction is split (up to 16 ways, each split keeping at least 8
+    // stages) so that the CTAs fill whole waves of the resident ones (A^T W two
+    // per SM, A H^T one): the fewest splits within 2% of the best wave
+    // efficiency. A H^T splits alike with and without the fused objective, so
+    // that its products are the same in both. (Unsplit, 24000 x 16000, k = 50
+    // ran 188 CTAs in two waves, 1.95 ms; 2000 x 1000, k = 10 ran 16 CTAs, 59
+    // us, and 101 us with the objective.)
     const int64_t tiles = cdiv(w.P > 0 ? w.P : 1, w.bp) * w.nch;
     const int64_t bq = trans ? F32_BQ1 : 4 * w.ncg;
     w.splits = 1;
-    if (trans) {
-        const int64_t slots = 2 * (int64_t)sm_count();
+    {
+        const int64_t slots = (trans ? 2 : 1) * (int64_t)sm_count();
         auto eff = [&](int64_t sp) {
             const int64_t ctas = tiles * sp;
             return (double)ctas / (double)(cdiv(ctas, slots) * slots);
@@ -511,14 +513,14 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool obj)
                 break;
             }
     }
-    (void)obj;
     w.q_per_split = cdiv(cdiv(w.Q > 0 ? w.Q : 1, w.splits), bq) * bq;
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     w.f_off = 0;
     const size_t fbytes = trans ? sizeof(float) * (size_t)(w.Q > 0 ? w.Q : 1) * w.kpt
                                 : sizeof(float) * (size_t)w.kpt * w.ldf;
     w.part_off = al(fbytes);
-    w.split_off = w.part_off + al(sizeof(double) * (size_t)cdiv(w.P > 0 ? w.P : 1, w.bp));
+    w.split_off = w.part_off +
+                  al(sizeof(double) * (size_t)(cdiv(w.P > 0 ? w.P : 1, w.bp) * w.splits));
     w.total = w.split_off +
               (w.splits > 1 ? al(sizeof(float) * 2 * (size_t)w.splits * (size_t)w.P * k) : 0);
     return w;
@@ -577,7 +579,7 @@ bool mm_f32_supported(const float *A, int64_t lda)
 
 size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans)
 {
-    return std::max(f32_plan(m, n, k, trans, false).total, f32_plan(m, n, k, trans, true).total);
+    return f32_plan(m, n, k, trans).total;
 }
 
 nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, const float *F, int k,
@@ -585,7 +587,7 @@ nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, cons
                          size_t work_bytes, cudaStream_t s)
 {
     const bool obj = W != nullptr;
-    const F32Plan w = f32_plan(m, n, k, trans, obj);
+    const F32Plan w = f32_plan(m, n, k, trans);
     if (w.P == 0)
         return NMF_OK;
     if (!mm_f32_supported(A, lda) || work_bytes < w.total || (obj && (trans || k > 64 || !f_dev)))
@@ -619,7 +621,7 @@ nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, cons
         NMF_LAUNCHED("f32_reduce_kernel");
     }
     if (obj)
-        return launch_sum_partials(part, (int)cdiv(w.P, w.bp), f_dev, s);
+        return launch_sum_partials(part, (int)(cdiv(w.P, w.bp) * w.splits), f_dev, s);
     return NMF_OK;
 }
 
