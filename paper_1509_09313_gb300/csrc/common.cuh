@@ -78,6 +78,31 @@ inline nmf_status ensure_smem(Kernel kernel, SmemOptIn &cache, size_t bytes)
     return NMF_OK;
 }
 
+// Sum of `n` floats `stride` apart, correct to about 2^-46 of their absolute
+// sum and rounded once: a pair of floats (Knuth's two-sum), since the FP64 pipe
+// does two additions per clock per SM (the sum of four 24000 x 50 partials
+// took 23 us in FP64, most of it additions and conversions). Where the FP32
+// sum is not finite (an infinity or NaN among the terms, or an overflow on the
+// way), the terms are added in FP64.
+__device__ __forceinline__ float sum_strided(const float *__restrict__ v, int n, int64_t stride)
+{
+    float s = 0.0f, c = 0.0f;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+        const float x = v[i * stride];
+        const float t = s + x;
+        const float b = t - s;
+        c += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    if (isfinite(s))
+        return s + c;
+    double d = 0.0;
+    for (int i = 0; i < n; ++i)
+        d += (double)v[i * stride];
+    return (float)d;
+}
+
 // True when [a, a + bytes) and [b, b + bytes) share a byte.
 inline bool ranges_overlap(const void *a, const void *b, size_t bytes)
 {

@@ -27,8 +27,8 @@
 // The partial sums of each stage (A H^T: two chains of 2 NCG steps; A^T W:
 // 32 steps) are added into the running totals with Kahan compensation, and
 // the output is the compensated total rounded once (with contraction splits:
-// each split's total and compensation, added over the splits in FP64 and
-// rounded once). So the products stay within about one FP32 rounding however
+// each split's total and compensation, added over the splits and rounded
+// once). So the products stay within about one FP32 rounding however
 // long the contraction: plain sequential FP32 accumulation over n = 64000
 // terms drifts by ~1e-6, and even product noise of a few 1e-8 moves the
 // objective of a short run by ~1e-6 through the NLS solves.
@@ -350,7 +350,7 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
     }
 
     // Output: the compensated total rounded once, or (contraction split)
-    // this split's total and compensation, for the FP64 sum over splits.
+    // this split's total and compensation, for the sum over splits.
     const bool split = gridDim.z > 1;
     float *dst = out + (int64_t)blockIdx.z * 2 * P * k;
 #pragma unroll
@@ -414,18 +414,13 @@ __global__ void __maxnreg__(128)
 }
 
 // out[p][c] = the sum over splits s of total[s][p][c] + compensation[s][p][c]
-// (part holds each split's two arrays in turn), in FP64 in split order,
-// rounded once.
+// (part holds each split's two arrays in turn), rounded once.
 __global__ void f32_reduce_kernel(const float *__restrict__ part, int splits, int64_t len,
                                   float *__restrict__ out)
 {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int sp = 0; sp < splits; ++sp)
-            s += (double)part[2 * sp * len + e] + (double)part[(2 * sp + 1) * len + e];
-        out[e] = (float)s;
-    }
+         e += (int64_t)gridDim.x * blockDim.x)
+        out[e] = sum_strided(part + e, 2 * splits, len);
 }
 
 // F^T (trans = 0): Ft[c][q] = F[q][c] for c < k, 0 for k <= c < kpt, rows of
