@@ -9,24 +9,37 @@
 //         with the newest values of the other entries; a column with
 //         G_ii <= 0 is set to 0.
 //
-// Rows are independent: one warp per row, lane l holding entries l, l + 32,
-// ... (KW slots), G in FP32 in shared memory lane-interleaved (entry (r, c) at
-// r * 32 KW + (c % 32) * KW + c / 32) so that a lane reads its KW entries of a
-// row as one vector. MU forms X G with one product. HALS forms each
-// coordinate's off-diagonal sum sum_{l != i} G_li x_l afresh, a warp dot
-// product with G staged with a zero diagonal. Keeping x G and adding d times
-// row i of G after each change would save the dot products but loses digits:
-// HALS often drives whole columns to zero, and the large steps d = -x_i leave
-// the updated sums as the rounding residue of a cancellation (measured on the
-// sparse 20000 x 10000 test: 1e-3 relative factor error after five iterations,
-// against 1e-7 for the direct form).
+// Rows are independent. row_update_kernel gives a warp a tile of 64 rows, held
+// transposed in shared memory (entry l of every row side by side), lane l
+// owning rows 2 l and 2 l + 1; the coordinates are taken in blocks of 8. For
+// a block, the sums over the entries outside it, sum_l G_li x_l, are a small
+// matrix product (the lane's two rows are the halves of packed FP32x2 FMAs, G
+// is staged with every value twice as their other operand); HALS then takes the block's coordinates in
+// turn, adding each new value to the sums still open. Every sum consists of
+// the terms of its own definition: keeping x G and adding d times row i of G
+// after each change would save the products but loses digits. HALS often
+// drives whole columns to zero, and the large steps d = -x_i leave the updated
+// sums as the rounding residue of a cancellation (measured on the sparse 20000
+// x 10000 test: 1e-3 relative factor error after five iterations, against 1e-7
+// for the direct form). Eight terms at a time are summed apart and then added
+// to the total.
 //
-// The same row kernel also forms the projected-gradient norm of the
-// stopping rule (Lin 2007): grad = X G - R, an entry counting where x_ij > 0
-// and, where x_ij = 0, only if negative; squares summed in FP32 per row, FP64
-// across rows, per-CTA partials added in a fixed order.
+// local_update_kernel (one warp per row) serves batches too small for tiles:
+// lane l holds entries l, l + 32, ... (KW slots), G in FP32 in shared memory
+// lane-interleaved (entry (r, c) at r * 32 KW + (c % 32) * KW + c / 32) so
+// that a lane reads its KW entries of a row as one vector; MU forms X G with
+// one product, HALS each coordinate's sum with a butterfly. It also forms the
+// projected-gradient norm of the stopping rule (Lin 2007): grad = X G - R, an
+// entry counting where x_ij > 0 and, where x_ij = 0, only if negative; squares
+// summed in FP32 per row, FP64 across rows, per-CTA partials added in a fixed
+// order.
 //
 // Roofline: HBM (12 k bytes per row: R and X in, X out); 2 k^2 FLOPs per row.
+// The tile kernel is bound by the latency of its instruction stream (some ten
+// warps per SM, one instruction in four cycles each). Measured, 96000 x 50:
+// HALS 45 us, MU 37 us (one warp per row: 272 and 51 us; HBM alone 8.5 us);
+// 1000000 x 50: HALS 411 us (2785), MU 356 us (478). 128-row tiles, four rows
+// per lane, were slower at 96000 rows (50 and 46 us) and 1000000 (457, 421).
 #include "common.cuh"
 
 namespace nmf {
@@ -34,6 +47,224 @@ namespace {
 
 constexpr int LU_WARPS = 8;
 enum LuOp { LU_MU = 0, LU_HALS = 1, LU_PGRAD = 2 };
+constexpr int RU_WARPS = 12;     // warps per CTA of row_update_kernel
+constexpr int RU_ROWS = 64;      // rows per warp tile, two per lane
+constexpr int RU_BLOCK = 8;      // coordinates per block, terms per partial sum
+constexpr int RU_DUP_K = 64;     // G staged with every value twice up to this k
+constexpr size_t LU_SMEM = 227 * 1024;
+
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool live)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(live ? 4 : 0)
+                 : "memory");
+}
+
+// a / g rounded to nearest for finite a >= 0, g > 0 and rg = 1 / g rounded: the
+// quotient corrected by its exact remainder (Markstein 1990), with the plain
+// division where the quotient is so large or small that a step of it could
+// overflow or lose bits.
+__device__ __forceinline__ float quotient(float a, float g, float rg)
+{
+    const float q = a * rg;
+    if (a > 0.0f && !(q > 1e-30f && q < 1e30f && g > 1e-30f && g < 1e30f))
+        return a / g;
+    return fmaf(fmaf(-q, g, a), rg, q);
+}
+
+// Shared memory: G (k rows of k rounded up to 8; every value twice when DUP, as
+// the operand pair of a packed FMA), then per warp the tile of X (k x RS) and
+// the block's panel of R, later of its new values (8 x RS); RS = 66.
+__host__ __device__ inline size_t ru_g_floats(int k, bool dup)
+{
+    return (size_t)k * ((k + 7) & ~7) * (dup ? 2 : 1);
+}
+__host__ __device__ inline size_t ru_warp_floats(int k)
+{
+    return (size_t)(k + RU_BLOCK) * (RU_ROWS + 2);
+}
+
+template <bool HALS, bool DUP>
+__global__ void __launch_bounds__(RU_WARPS * 32, 1)
+    row_update_kernel(const double *__restrict__ G, int k, const float *__restrict__ R,
+                      float *__restrict__ X, int64_t rows, int nw)
+{
+    constexpr int TR = RU_ROWS, RS = RU_ROWS + 2, D = DUP ? 2 : 1;
+    extern __shared__ __align__(16) float lu_smem[];
+    const int KP = (k + 7) & ~7;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *Gs = lu_smem;
+    float *Xs = Gs + ru_g_floats(k, DUP) + warp * ru_warp_floats(k);
+    float *Ps = Xs + k * RS;
+    const uint32_t magic = 0xffffffffu / (uint32_t)k + 1u;   // e / k for e < 2^16
+    const int64_t ntiles = cdiv(rows, TR);
+    int64_t tile = warp < nw ? (int64_t)blockIdx.x * nw + warp : ntiles;
+    // A tile of X (its rows are one stretch), transposed on the way; all of it
+    // in flight at once.
+    auto load_tile = [&]() {
+        const float *src = X + tile * TR * k;
+        const int ne = (int)min((int64_t)TR, rows - tile * TR) * k;
+#pragma unroll 4
+        for (int e = lane; e < ne; e += 32) {
+            const int r = k == 1 ? e : (int)__umulhi((uint32_t)e, magic);
+            cp_async4(Xs + (e - r * k) * RS + r, src + e, true);
+        }
+    };
+    if (tile < ntiles)
+        load_tile();
+    // All the CTA's warps stage G; those without a tile of their own then leave.
+#pragma unroll 4
+    for (int e = threadIdx.x; e < k * KP; e += RU_WARPS * 32) {
+        const int r = e / KP, c = e - r * KP;
+        const float g = c < k ? (float)G[r * k + c] : 0.0f;
+        if (DUP)
+            reinterpret_cast<float2 *>(Gs)[e] = make_float2(g, g);
+        else
+            Gs[e] = g;
+    }
+    __syncthreads();
+    const float2 zero2 = make_float2(0.0f, 0.0f), neg1 = make_float2(-1.0f, -1.0f);
+    const int pr = lane >> 3, pc = lane & 7;   // panel copies: row pr + 4 t, column pc
+    while (tile < ntiles) {
+        const int64_t row0 = tile * TR;
+        const int nr = (int)min((int64_t)TR, rows - row0);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        for (int i0 = 0; i0 < k; i0 += RU_BLOCK) {
+            const int nb = min(RU_BLOCK, k - i0);
+            __syncwarp();   // X staged; the last panel is read
+            // The block's panel of R, in flight while the sums are formed.
+            {
+                const float *src = R + (row0 + pr) * k + i0 + pc;
+                float *dst = Ps + pc * RS + pr;
+#pragma unroll 4
+                for (int t = 0; t < TR / 4; ++t) {
+                    const bool live = pr + 4 * t < nr && pc < nb;
+                    cp_async4(dst + 4 * t, live ? src : R, live);
+                    src += 4 * k;
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            // Lane l: rows 2 l and 2 l + 1, as the pairs of packed FMAs.
+            // HALS keeps the total's rounding errors beside it (Dekker's
+            // two-sum: exact while the total is the larger), since the
+            // coordinate is a small difference of two large sums: plain adds
+            // lost 1.3 times what the warp's butterfly sum loses, this loses
+            // half as much (2 us of 43).
+            float2 tot[RU_BLOCK], err[RU_BLOCK], part[RU_BLOCK];
+#pragma unroll
+            for (int b = 0; b < RU_BLOCK; ++b)
+                tot[b] = err[b] = zero2;
+            auto add = [&](int b) {   // tot + err += part
+                const float2 s = __fadd2_rn(tot[b], part[b]);
+                if (HALS) {
+                    const float2 d = __ffma2_rn(tot[b], neg1, s);
+                    err[b] = __fadd2_rn(err[b], __ffma2_rn(d, neg1, part[b]));
+                }
+                tot[b] = s;
+            };
+            auto pair_of_x = [&](int l) {
+                return *reinterpret_cast<const float2 *>(Xs + l * RS + 2 * lane);
+            };
+            // v += G[l][i0 + lo .. hi) x_l.
+            auto term = [&](int l, float2 (&v)[RU_BLOCK], int lo, int hi) {
+                const float4 *gr = reinterpret_cast<const float4 *>(Gs + (l * KP + i0) * D);
+                const float2 x = pair_of_x(l);
+#pragma unroll
+                for (int h = 0; h < 2 * D; ++h) {
+                    const float4 g = gr[h];
+                    constexpr int W = 4 / D;   // coordinates per 16 bytes
+#pragma unroll
+                    for (int b = 0; b < W; ++b) {
+                        const int i = W * h + b;
+                        const float2 gg = DUP ? (b ? make_float2(g.z, g.w) : make_float2(g.x, g.y))
+                                          : b == 0 ? make_float2(g.x, g.x)
+                                          : b == 1 ? make_float2(g.y, g.y)
+                                          : b == 2 ? make_float2(g.z, g.z)
+                                                   : make_float2(g.w, g.w);
+                        if (i >= lo && i < hi)
+                            v[i] = __ffma2_rn(gg, x, v[i]);
+                    }
+                }
+            };
+            for (int l0 = 0; l0 < k; l0 += RU_BLOCK) {
+                if (HALS && l0 == i0)
+                    continue;
+#pragma unroll
+                for (int b = 0; b < RU_BLOCK; ++b)
+                    part[b] = zero2;
+                if (l0 + RU_BLOCK <= k) {
+#pragma unroll
+                    for (int j = 0; j < RU_BLOCK; ++j)
+                        term(l0 + j, part, 0, RU_BLOCK);
+                } else {
+                    for (int l = l0; l < k; ++l)
+                        term(l, part, 0, RU_BLOCK);
+                }
+#pragma unroll
+                for (int b = 0; b < RU_BLOCK; ++b)
+                    add(b);
+            }
+            // HALS: the terms of the block's own entries, summed apart: first
+            // those still to come (coordinates below j), before they change.
+#pragma unroll
+            for (int b = 0; b < RU_BLOCK; ++b)
+                part[b] = zero2;
+            if (HALS) {
+#pragma unroll
+                for (int j = 1; j < RU_BLOCK; ++j)
+                    if (j < nb)
+                        term(i0 + j, part, 0, j);
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < RU_BLOCK; ++i) {
+                if (i >= nb)
+                    break;
+                const float gii = Gs[((i0 + i) * KP + i0 + i) * D];
+                const float rg = 1.0f / gii;
+                float *pp = Ps + i * RS + 2 * lane;
+                const float2 r = *reinterpret_cast<const float2 *>(pp);
+                float2 x;
+                if (HALS) {
+                    add(i);
+                    const float n0 = (r.x - tot[i].x) - err[i].x;
+                    const float n1 = (r.y - tot[i].y) - err[i].y;
+                    x.x = gii > 0.0f ? quotient(n0 > 0.0f ? n0 : 0.0f, gii, rg) : 0.0f;
+                    x.y = gii > 0.0f ? quotient(n1 > 0.0f ? n1 : 0.0f, gii, rg) : 0.0f;
+                    *reinterpret_cast<float2 *>(Xs + (i0 + i) * RS + 2 * lane) = x;
+                } else {
+                    const float2 t = tot[i];
+                    x = pair_of_x(i0 + i);   // (stays for the blocks to come)
+                    if (t.x > 0.0f)
+                        x.x = x.x * r.x / t.x;
+                    if (t.y > 0.0f)
+                        x.y = x.y * r.y / t.y;
+                }
+                *reinterpret_cast<float2 *>(pp) = x;
+                // ... then the new values, as they come.
+                if (HALS)
+                    term(i0 + i, part, i + 1, RU_BLOCK);
+            }
+            __syncwarp();
+            {
+                float *dst = X + (row0 + pr) * k + i0 + pc;
+                const float *src = Ps + pc * RS + pr;
+#pragma unroll 4
+                for (int t = 0; t < TR / 4; ++t) {
+                    if (pr + 4 * t < nr && pc < nb)
+                        *dst = src[4 * t];
+                    dst += 4 * k;
+                }
+            }
+        }
+        __syncwarp();   // the next tile overwrites Xs
+        tile += (int64_t)gridDim.x * nw;
+        if (tile < ntiles)
+            load_tile();
+    }
+}
 
 template <int KW>
 __device__ __forceinline__ void lu_row_fma(const float *__restrict__ p, float a, float (&acc)[KW])
@@ -179,6 +410,31 @@ __global__ void lu_sum_kernel(const double *__restrict__ partials, int n, double
     }
 }
 
+template <bool HALS, bool DUP>
+nmf_status launch_rows(const double *G, int k, const float *R, float *X, int64_t rows,
+                       cudaStream_t s)
+{
+    const int64_t tiles = cdiv(rows, RU_ROWS);
+    // One CTA per SM, with the warps that share the tiles out evenly (as many
+    // as the shared memory holds), so that G is staged once per SM.
+    const size_t g = sizeof(float) * ru_g_floats(k, DUP), w = sizeof(float) * ru_warp_floats(k);
+    int64_t nw = cdiv(tiles, sm_count());
+    if (nw > RU_WARPS)
+        nw = RU_WARPS;
+    while (nw > 1 && g + nw * w > LU_SMEM)
+        --nw;
+    const size_t smem = g + nw * w;
+    static SmemOptIn opt_in;
+    NMF_TRY(ensure_smem(row_update_kernel<HALS, DUP>, opt_in, smem));
+    int64_t blocks = cdiv(tiles, nw);
+    if (blocks > sm_count())
+        blocks = sm_count();
+    row_update_kernel<HALS, DUP><<<(unsigned)blocks, 32 * RU_WARPS, smem, s>>>(G, k, R, X, rows,
+                                                                                  (int)nw);
+    NMF_LAUNCHED(HALS ? "row_update_kernel<hals>" : "row_update_kernel<mu>");
+    return NMF_OK;
+}
+
 // LU_PGRAD writes one partial per CTA (at most max_parts); *nparts gets the
 // count.
 template <int KW, int OP>
@@ -221,17 +477,30 @@ nmf_status launch_lu_k(const double *G, int k, const float *R, float *X, int64_t
 
 }  // namespace
 
+// The tile kernel from the row count where its tiles keep the GPU busy: a tile
+// of 64 rows takes 20-25 us whatever the batch, a wave of single rows 10 (MU)
+// or 17 (HALS) us. Measured, k = 50, tiles against single rows: HALS 5000 rows
+// 29 / 25 us, 20000 29 / 70, 96000 45 / 278; MU 20000 rows 33 / 19, 50000
+// 33 / 31, 77824 33 / 44.
 nmf_status launch_local_update(int solver, const double *G, int k, const float *R, float *X,
                                int64_t rows, cudaStream_t s)
 {
     if (rows == 0)
         return NMF_OK;
-    int np = 0;
-    if (solver == NMF_SOLVER_MU)
+    if (solver != NMF_SOLVER_MU && solver != NMF_SOLVER_HALS)
+        return NMF_ERR_INVALID_ARG;
+    const bool hals = solver == NMF_SOLVER_HALS;
+    if (rows < (hals ? 48 : 384) * (int64_t)sm_count()) {
+        int np = 0;
+        if (hals)
+            return launch_lu_k<LU_HALS>(G, k, R, X, rows, nullptr, 0, &np, s);
         return launch_lu_k<LU_MU>(G, k, R, X, rows, nullptr, 0, &np, s);
-    if (solver == NMF_SOLVER_HALS)
-        return launch_lu_k<LU_HALS>(G, k, R, X, rows, nullptr, 0, &np, s);
-    return NMF_ERR_INVALID_ARG;
+    }
+    if (hals)
+        return k <= RU_DUP_K ? launch_rows<true, true>(G, k, R, X, rows, s)
+                             : launch_rows<true, false>(G, k, R, X, rows, s);
+    return k <= RU_DUP_K ? launch_rows<false, true>(G, k, R, X, rows, s)
+                         : launch_rows<false, false>(G, k, R, X, rows, s);
 }
 
 int pgrad_partials_len() { return 2 * sm_count(); }

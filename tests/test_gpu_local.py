@@ -142,3 +142,17 @@ def test_proposal_rejected_for_mu(nmf):
     with pytest.raises(nmf.NMFError):
         h.nmf_set_proposal(net, "train")
     h.nmf_destroy()
+
+
+# Row counts at the edges of the kernels (one warp per row, 64-row tiles from 48 or
+# 384 rows per SM on, their last one ragged), block edges of k. Same bound as above.
+@pytest.mark.parametrize("rows", [1, 31, 33, 7295, 7297, 38913, 58367, 58369])
+@pytest.mark.parametrize("k", [1, 8, 9, 50, 64, 65, 128])
+@pytest.mark.parametrize("solver", ["mu", "hals"])
+def test_step_at_tile_edges(nmf, solver, k, rows):
+    G, R, X = problem(rows, k, seed=rows + k)
+    Xd = dev(X)
+    fn = nmf.nmf_update_mu if solver == "mu" else nmf.nmf_update_hals
+    fn(dev(G, torch.float64), dev(R), Xd)
+    ref = (oracle.mu if solver == "mu" else oracle.hals)(G, R, X)
+    assert row_rel_err(Xd.double().cpu().numpy(), ref) <= 2e-5
