@@ -161,7 +161,8 @@ nmf_status nmf_nls_bpp_tune(const nmf_nls_desc *d, void *stream, int32_t *warps,
 
 /* Sets the launch shape of every later solve of this k in the process, as the
  * tuner would (an interface of this library): warps per CTA 1..16 (the FP64
- * solves use at most 8), right-hand sides per grab of the work counter
+ * solves use at most 8; the FP32 ones of k > 64, which leave one CTA per SM,
+ * take twice as many, at most 16), right-hand sides per grab of the work counter
  * 1..1024 (fewer where the batch is too small to give every warp several
  * grabs), and the group-tile pass of FP32 half-steps (right-hand sides whose
  * first candidate partition is all usable indices are solved together by

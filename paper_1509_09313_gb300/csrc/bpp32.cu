@@ -2,15 +2,14 @@
 // diagonally scaled cond_1 the preparation found at most 1e4 (mode 0).
 //
 // Same method as the FP64 kernel in bpp.cu: one warp per right-hand side,
-// lane l holding indices l, l + 32, ... (KW slots); each exchange round solves
+// its indices over the lanes (KW slots each); each exchange round solves
 // the smaller of the direct system G_FF x_F = g_F and the complement system
 // M_AA y_A = -u_A (u = M g, x_F = u_F + M_FA y_A), refines once through the
 // same factor, recomputes y = G x - g, and tests the signs with the FP32
 // tolerances in the diagonally scaled variables. Organised for fewer
 // instructions per solve:
-//  * G and M sit in shared memory lane-interleaved: entry (r, c) at
-//    r * 32 KW + (c % 32) * KW + c / 32, so a lane reads its KW entries of a
-//    row with one vector load and updates them with packed FP32x2 FMAs;
+//  * G and M sit in shared memory so that a lane reads its KW entries of a row
+//    with one vector load and updates them with packed FP32x2 FMAs;
 //  * a product with a vector supported on a short index list (F in the direct
 //    form, the active set in the complement form) loops over that list only:
 //    y = G_{:,F} x_F costs |F| row reads, not k;
@@ -19,8 +18,10 @@
 //    trailing rows stay in registers, one row per lane, shifted one column per
 //    step so that a rolled loop keeps constant register indices; the
 //    multipliers go to shared memory for the two substitutions;
-//  * k > 64: a left-looking Cholesky that keeps each row's reciprocal pivot in
-//    its lane: with q = rsqrt(d), L_jj = d q and L_ij = s_i q;
+//  * k > 64: the same LDL^T for systems of at most 32 rows with the pivot rows
+//    read from shared memory; above, a left-looking Cholesky that keeps each
+//    row's reciprocal pivot in its lane: with q = rsqrt(d), L_jj = d q and
+//    L_ij = s_i q;
 //  * no FP64 arithmetic: a system that meets the pivot floor defers its
 //    right-hand side to the FP64 kernel's second pass, which re-solves it from
 //    its starting partition.
@@ -34,7 +35,56 @@ namespace {
 
 constexpr int S32_MAX_WARPS = 16;
 constexpr int DEFERRED = -1;   // internal status: re-solve this right-hand side in FP64
-constexpr size_t SMEM_LIMIT32 = 227 * 1024;
+constexpr size_t SMEM_LIMIT32 = 226 * 1024;   // leaves room for the static arrays
+
+// Layout of G and M in shared memory and of the indices over the lanes. KW <= 2:
+// lane l holds indices l, l + 32, ...; entry (r, c) at r 32 KW + (c mod 32) KW +
+// c / 32. KW = 4 (k > 64): lane l holds indices 4 l .. 4 l + 3 and the rows are
+// stored as they are, k4 (k rounded up to 4) floats each (at k = 100 this
+// leaves room for twice the warps that padded rows of 128 do). Either way a
+// lane's KW entries of a row are one vector at lane KW.
+template <int KW>
+__device__ __forceinline__ int slot_index(int lane, int s)
+{
+    return KW == 4 ? 4 * lane + s : lane + 32 * s;
+}
+template <int KW>
+__host__ __device__ __forceinline__ constexpr int row_stride(int k4)
+{
+    return KW == 4 ? k4 : 32 * KW;
+}
+template <int KW>
+__device__ __forceinline__ int col_offset(int c)
+{
+    return KW == 4 ? c : (c & 31) * KW + (c >> 5);
+}
+
+// The 64-bit words of a set of indices (f[s]: index slot_index(lane, s) is in).
+template <int KW>
+__device__ __forceinline__ void write_words(const bool (&f)[KW], uint64_t *__restrict__ dst,
+                                            int lane)
+{
+    if constexpr (KW == 4) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            v |= (uint32_t)f[s] << s;
+        v <<= 4 * (lane & 7);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1)
+            v |= __shfl_xor_sync(FULL, v, o);
+        const uint32_t hi = __shfl_down_sync(FULL, v, 8);
+        if (lane == 0 || lane == 16)
+            dst[lane >> 4] = v | ((uint64_t)hi << 32);
+    } else {
+        unsigned bm[KW];
+#pragma unroll
+        for (int s = 0; s < KW; ++s)
+            bm[s] = __ballot_sync(FULL, f[s]);
+        if (lane == 0)
+            dst[0] = bm[0] | (KW == 2 ? (uint64_t)bm[KW - 1] << 32 : 0ull);
+    }
+}
 
 // acc[s] += p[s] * a for the KW entries of one row that a lane owns.
 template <int KW>
@@ -66,7 +116,7 @@ template <int KW>
 __device__ __forceinline__ void mv_full(const float *__restrict__ Mat, int k4,
                                         const float *__restrict__ vec, float (&out)[KW], int lane)
 {
-    constexpr int RS = 32 * KW;
+    const int RS = row_stride<KW>(k4);
     float a1[KW];
 #pragma unroll
     for (int s = 0; s < KW; ++s)
@@ -89,9 +139,9 @@ __device__ __forceinline__ void mv_full(const float *__restrict__ Mat, int k4,
 template <int KW>
 __device__ __forceinline__ void mv_list(const float *__restrict__ Mat, const int *__restrict__ idx,
                                         const float *__restrict__ val, int n4, float (&out)[KW],
-                                        int lane)
+                                        int k4, int lane)
 {
-    constexpr int RS = 32 * KW;
+    const int RS = row_stride<KW>(k4);
     float a1[KW];
 #pragma unroll
     for (int s = 0; s < KW; ++s)
@@ -114,22 +164,32 @@ template <int KW>
 __device__ __forceinline__ void stage_vec(float *__restrict__ stage, const float (&v)[KW], int lane)
 {
     __syncwarp();
+    if constexpr (KW == 4) {
+        *reinterpret_cast<float4 *>(stage + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
 #pragma unroll
-    for (int s = 0; s < KW; ++s)
-        stage[32 * s + lane] = v[s];
+        for (int s = 0; s < KW; ++s)
+            stage[32 * s + lane] = v[s];
+    }
     __syncwarp();
 }
 
-// Cholesky of the p x p system S_ab = Src(idx[a], idx[b]) (lane-per-row,
-// left-looking, rows a = lane + 32 t). L goes to Lw (row stride LS, even, so
-// that rows are read as float2); inv[t] receives 1 / L_aa for the lane's rows.
-// Returns false (uniformly) when a pivot is at most PIVOT_TOL of its diagonal.
-template <int KW, int PT>
+// Start of row a of a lower triangle stored row by row, every row padded to an
+// even length (rows are read as float2).
+__host__ __device__ __forceinline__ constexpr int tri_off(int a)
+{
+    return (a + 1) * (a + 1) / 4 * 2;
+}
+
+// k > 64, systems of more than 32 rows: Cholesky of S_ab = Src(idx[a], idx[b])
+// (lane-per-row, left-looking, rows a = lane + 32 t). L goes to Lw (rows at
+// tri_off); inv[t] receives 1 / L_aa for the lane's rows. Returns false
+// (uniformly) when a pivot is at most PIVOT_TOL of its diagonal.
+template <int PT>
 __device__ __forceinline__ bool chol32(const float *__restrict__ Src, const int *__restrict__ idx,
-                                       int p, float *__restrict__ Lw, int LS, float (&inv)[PT],
+                                       int p, float *__restrict__ Lw, float (&inv)[PT], int RS,
                                        int lane)
 {
-    constexpr int RS = 32 * KW;
     int roff[PT], coff[PT];
     float dg[PT];
 #pragma unroll
@@ -142,7 +202,7 @@ __device__ __forceinline__ bool chol32(const float *__restrict__ Src, const int 
         if (a < p) {
             const int c = idx[a];
             roff[t] = c * RS;
-            coff[t] = (c & 31) * KW + (c >> 5);
+            coff[t] = c;
             dg[t] = Src[roff[t] + coff[t]];
         }
     }
@@ -154,14 +214,14 @@ __device__ __forceinline__ bool chol32(const float *__restrict__ Src, const int 
             if (tj == t)
                 cj = coff[t];
         cj = __shfl_sync(FULL, cj, owner);
-        const float *lj = Lw + j * LS;
+        const float *lj = Lw + tri_off(j);
         float sv[PT];
 #pragma unroll
         for (int t = 0; t < PT; ++t) {
             const int a = lane + 32 * t;
             sv[t] = 0.0f;
             if (a >= j && a < p) {
-                const float *la = Lw + a * LS;
+                const float *la = Lw + tri_off(a);
                 float2 acc = make_float2(0.0f, 0.0f);
                 int c = 0;
                 for (; c + 2 <= j; c += 2)
@@ -185,7 +245,7 @@ __device__ __forceinline__ bool chol32(const float *__restrict__ Src, const int 
         for (int t = 0; t < PT; ++t) {
             const int a = lane + 32 * t;
             if (a >= j && a < p)
-                Lw[a * LS + j] = sv[t] * q;
+                Lw[tri_off(a) + j] = sv[t] * q;
             if (t == tj && lane == owner)
                 inv[t] = q;
         }
@@ -196,7 +256,7 @@ __device__ __forceinline__ bool chol32(const float *__restrict__ Src, const int 
 
 // Solve L L^T z = r in place (row a of r in lane a % 32, slot a / 32).
 template <int PT>
-__device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw, int LS,
+__device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw,
                                         const float (&inv)[PT], float (&r)[PT], int lane)
 {
     for (int j = 0; j < p; ++j) {
@@ -211,7 +271,7 @@ __device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw, int
         for (int t = 0; t < PT; ++t) {
             const int a = lane + 32 * t;
             if (a > j && a < p)
-                r[t] = fmaf(-Lw[a * LS + j], z, r[t]);
+                r[t] = fmaf(-Lw[tri_off(a) + j], z, r[t]);
             if (t == tj && lane == owner)
                 r[t] = z;
         }
@@ -224,7 +284,7 @@ __device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw, int
             if (tj == t)
                 v = r[t] * inv[t];
         const float xj = __shfl_sync(FULL, v, owner);
-        const float *lj = Lw + j * LS;
+        const float *lj = Lw + tri_off(j);
 #pragma unroll
         for (int t = 0; t < PT; ++t) {
             const int a = lane + 32 * t;
@@ -234,6 +294,119 @@ __device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw, int
                 r[t] = xj;
         }
     }
+}
+
+// k > 64, systems of at most 32 rows: LDL^T of S_ab = Src(idx[a], idx[b]), lane
+// a keeping the live part of row a of the trailing matrix in registers,
+// shifted one column per step like ldl_regs. Step j's row reaches the lanes
+// through shared memory: by symmetry it is the column the lanes hold in s[0],
+// so each lane stores one value and all read the row four entries at a time
+// (a shuffle per entry took a third of the factorisation's instructions).
+// The stored columns, unscaled (S_aj, lane a at Lc[j LDL_LS + a - j]), are also
+// the factor: L_aj = S_aj / D_j, the divisors 1 / D_a staying in rp of lane a.
+// Src is read by columns (idx[a]) of the rows idx[b], whose banks differ more
+// than those of the rows. The registers (128 per thread at 16 warps per SM)
+// allow this here; at k <= 64, with 64, it spilled.
+constexpr int LDL_LS = 36;   // a multiple of 4; LDL_LS - 1 odd: conflict-free rows and columns
+__device__ __forceinline__ bool ldl_cols(const float *__restrict__ Src, const int *__restrict__ idx,
+                                         int p, float *__restrict__ Lc, float &rp, int RS, int lane)
+{
+    const int c = lane < p ? idx[lane] : 0;
+    const float dtol = PIVOT_TOL * Src[c * RS + c];
+    float s[32];
+#pragma unroll
+    for (int b0 = 0; b0 < 32; b0 += 4) {
+        if (b0 < p) {
+            const int4 o = *reinterpret_cast<const int4 *>(idx + b0);
+            s[b0] = Src[o.x * RS + c];
+            s[b0 + 1] = Src[o.y * RS + c];
+            s[b0 + 2] = Src[o.z * RS + c];
+            s[b0 + 3] = Src[o.w * RS + c];
+        } else {
+#pragma unroll
+            for (int b = b0; b < b0 + 4; ++b)
+                s[b] = 0.0f;
+        }
+    }
+    bool ok = true;
+    rp = 0.0f;
+    for (int j = 0; j < p; ++j) {
+        float *col = Lc + j * LDL_LS;
+        if (lane >= j && lane < p)
+            col[lane - j] = s[0];
+        __syncwarp();
+        const int w = p - j;   // live columns: s[0 .. w)
+        const float4 c0 = *reinterpret_cast<const float4 *>(col);
+        const float q = rsqrtf(c0.x);
+        const float r = q * q;
+        if (lane == j) {
+            ok = c0.x > dtol;
+            rp = r;
+        }
+        // (Entries of col past the live columns are not set: they only reach
+        // registers past the live ones.)
+        const float m = s[0] * r;
+        s[0] = fmaf(-m, c0.y, s[1]);
+        s[1] = fmaf(-m, c0.z, s[2]);
+        s[2] = fmaf(-m, c0.w, s[3]);
+#pragma unroll
+        for (int b0 = 4; b0 < 32; b0 += 4) {
+            if (b0 >= w)
+                break;
+            const float4 cv = *reinterpret_cast<const float4 *>(col + b0);
+            s[b0 - 1] = fmaf(-m, cv.x, s[b0]);
+            s[b0] = fmaf(-m, cv.y, s[b0 + 1]);
+            s[b0 + 1] = fmaf(-m, cv.z, s[b0 + 2]);
+            s[b0 + 2] = fmaf(-m, cv.w, s[b0 + 3]);
+        }
+    }
+    return __all_sync(FULL, ok);
+}
+
+// Solve S z = r with the factor of ldl_cols (row a of r and z in lane a):
+// forward v_a -= S_aj (v_j / D_j), backward v_a -= S_ja z_j with z_a = v_a / D_a.
+// Four steps at a time with their factors loaded first (every address is
+// within the factor; lanes outside a step discard theirs).
+__device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, float rp, int p,
+                                                float v, int lane)
+{
+    const float *fw = Lc + lane, *bw = Lc + lane * (LDL_LS - 1);
+    int j = 0;
+    for (; j + 4 < p; j += 4) {
+        const float l0 = fw[j * (LDL_LS - 1)], l1 = fw[(j + 1) * (LDL_LS - 1)];
+        const float l2 = fw[(j + 2) * (LDL_LS - 1)], l3 = fw[(j + 3) * (LDL_LS - 1)];
+        float t = __shfl_sync(FULL, v * rp, j);
+        if (lane > j) v = fmaf(-l0, t, v);
+        t = __shfl_sync(FULL, v * rp, j + 1);
+        if (lane > j + 1) v = fmaf(-l1, t, v);
+        t = __shfl_sync(FULL, v * rp, j + 2);
+        if (lane > j + 2) v = fmaf(-l2, t, v);
+        t = __shfl_sync(FULL, v * rp, j + 3);
+        if (lane > j + 3) v = fmaf(-l3, t, v);
+    }
+    for (; j + 1 < p; ++j) {
+        const float t = __shfl_sync(FULL, v * rp, j);
+        if (lane > j)
+            v = fmaf(-fw[j * (LDL_LS - 1)], t, v);
+    }
+    j = p - 1;
+    for (; j >= 4; j -= 4) {
+        const float l0 = bw[j], l1 = bw[j - 1], l2 = bw[j - 2], l3 = bw[j - 3];
+        float z = __shfl_sync(FULL, v * rp, j);
+        if (lane < j) v = fmaf(-l0, z, v);
+        z = __shfl_sync(FULL, v * rp, j - 1);
+        if (lane < j - 1) v = fmaf(-l1, z, v);
+        z = __shfl_sync(FULL, v * rp, j - 2);
+        if (lane < j - 2) v = fmaf(-l2, z, v);
+        z = __shfl_sync(FULL, v * rp, j - 3);
+        if (lane < j - 3) v = fmaf(-l3, z, v);
+    }
+    for (; j >= 1; --j) {
+        const float z = __shfl_sync(FULL, v * rp, j);
+        if (lane < j)
+            v = fmaf(-bw[j], z, v);
+    }
+    return v * rp;
 }
 
 // Systems of at most PM rows (k <= 64; PM >= k / 2 >= p): LDL^T of
@@ -355,20 +528,30 @@ __device__ __forceinline__ float ldl_solve(const float *__restrict__ Lw, int LS,
     return z;
 }
 
-// Shared memory: G and M (k rounded up to 4 rows of 32 KW floats each), then
-// per warp an index list, its values, a staging vector (32 KW each), the
-// list's column offsets (k <= 64) and the pmax x LS factor.
+// Shared memory: G and M (k rounded up to 4 rows of row_stride floats each),
+// then per warp an index list, its values, the list's column offsets (KW <= 2),
+// a staging vector and the factor (pmax x LS floats, KW <= 2; the larger of
+// ldl_cols's and the packed triangle of pmax rows, KW = 4).
 __host__ __device__ inline size_t mats_bytes32(int k, int KW)
 {
-    return 2 * sizeof(float) * (size_t)((k + 3) & ~3) * 32 * KW;
+    const size_t k4 = (size_t)((k + 3) & ~3);
+    return 2 * sizeof(float) * k4 * (KW == 4 ? k4 : 32 * KW);
+}
+// Entries of the index list, its values and column offsets (systems of at most
+// pmax rows, padded to a multiple of four).
+__host__ __device__ constexpr int list_len(int KW, int pmax)
+{
+    return KW == 4 ? (pmax + 7) & ~3 : 32 * KW;
 }
 __host__ __device__ inline size_t warp_bytes32(int KW, int pmax, int LS)
 {
-    // k <= 64: column offsets, and 32 floats of slack after the factor (read
-    // past its end by the unrolled substitutions).
-    const size_t cols = KW <= 2 ? sizeof(int) * 32 * KW + sizeof(float) * 32 : 0;
-    return (3 * sizeof(float) * 32 * KW + cols + sizeof(float) * (size_t)pmax * LS + 15) &
-           ~size_t(15);
+    if (KW == 4) {
+        const int fac = tri_off(pmax) > 32 * LDL_LS ? tri_off(pmax) : 32 * LDL_LS;
+        return (sizeof(float) * (size_t)(2 * list_len(4, pmax) + 128 + fac) + 15) & ~size_t(15);
+    }
+    // 32 floats of slack after the factor (read past its end by the unrolled
+    // substitutions).
+    return (sizeof(float) * (4 * 32 * (size_t)KW + 32 + (size_t)pmax * LS) + 15) & ~size_t(15);
 }
 
 // 64 registers for KW <= 2 (two 16-warp CTAs per SM); the KW = 4 form needs
@@ -377,7 +560,6 @@ template <int KW, int PM>
 __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     bpp_solve32_kernel(const SolveParams P, int pmax, int LS)
 {
-    constexpr int RS = 32 * KW;
     constexpr int PT = (KW + 1) / 2;
     const int mode = P.flags[0];
     const bool predict = mode == 1 && P.predict;
@@ -389,6 +571,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
         return;   // the group-tile pass solved them all
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = P.k, k4 = (k + 3) & ~3;
+    const int RS = row_stride<KW>(k4), LL = list_len(KW, pmax);
     const int max_rounds = predict ? PREDICT_ROUNDS : P.max_rounds;
     unsigned long long *counter = &P.counters[predict ? CNT_PREDICT : CNT_WORK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -396,17 +579,17 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     float *Ms = Gs + k4 * RS;
     for (int e = threadIdx.x; e < k4 * RS; e += blockDim.x) {
         const int r = e / RS, q = e - r * RS;
-        const int c = q / KW + 32 * (q % KW);
+        const int c = KW == 4 ? q : q / KW + 32 * (q % KW);
         const bool in = r < k && c < k;
         Gs[e] = in ? P.G32[r * k + c] : 0.0f;
         Ms[e] = in ? P.M32[r * k + c] : 0.0f;
     }
     unsigned char *wp = smem_raw + mats_bytes32(k, KW) + warp * warp_bytes32(KW, pmax, LS);
     int *widx = reinterpret_cast<int *>(wp);
-    float *zbuf = reinterpret_cast<float *>(widx + RS);
-    float *stage = zbuf + RS;
-    int *wcol = reinterpret_cast<int *>(stage + RS);   // KW <= 2: column offsets of the list
-    float *Lw = stage + RS + (KW <= 2 ? RS : 0);
+    float *zbuf = reinterpret_cast<float *>(widx + LL);
+    float *stage = zbuf + LL;
+    int *wcol = reinterpret_cast<int *>(stage + 32 * KW);   // KW <= 2: column offsets of the list
+    float *Lw = stage + 32 * KW + (KW <= 2 ? LL : 0);
     __syncthreads();
 
     bool usable[KW];
@@ -414,10 +597,9 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     int nU = 0;
 #pragma unroll
     for (int s = 0; s < KW; ++s) {
-        const uint32_t w = P.usable_words[s];
-        usable[s] = (w >> lane) & 1u;
-        nU += __popc(w);
-        const int i = lane + 32 * s;
+        const int i = slot_index<KW>(lane, s);
+        usable[s] = (P.usable_words[i >> 5] >> (i & 31)) & 1u;
+        nU += __popc(P.usable_words[s]);
         dsq[s] = usable[s] ? sqrtf(Gs[i * RS + lane * KW + s]) : 1.0f;
     }
 
@@ -472,7 +654,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             const float *frow = P.gat.F + cl * k;
 #pragma unroll
                             for (int s = 0; s < KW; ++s) {
-                                const int i = lane + 32 * s;
+                                const int i = slot_index<KW>(lane, s);
                                 fv[q][s] = i < k ? frow[i] : 0.0f;
                             }
                         }
@@ -480,7 +662,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         for (int q = 0; q < 4; ++q)
 #pragma unroll
                             for (int s = 0; s < KW; ++s)
-                                if (lane + 32 * s < k)
+                                if (slot_index<KW>(lane, s) < k)
                                     g[s] = fmaf(vl[q], fv[q][s], g[s]);
                     }
                     for (; l < cnt; ++l) {
@@ -489,7 +671,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         const float *frow = P.gat.F + cl * k;
 #pragma unroll
                         for (int s = 0; s < KW; ++s) {
-                            const int i = lane + 32 * s;
+                            const int i = slot_index<KW>(lane, s);
                             if (i < k)
                                 g[s] = fmaf(vl, frow[i], g[s]);
                         }
@@ -498,14 +680,14 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                 float *Bw = const_cast<float *>(P.B);   // the caller's right-hand-side buffer
 #pragma unroll
                 for (int s = 0; s < KW; ++s) {
-                    const int i = lane + 32 * s;
+                    const int i = slot_index<KW>(lane, s);
                     if (i < k)
                         Bw[j * k + i] = g[s];
                 }
             }
 #pragma unroll
             for (int s = 0; s < KW; ++s) {
-                const int i = lane + 32 * s;
+                const int i = slot_index<KW>(lane, s);
                 if (!fused)
                     g[s] = i < k ? P.B[j * k + i] : 0.0f;
                 bad |= !isfinite(g[s]);
@@ -530,7 +712,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                 if (P.pin) {
 #pragma unroll
                     for (int s = 0; s < KW; ++s) {
-                        const int i = lane + 32 * s;
+                        const int i = slot_index<KW>(lane, s);
                         bool f = false;
                         if (i < k) {
                             const uint64_t wv = P.pin[j * P.nwords + (i >> 6)];
@@ -576,18 +758,37 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                     int rank[KW];
                     int pos = 0;
                     __syncwarp();
+                    if constexpr (KW == 4) {
+                        int r = 0;
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) {
-                        inS[s] = comp ? (usable[s] && !inF[s]) : inF[s];
-                        const unsigned mk = __ballot_sync(FULL, inS[s]);
-                        rank[s] = pos + __popc(mk & lanemask_lt(lane));
-                        if (inS[s]) {
-                            widx[rank[s]] = lane + 32 * s;
-                            zbuf[rank[s]] = comp ? -u[s] : g[s];
-                            if constexpr (KW <= 2)
-                                wcol[rank[s]] = lane * KW + s;
+                        for (int s = 0; s < KW; ++s) {
+                            inS[s] = comp ? (usable[s] && !inF[s]) : inF[s];
+                            const unsigned mk = __ballot_sync(FULL, inS[s]);
+                            r += __popc(mk & lanemask_lt(lane));
+                            pos += __popc(mk);
                         }
-                        pos += __popc(mk);
+#pragma unroll
+                        for (int s = 0; s < KW; ++s) {
+                            rank[s] = r;
+                            if (inS[s]) {
+                                widx[r] = 4 * lane + s;
+                                zbuf[r] = comp ? -u[s] : g[s];
+                                ++r;
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int s = 0; s < KW; ++s) {
+                            inS[s] = comp ? (usable[s] && !inF[s]) : inF[s];
+                            const unsigned mk = __ballot_sync(FULL, inS[s]);
+                            rank[s] = pos + __popc(mk & lanemask_lt(lane));
+                            if (inS[s]) {
+                                widx[rank[s]] = lane + 32 * s;
+                                zbuf[rank[s]] = comp ? -u[s] : g[s];
+                                wcol[rank[s]] = lane * KW + s;
+                            }
+                            pos += __popc(mk);
+                        }
                     }
                     const int p = pos, p4 = (p + 3) & ~3;
                     if (lane < p4 - p) {
@@ -603,7 +804,8 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             !ldl_regs<KW, PM>(comp ? Ms : Gs, widx, wcol, p, Lw, LS, rp, lane))
                             return DEFERRED;
                     } else {
-                        if (p > 0 && !chol32<KW, PT>(comp ? Ms : Gs, widx, p, Lw, LS, inv, lane))
+                        if (p > 32 ? !chol32<PT>(comp ? Ms : Gs, widx, p, Lw, inv, RS, lane)
+                                   : p > 0 && !ldl_cols(comp ? Ms : Gs, widx, p, Lw, rp, RS, lane))
                             return DEFERRED;
                     }
                     // Pass 0 solves the system (zbuf = g_F, or -u_A in the
@@ -624,8 +826,10 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             }
                             if constexpr (KW <= 2)
                                 r[0] = ldl_solve(Lw, LS, rp, p, r[0], lane);
+                            else if (p > 32)
+                                subst32<PT>(p, Lw, inv, r, lane);
                             else
-                                subst32<PT>(p, Lw, LS, inv, r, lane);
+                                r[0] = ldl_cols_solve(Lw, rp, p, r[0], lane);
                             __syncwarp();
 #pragma unroll
                             for (int t = 0; t < PT; ++t)
@@ -636,7 +840,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         // The step: dx_F from the direct solution, or
                         // base_F + M_FA z_A from the complement one.
                         if (comp)
-                            mv_list<KW>(Ms, widx, zbuf, p4, base, lane);
+                            mv_list<KW>(Ms, widx, zbuf, p4, base, k4, lane);
 #pragma unroll
                         for (int s = 0; s < KW; ++s) {
                             const float dx = inF[s] ? (comp ? base[s] : zbuf[rank[s]]) : 0.0f;
@@ -652,7 +856,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                                 if (inS[s])
                                     zbuf[rank[s]] = x[s];
                             __syncwarp();
-                            mv_list<KW>(Gs, widx, zbuf, p4, w, lane);
+                            mv_list<KW>(Gs, widx, zbuf, p4, w, k4, lane);
                         } else {
                             stage_vec<KW>(stage, x, lane);
                             mv_full<KW>(Gs, k4, stage, w, lane);
@@ -731,13 +935,21 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             inF[s] = inF[s] != inf[s];
                     } else {   // backup rule: the largest infeasible index alone
                         int top = -1;
+                        if constexpr (KW == 4) {
 #pragma unroll
-                        for (int s = KW - 1; s >= 0; --s)
-                            if (top < 0 && vm[s])
-                                top = 32 * s + 31 - __clz(vm[s]);
+                            for (int s = 0; s < KW; ++s)
+                                if (inf[s])
+                                    top = 4 * lane + s;
+                            top = __reduce_max_sync(FULL, top);
+                        } else {
+#pragma unroll
+                            for (int s = KW - 1; s >= 0; --s)
+                                if (top < 0 && vm[s])
+                                    top = 32 * s + 31 - __clz(vm[s]);
+                        }
 #pragma unroll
                         for (int s = 0; s < KW; ++s)
-                            if (lane + 32 * s == top)
+                            if (slot_index<KW>(lane, s) == top)
                                 inF[s] = !inF[s];
                     }
                     rounds += 1;
@@ -757,24 +969,17 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                 // Only the partition reached seeds the FP64 solves; where the
                 // FP32 system was singular, the starting one (given or empty).
                 if (P.pout) {
-                    unsigned bm[KW];
+                    bool f[KW];
 #pragma unroll
                     for (int s = 0; s < KW; ++s) {
-                        bool f = inF[s];
+                        f[s] = inF[s];
                         if (status == DEFERRED) {
-                            const int i = lane + 32 * s;
-                            f = P.pin && i < k && ((P.pin[j * P.nwords + (i >> 6)] >> (i & 63)) & 1ull);
-                        }
-                        bm[s] = __ballot_sync(FULL, f);
-                    }
-                    if (lane == 0) {
-#pragma unroll
-                        for (int w = 0; w < (KW + 1) / 2; ++w) {
-                            const uint64_t lo = bm[2 * w];
-                            const uint64_t hi = (2 * w + 1 < KW) ? bm[2 * w + 1] : 0u;
-                            P.pout[j * P.nwords + w] = lo | (hi << 32);
+                            const int i = slot_index<KW>(lane, s);
+                            f[s] = P.pin && i < k &&
+                                   ((P.pin[j * P.nwords + (i >> 6)] >> (i & 63)) & 1ull);
                         }
                     }
+                    write_words<KW>(f, P.pout + j * P.nwords, lane);
                 }
                 continue;
             }
@@ -789,24 +994,12 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
             }
 #pragma unroll
             for (int s = 0; s < KW; ++s) {
-                const int i = lane + 32 * s;
+                const int i = slot_index<KW>(lane, s);
                 if (i < k)
                     P.X[j * k + i] = x[s];
             }
-            if (P.pout) {
-                unsigned bm[KW];
-#pragma unroll
-                for (int s = 0; s < KW; ++s)
-                    bm[s] = __ballot_sync(FULL, inF[s]);
-                if (lane == 0) {
-#pragma unroll
-                    for (int w = 0; w < (KW + 1) / 2; ++w) {
-                        const uint64_t lo = bm[2 * w];
-                        const uint64_t hi = (2 * w + 1 < KW) ? bm[2 * w + 1] : 0u;
-                        P.pout[j * P.nwords + w] = lo | (hi << 32);
-                    }
-                }
-            }
+            if (P.pout)
+                write_words<KW>(inF, P.pout + j * P.nwords, lane);
             if (lane == 0) {
                 if (P.rounds_out)
                     P.rounds_out[j] = rounds;
@@ -838,13 +1031,13 @@ nmf_status launch32(const SolveParams &P, cudaStream_t s)
 {
     const int k = P.k;
     const int pmax = k / 2 > 1 ? k / 2 : 1;   // min(|F|, |A|) <= k / 2
-    int q = (pmax + 1) / 2;
-    if (!(q & 1))
-        ++q;
-    // k > 64: 2 * odd, conflict-free float2 row reads and column accesses;
-    // k <= 64: odd, conflict-free rows and columns of single floats.
-    const int LS = KW <= 2 ? (pmax | 1) : 2 * q;
-    int nwarps = P.warps < S32_MAX_WARPS ? P.warps : S32_MAX_WARPS;
+    const int LS = pmax | 1;   // k <= 64: odd, conflict-free rows and columns
+    // k > 64: G and M leave one CTA per SM, which takes twice the shape's warps
+    // (k = 100: 24.9 ms for 1000000 right-hand sides of mixed signs with 16
+    // warps, 32.7 with 8; 41.4 before, with 8 and rows padded to 128).
+    int nwarps = KW == 4 ? 2 * P.warps : P.warps;
+    if (nwarps > S32_MAX_WARPS)
+        nwarps = S32_MAX_WARPS;
     const size_t mats = mats_bytes32(k, KW);
     auto bytes = [&](int nw) { return mats + (size_t)nw * warp_bytes32(KW, pmax, LS); };
     while (nwarps > 1 && bytes(nwarps) > SMEM_LIMIT32)
