@@ -160,6 +160,71 @@ __device__ __forceinline__ void mv_list(const float *__restrict__ Mat, const int
         out[s] += a1[s];
 }
 
+// k > 64: out += Mat^T vec for a vec that is zero off a set F, over the rows of
+// F only. off holds the rows' offsets and val their entries of vec, the even
+// rows at even places and the odd rows at odd places, n2 of each (padded with
+// offset 0 and value 0): the additions are those of mv_full without its zeros.
+__device__ __forceinline__ void mv_set(const float *__restrict__ Mat, const int *__restrict__ off,
+                                       const float *__restrict__ val, int n2, float (&out)[4],
+                                       int lane)
+{
+    float a1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const float *base = Mat + lane * 4;
+    for (int a = 0; a < 2 * n2; a += 4) {
+        const int4 c = *reinterpret_cast<const int4 *>(off + a);
+        const float4 v = *reinterpret_cast<const float4 *>(val + a);
+        row_fma<4>(base + c.x, v.x, out);
+        row_fma<4>(base + c.y, v.y, a1);
+        row_fma<4>(base + c.z, v.z, out);
+        row_fma<4>(base + c.w, v.w, a1);
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+        out[s] += a1[s];
+}
+
+// k > 64: lane a gets sum_i Mat[idx[a]][i] x_i for the p <= 32 rows of a list
+// (padded with 0 to a multiple of four; lanes past p get values of no use).
+// Each lane adds up its own four indices of every row, then the 32 sums are
+// reduced across the lanes and dealt out in one butterfly (31 shuffles).
+__device__ __forceinline__ float mv_rows(const float *__restrict__ Mat, const int *__restrict__ idx,
+                                         int p, const float (&x)[4], int k4, int lane)
+{
+    // (Lanes past the row's end, whose x is zero, read its last entries.)
+    const float *base = Mat + (4 * lane < k4 ? 4 * lane : k4 - 4);
+    float t[32];
+#pragma unroll
+    for (int b0 = 0; b0 < 32; b0 += 4) {
+        if (b0 < p) {
+            const int4 c = *reinterpret_cast<const int4 *>(idx + b0);
+            const int r[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 m = *reinterpret_cast<const float4 *>(base + r[q] * k4);
+                const float2 h = __ffma2_rn(make_float2(m.z, m.w), make_float2(x[2], x[3]),
+                                            __fmul2_rn(make_float2(m.x, m.y),
+                                                       make_float2(x[0], x[1])));
+                t[b0 + q] = h.x + h.y;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                t[b0 + q] = 0.0f;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const float give = up ? t[i] : t[i + o];
+            const float keep = up ? t[i + o] : t[i];
+            t[i] = keep + __shfl_xor_sync(FULL, give, o);
+        }
+    }
+    return t[0];
+}
+
 template <int KW>
 __device__ __forceinline__ void stage_vec(float *__restrict__ stage, const float (&v)[KW], int lane)
 {
@@ -530,7 +595,7 @@ __device__ __forceinline__ float ldl_solve(const float *__restrict__ Lw, int LS,
 
 // Shared memory: G and M (k rounded up to 4 rows of row_stride floats each),
 // then per warp an index list, its values, the list's column offsets (KW <= 2),
-// a staging vector and the factor (pmax x LS floats, KW <= 2; the larger of
+// a staging vector (KW = 4: also the set product's row offsets) and the factor (pmax x LS floats, KW <= 2; the larger of
 // ldl_cols's and the packed triangle of pmax rows, KW = 4).
 __host__ __device__ inline size_t mats_bytes32(int k, int KW)
 {
@@ -547,7 +612,7 @@ __host__ __device__ inline size_t warp_bytes32(int KW, int pmax, int LS)
 {
     if (KW == 4) {
         const int fac = tri_off(pmax) > 32 * LDL_LS ? tri_off(pmax) : 32 * LDL_LS;
-        return (sizeof(float) * (size_t)(2 * list_len(4, pmax) + 128 + fac) + 15) & ~size_t(15);
+        return (sizeof(float) * (size_t)(2 * list_len(4, pmax) + 256 + fac) + 15) & ~size_t(15);
     }
     // 32 floats of slack after the factor (read past its end by the unrolled
     // substitutions).
@@ -589,7 +654,8 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     float *zbuf = reinterpret_cast<float *>(widx + LL);
     float *stage = zbuf + LL;
     int *wcol = reinterpret_cast<int *>(stage + 32 * KW);   // KW <= 2: column offsets of the list
-    float *Lw = stage + 32 * KW + (KW <= 2 ? LL : 0);
+    int *foff = reinterpret_cast<int *>(stage + 128);   // KW = 4: row offsets of the set F
+    float *Lw = stage + (KW <= 2 ? 32 * KW + LL : 256);
     __syncthreads();
 
     bool usable[KW];
@@ -799,6 +865,47 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                     }
                     __syncwarp();
                     float inv[PT], rp = 0.0f;
+                    // KW = 4, complement form: products with vectors on F go
+                    // over its rows (mv_set): their offsets, and the place of
+                    // each index's value in the staging vector.
+                    int place[KW], n2 = 0;
+                    if constexpr (KW == 4) {
+                        if (comp) {
+                            int ne = 0, no = 0, re = 0, ro = 0;
+#pragma unroll
+                            for (int s = 0; s < KW; ++s) {
+                                const unsigned mk = __ballot_sync(FULL, inF[s]);
+                                (s & 1 ? no : ne) += __popc(mk);
+                                (s & 1 ? ro : re) += __popc(mk & lanemask_lt(lane));
+                            }
+#pragma unroll
+                            for (int s = 0; s < KW; ++s) {
+                                int &r = s & 1 ? ro : re;
+                                place[s] = 2 * r + (s & 1);
+                                if (inF[s]) {
+                                    foff[place[s]] = (4 * lane + s) * RS;
+                                    ++r;
+                                }
+                            }
+                            n2 = ((ne > no ? ne : no) + 1) & ~1;
+                            for (int a = ne + lane; a < n2; a += 32) {
+                                foff[2 * a] = 0;
+                                stage[2 * a] = 0.0f;
+                            }
+                            for (int a = no + lane; a < n2; a += 32) {
+                                foff[2 * a + 1] = 0;
+                                stage[2 * a + 1] = 0.0f;
+                            }
+                        }
+                    }
+                    auto stage_set = [&](const float (&v)[KW]) {
+                        __syncwarp();
+#pragma unroll
+                        for (int s = 0; s < KW; ++s)
+                            if (inF[s])
+                                stage[place[s]] = v[s];
+                        __syncwarp();
+                    };
                     if constexpr (KW <= 2) {
                         if (p > 0 &&
                             !ldl_regs<KW, PM>(comp ? Ms : Gs, widx, wcol, p, Lw, LS, rp, lane))
@@ -857,6 +964,21 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                                     zbuf[rank[s]] = x[s];
                             __syncwarp();
                             mv_list<KW>(Gs, widx, zbuf, p4, w, k4, lane);
+                        } else if constexpr (KW == 4) {
+                            if (pass == 0 || p > 32) {
+                                stage_set(x);
+                                mv_set(Gs, foff, stage, n2, w, lane);
+                            } else if (p > 0) {   // y is all that is left to form
+                                const float t = mv_rows(Gs, widx, p, x, k4, lane);
+                                __syncwarp();
+                                if (lane < p)
+                                    zbuf[lane] = t;
+                                __syncwarp();
+#pragma unroll
+                                for (int s = 0; s < KW; ++s)
+                                    if (inS[s])
+                                        w[s] = zbuf[rank[s]];
+                            }
                         } else {
                             stage_vec<KW>(stage, x, lane);
                             mv_full<KW>(Gs, k4, stage, w, lane);
@@ -870,8 +992,13 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             base[s] = 0.0f;
                         }
                         if (comp) {
-                            stage_vec<KW>(stage, res, lane);
-                            mv_full<KW>(Ms, k4, stage, base, lane);   // up = M res
+                            if constexpr (KW == 4) {
+                                stage_set(res);
+                                mv_set(Ms, foff, stage, n2, base, lane);   // up = M res
+                            } else {
+                                stage_vec<KW>(stage, res, lane);
+                                mv_full<KW>(Ms, k4, stage, base, lane);
+                            }
                         }
                         __syncwarp();
 #pragma unroll
