@@ -475,7 +475,7 @@ __device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, fl
 }
 
 // Systems of at most PM rows (k <= 64; PM >= k / 2 >= p): LDL^T of
-// S_ab = Src(idx[a], idx[b]) with lane a keeping the live part of row a in
+// S_ab = Src(idx[a], idx[b]), with lane a keeping the live part of row a in
 // registers. At step j, s[0 .. p - j) holds columns j .. p - 1 of row a of the
 // trailing (Schur complement) matrix; the update writes column b + 1 into
 // s[b], so the row shifts one place per step and every register index stays a
@@ -483,28 +483,30 @@ __device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, fl
 // overflowed the instruction cache). Row j reaches the other lanes by
 // shuffles, four columns at a time up to the live width. The multipliers
 // L_aj = S_aj / S_jj go to Lw[a * LS + j] (LS odd: conflict-free rows and
-// columns); lane a keeps rp = 1 / D_aa. col[b] is the offset of column
-// idx[b] within a row of Src (the list padded to a multiple of four with
-// offset 0). Returns false (uniformly) when a pivot is at most PIVOT_TOL of
+// columns); lane a keeps rp = 1 / D_aa. row[b] is the offset of row idx[b] of
+// Src (the list padded to a multiple of four with offset 0). The system is
+// read by columns, S_ab = Src(idx[b], idx[a]): the rows start at the same
+// shared-memory bank, so that lanes reading one column of their own rows wait
+// for one another (p-fold conflicts, a third of the kernel's wavefronts on the
+// sparse 200000 x 100000 solves). Returns false (uniformly) when a pivot is at most PIVOT_TOL of
 // its diagonal.
 template <int KW, int PM>
 __device__ __forceinline__ bool ldl_regs(const float *__restrict__ Src, const int *__restrict__ idx,
-                                         const int *__restrict__ col, int p,
+                                         const int *__restrict__ row, int p,
                                          float *__restrict__ Lw, int LS, float &rp, int lane)
 {
-    constexpr int RS = 32 * KW;
     const int c = lane < p ? idx[lane] : 0;
-    const float *row = Src + c * RS;
-    const float dtol = PIVOT_TOL * row[(c & 31) * KW + (c >> 5)];
+    const float *col = Src + col_offset<KW>(c);
+    const float dtol = PIVOT_TOL * col[lane < p ? row[lane] : 0];
     float s[PM];
 #pragma unroll
     for (int b0 = 0; b0 < PM; b0 += 4) {
         if (b0 < p) {
-            const int4 o = *reinterpret_cast<const int4 *>(col + b0);
-            s[b0] = row[o.x];
-            s[b0 + 1] = row[o.y];
-            s[b0 + 2] = row[o.z];
-            s[b0 + 3] = row[o.w];
+            const int4 o = *reinterpret_cast<const int4 *>(row + b0);
+            s[b0] = col[o.x];
+            s[b0 + 1] = col[o.y];
+            s[b0 + 2] = col[o.z];
+            s[b0 + 3] = col[o.w];
         } else {
 #pragma unroll
             for (int b = b0; b < b0 + 4; ++b)
@@ -594,7 +596,7 @@ __device__ __forceinline__ float ldl_solve(const float *__restrict__ Lw, int LS,
 }
 
 // Shared memory: G and M (k rounded up to 4 rows of row_stride floats each),
-// then per warp an index list, its values, the list's column offsets (KW <= 2),
+// then per warp an index list, its values, the list's row offsets (KW <= 2),
 // a staging vector (KW = 4: also the set product's row offsets) and the factor (pmax x LS floats, KW <= 2; the larger of
 // ldl_cols's and the packed triangle of pmax rows, KW = 4).
 __host__ __device__ inline size_t mats_bytes32(int k, int KW)
@@ -602,7 +604,7 @@ __host__ __device__ inline size_t mats_bytes32(int k, int KW)
     const size_t k4 = (size_t)((k + 3) & ~3);
     return 2 * sizeof(float) * k4 * (KW == 4 ? k4 : 32 * KW);
 }
-// Entries of the index list, its values and column offsets (systems of at most
+// Entries of the index list, its values and row offsets (systems of at most
 // pmax rows, padded to a multiple of four).
 __host__ __device__ constexpr int list_len(int KW, int pmax)
 {
@@ -653,7 +655,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     int *widx = reinterpret_cast<int *>(wp);
     float *zbuf = reinterpret_cast<float *>(widx + LL);
     float *stage = zbuf + LL;
-    int *wcol = reinterpret_cast<int *>(stage + 32 * KW);   // KW <= 2: column offsets of the list
+    int *wrow = reinterpret_cast<int *>(stage + 32 * KW);   // KW <= 2: row offsets of the list
     int *foff = reinterpret_cast<int *>(stage + 128);   // KW = 4: row offsets of the set F
     float *Lw = stage + (KW <= 2 ? 32 * KW + LL : 256);
     __syncthreads();
@@ -851,7 +853,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             if (inS[s]) {
                                 widx[rank[s]] = lane + 32 * s;
                                 zbuf[rank[s]] = comp ? -u[s] : g[s];
-                                wcol[rank[s]] = lane * KW + s;
+                                wrow[rank[s]] = (lane + 32 * s) * RS;
                             }
                             pos += __popc(mk);
                         }
@@ -861,7 +863,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         widx[p + lane] = 0;
                         zbuf[p + lane] = 0.0f;
                         if constexpr (KW <= 2)
-                            wcol[p + lane] = 0;
+                            wrow[p + lane] = 0;
                     }
                     __syncwarp();
                     float inv[PT], rp = 0.0f;
@@ -908,7 +910,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                     };
                     if constexpr (KW <= 2) {
                         if (p > 0 &&
-                            !ldl_regs<KW, PM>(comp ? Ms : Gs, widx, wcol, p, Lw, LS, rp, lane))
+                            !ldl_regs<KW, PM>(comp ? Ms : Gs, widx, wrow, p, Lw, LS, rp, lane))
                             return DEFERRED;
                     } else {
                         if (p > 32 ? !chol32<PT>(comp ? Ms : Gs, widx, p, Lw, inv, RS, lane)
