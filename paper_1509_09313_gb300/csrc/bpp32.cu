@@ -134,26 +134,26 @@ __device__ __forceinline__ void mv_full(const float *__restrict__ Mat, int k4,
         out[s] += a1[s];
 }
 
-// out += sum_a Mat[idx[a]] * val[a] over a list padded to n4 entries (the
-// padding has idx 0 and val 0).
+// out += sum_a (row a) * val[a] over a list of row offsets padded to n4 entries
+// (the padding has offset 0 and val 0).
 template <int KW>
-__device__ __forceinline__ void mv_list(const float *__restrict__ Mat, const int *__restrict__ idx,
+__device__ __forceinline__ void mv_list(const float *__restrict__ Mat, const int *__restrict__ off,
                                         const float *__restrict__ val, int n4, float (&out)[KW],
-                                        int k4, int lane)
+                                        int lane)
 {
-    const int RS = row_stride<KW>(k4);
     float a1[KW];
 #pragma unroll
     for (int s = 0; s < KW; ++s)
         a1[s] = 0.0f;
     const float *base = Mat + lane * KW;
+#pragma unroll 1
     for (int a = 0; a < n4; a += 4) {
-        const int4 c = *reinterpret_cast<const int4 *>(idx + a);
+        const int4 c = *reinterpret_cast<const int4 *>(off + a);
         const float4 v = *reinterpret_cast<const float4 *>(val + a);
-        row_fma<KW>(base + c.x * RS, v.x, out);
-        row_fma<KW>(base + c.y * RS, v.y, a1);
-        row_fma<KW>(base + c.z * RS, v.z, out);
-        row_fma<KW>(base + c.w * RS, v.w, a1);
+        row_fma<KW>(base + c.x, v.x, out);
+        row_fma<KW>(base + c.y, v.y, a1);
+        row_fma<KW>(base + c.z, v.z, out);
+        row_fma<KW>(base + c.w, v.w, a1);
     }
 #pragma unroll
     for (int s = 0; s < KW; ++s)
@@ -183,11 +183,11 @@ __device__ __forceinline__ void mv_set(const float *__restrict__ Mat, const int 
         out[s] += a1[s];
 }
 
-// k > 64: lane a gets sum_i Mat[idx[a]][i] x_i for the p <= 32 rows of a list
-// (padded with 0 to a multiple of four; lanes past p get values of no use).
+// k > 64: lane a gets sum_i (row a)_i x_i for the p <= 32 rows of a list of
+// offsets (padded with 0 to a multiple of four; lanes past p get values of no use).
 // Each lane adds up its own four indices of every row, then the 32 sums are
 // reduced across the lanes and dealt out in one butterfly (31 shuffles).
-__device__ __forceinline__ float mv_rows(const float *__restrict__ Mat, const int *__restrict__ idx,
+__device__ __forceinline__ float mv_rows(const float *__restrict__ Mat, const int *__restrict__ off,
                                          int p, const float (&x)[4], int k4, int lane)
 {
     // (Lanes past the row's end, whose x is zero, read its last entries.)
@@ -196,11 +196,11 @@ __device__ __forceinline__ float mv_rows(const float *__restrict__ Mat, const in
 #pragma unroll
     for (int b0 = 0; b0 < 32; b0 += 4) {
         if (b0 < p) {
-            const int4 c = *reinterpret_cast<const int4 *>(idx + b0);
+            const int4 c = *reinterpret_cast<const int4 *>(off + b0);
             const int r[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float4 m = *reinterpret_cast<const float4 *>(base + r[q] * k4);
+                const float4 m = *reinterpret_cast<const float4 *>(base + r[q]);
                 const float2 h = __ffma2_rn(make_float2(m.z, m.w), make_float2(x[2], x[3]),
                                             __fmul2_rn(make_float2(m.x, m.y),
                                                        make_float2(x[0], x[1])));
@@ -374,19 +374,20 @@ __device__ __forceinline__ void subst32(int p, const float *__restrict__ Lw,
 // allow this here; at k <= 64, with 64, it spilled.
 constexpr int LDL_LS = 36;   // a multiple of 4; LDL_LS - 1 odd: conflict-free rows and columns
 __device__ __forceinline__ bool ldl_cols(const float *__restrict__ Src, const int *__restrict__ idx,
-                                         int p, float *__restrict__ Lc, float &rp, int RS, int lane)
+                                         const int *__restrict__ row, int p,
+                                         float *__restrict__ Lc, float &rp, int lane)
 {
-    const int c = lane < p ? idx[lane] : 0;
-    const float dtol = PIVOT_TOL * Src[c * RS + c];
+    const float *col = Src + (lane < p ? idx[lane] : 0);
+    const float dtol = PIVOT_TOL * col[lane < p ? row[lane] : 0];
     float s[32];
 #pragma unroll
     for (int b0 = 0; b0 < 32; b0 += 4) {
         if (b0 < p) {
-            const int4 o = *reinterpret_cast<const int4 *>(idx + b0);
-            s[b0] = Src[o.x * RS + c];
-            s[b0 + 1] = Src[o.y * RS + c];
-            s[b0 + 2] = Src[o.z * RS + c];
-            s[b0 + 3] = Src[o.w * RS + c];
+            const int4 o = *reinterpret_cast<const int4 *>(row + b0);
+            s[b0] = col[o.x];
+            s[b0 + 1] = col[o.y];
+            s[b0 + 2] = col[o.z];
+            s[b0 + 3] = col[o.w];
         } else {
 #pragma unroll
             for (int b = b0; b < b0 + 4; ++b)
@@ -396,19 +397,19 @@ __device__ __forceinline__ bool ldl_cols(const float *__restrict__ Src, const in
     bool ok = true;
     rp = 0.0f;
     for (int j = 0; j < p; ++j) {
-        float *col = Lc + j * LDL_LS;
+        float *fc = Lc + j * LDL_LS;
         if (lane >= j && lane < p)
-            col[lane - j] = s[0];
+            fc[lane - j] = s[0];
         __syncwarp();
         const int w = p - j;   // live columns: s[0 .. w)
-        const float4 c0 = *reinterpret_cast<const float4 *>(col);
+        const float4 c0 = *reinterpret_cast<const float4 *>(fc);
         const float q = rsqrtf(c0.x);
         const float r = q * q;
         if (lane == j) {
             ok = c0.x > dtol;
             rp = r;
         }
-        // (Entries of col past the live columns are not set: they only reach
+        // (Entries of fc past the live columns are not set: they only reach
         // registers past the live ones.)
         const float m = s[0] * r;
         s[0] = fmaf(-m, c0.y, s[1]);
@@ -418,7 +419,7 @@ __device__ __forceinline__ bool ldl_cols(const float *__restrict__ Src, const in
         for (int b0 = 4; b0 < 32; b0 += 4) {
             if (b0 >= w)
                 break;
-            const float4 cv = *reinterpret_cast<const float4 *>(col + b0);
+            const float4 cv = *reinterpret_cast<const float4 *>(fc + b0);
             s[b0 - 1] = fmaf(-m, cv.x, s[b0]);
             s[b0] = fmaf(-m, cv.y, s[b0 + 1]);
             s[b0 + 1] = fmaf(-m, cv.z, s[b0 + 2]);
@@ -437,6 +438,7 @@ __device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, fl
 {
     const float *fw = Lc + lane, *bw = Lc + lane * (LDL_LS - 1);
     int j = 0;
+#pragma unroll 1
     for (; j + 4 < p; j += 4) {
         const float l0 = fw[j * (LDL_LS - 1)], l1 = fw[(j + 1) * (LDL_LS - 1)];
         const float l2 = fw[(j + 2) * (LDL_LS - 1)], l3 = fw[(j + 3) * (LDL_LS - 1)];
@@ -449,12 +451,14 @@ __device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, fl
         t = __shfl_sync(FULL, v * rp, j + 3);
         if (lane > j + 3) v = fmaf(-l3, t, v);
     }
+#pragma unroll 1
     for (; j + 1 < p; ++j) {
         const float t = __shfl_sync(FULL, v * rp, j);
         if (lane > j)
             v = fmaf(-fw[j * (LDL_LS - 1)], t, v);
     }
     j = p - 1;
+#pragma unroll 1
     for (; j >= 4; j -= 4) {
         const float l0 = bw[j], l1 = bw[j - 1], l2 = bw[j - 2], l3 = bw[j - 3];
         float z = __shfl_sync(FULL, v * rp, j);
@@ -466,6 +470,7 @@ __device__ __forceinline__ float ldl_cols_solve(const float *__restrict__ Lc, fl
         z = __shfl_sync(FULL, v * rp, j - 3);
         if (lane < j - 3) v = fmaf(-l3, z, v);
     }
+#pragma unroll 1
     for (; j >= 1; --j) {
         const float z = __shfl_sync(FULL, v * rp, j);
         if (lane < j)
@@ -515,6 +520,7 @@ __device__ __forceinline__ bool ldl_regs(const float *__restrict__ Src, const in
     }
     bool ok = true;
     rp = 0.0f;
+    float *lrow = Lw + lane * LS;
     for (int j = 0; j < p; ++j) {
         const float d = __shfl_sync(FULL, s[0], j);
         const float q = rsqrtf(d);
@@ -523,10 +529,9 @@ __device__ __forceinline__ bool ldl_regs(const float *__restrict__ Src, const in
             ok = d > dtol;
             rp = r;
         }
-        const bool below = lane > j && lane < p;
-        const float m = below ? s[0] * r : 0.0f;
-        if (below)
-            Lw[lane * LS + j] = m;
+        const float m = lane > j ? s[0] * r : 0.0f;
+        if (lane < p)
+            lrow[j] = m;   // zero on and above the diagonal
         const int w = p - j;   // live columns: s[0 .. w)
 #pragma unroll
         for (int b0 = 0; b0 < PM; b0 += 4) {
@@ -541,64 +546,55 @@ __device__ __forceinline__ bool ldl_regs(const float *__restrict__ Src, const in
 }
 
 // Solve S z = r with the factor of ldl_regs (row a of r and z in lane a):
-// L y = r forward, then L^T z = D^{-1} y backward. Four steps at a time with
-// their multipliers loaded first, so only the shuffle and the FMA of each step
-// are on the dependency chain (a lane's loads may run past its row or the
+// L y = r forward, then L^T z = D^{-1} y backward. The factor's zeros on and
+// above its diagonal keep a step from the lanes it does not concern, without a
+// test: a lane's value is final from its own step on. Four steps at a time
+// with their multipliers loaded first, so only the shuffle and the FMA of each
+// step are on the dependency chain (a lane's loads may run past its row or the
 // factor: the per-warp area ends with 32 floats of slack; lanes >= p carry
-// values that are never read).
+// values that are never read). The loops are kept rolled: unrolled further by
+// the compiler, they cost more in instruction fetch than the tests they drop
+// save (sparse 200000 x 100000, three iterations: 7.1 ms against 6.3; 6.65
+// with the tests).
 __device__ __forceinline__ float ldl_solve(const float *__restrict__ Lw, int LS, float rp, int p,
                                            float r, int lane)
 {
     const float *lrow = Lw + (lane < p ? lane : 0) * LS;
     int j = 0;
+#pragma unroll 1
     for (; j + 4 < p; j += 4) {
         const float l0 = lrow[j], l1 = lrow[j + 1], l2 = lrow[j + 2], l3 = lrow[j + 3];
-        float t = __shfl_sync(FULL, r, j);
-        if (lane > j) r = fmaf(-l0, t, r);
-        t = __shfl_sync(FULL, r, j + 1);
-        if (lane > j + 1) r = fmaf(-l1, t, r);
-        t = __shfl_sync(FULL, r, j + 2);
-        if (lane > j + 2) r = fmaf(-l2, t, r);
-        t = __shfl_sync(FULL, r, j + 3);
-        if (lane > j + 3) r = fmaf(-l3, t, r);
+        r = fmaf(-l0, __shfl_sync(FULL, r, j), r);
+        r = fmaf(-l1, __shfl_sync(FULL, r, j + 1), r);
+        r = fmaf(-l2, __shfl_sync(FULL, r, j + 2), r);
+        r = fmaf(-l3, __shfl_sync(FULL, r, j + 3), r);
     }
-    for (; j + 1 < p; ++j) {
-        const float t = __shfl_sync(FULL, r, j);
-        if (lane > j)
-            r = fmaf(-lrow[j], t, r);
-    }
-    float v = r * rp, z = 0.0f;
+#pragma unroll 1
+    for (; j + 1 < p; ++j)
+        r = fmaf(-lrow[j], __shfl_sync(FULL, r, j), r);
+    float v = r * rp;
+    const float *lcol = Lw + lane;
     j = p - 1;
-    for (; j >= 3; j -= 4) {
-        const float l0 = Lw[j * LS + lane], l1 = Lw[(j - 1) * LS + lane];
-        const float l2 = Lw[(j - 2) * LS + lane], l3 = Lw[(j - 3) * LS + lane];
-        float zj = __shfl_sync(FULL, v, j);
-        if (lane < j) v = fmaf(-l0, zj, v);
-        if (lane == j) z = zj;
-        zj = __shfl_sync(FULL, v, j - 1);
-        if (lane < j - 1) v = fmaf(-l1, zj, v);
-        if (lane == j - 1) z = zj;
-        zj = __shfl_sync(FULL, v, j - 2);
-        if (lane < j - 2) v = fmaf(-l2, zj, v);
-        if (lane == j - 2) z = zj;
-        zj = __shfl_sync(FULL, v, j - 3);
-        if (lane < j - 3) v = fmaf(-l3, zj, v);
-        if (lane == j - 3) z = zj;
+#pragma unroll 1
+    for (; j >= 4; j -= 4) {
+        const float l0 = lcol[j * LS], l1 = lcol[(j - 1) * LS];
+        const float l2 = lcol[(j - 2) * LS], l3 = lcol[(j - 3) * LS];
+        v = fmaf(-l0, __shfl_sync(FULL, v, j), v);
+        v = fmaf(-l1, __shfl_sync(FULL, v, j - 1), v);
+        v = fmaf(-l2, __shfl_sync(FULL, v, j - 2), v);
+        v = fmaf(-l3, __shfl_sync(FULL, v, j - 3), v);
     }
-    for (; j >= 0; --j) {
-        const float zj = __shfl_sync(FULL, v, j);
-        if (lane < j)
-            v = fmaf(-Lw[j * LS + lane], zj, v);
-        if (lane == j)
-            z = zj;
-    }
-    return z;
+#pragma unroll 1
+    for (; j >= 1; --j)
+        v = fmaf(-lcol[j * LS], __shfl_sync(FULL, v, j), v);
+    return v;
 }
 
 // Shared memory: G and M (k rounded up to 4 rows of row_stride floats each),
-// then per warp an index list, its values, the list's row offsets (KW <= 2),
-// a staging vector (KW = 4: also the set product's row offsets) and the factor (pmax x LS floats, KW <= 2; the larger of
-// ldl_cols's and the packed triangle of pmax rows, KW = 4).
+// then per warp an index list, its values, a staging vector, the list's row
+// offsets, (KW = 4) the row offsets of the set F, and the factor (KW <= 2:
+// pmax x LS floats; KW = 4: the larger of ldl_cols's and the packed triangle of
+// pmax rows).
 __host__ __device__ inline size_t mats_bytes32(int k, int KW)
 {
     const size_t k4 = (size_t)((k + 3) & ~3);
@@ -614,7 +610,7 @@ __host__ __device__ inline size_t warp_bytes32(int KW, int pmax, int LS)
 {
     if (KW == 4) {
         const int fac = tri_off(pmax) > 32 * LDL_LS ? tri_off(pmax) : 32 * LDL_LS;
-        return (sizeof(float) * (size_t)(2 * list_len(4, pmax) + 256 + fac) + 15) & ~size_t(15);
+        return (sizeof(float) * (size_t)(3 * list_len(4, pmax) + 256 + fac) + 15) & ~size_t(15);
     }
     // 32 floats of slack after the factor (read past its end by the unrolled
     // substitutions).
@@ -655,9 +651,9 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     int *widx = reinterpret_cast<int *>(wp);
     float *zbuf = reinterpret_cast<float *>(widx + LL);
     float *stage = zbuf + LL;
-    int *wrow = reinterpret_cast<int *>(stage + 32 * KW);   // KW <= 2: row offsets of the list
-    int *foff = reinterpret_cast<int *>(stage + 128);   // KW = 4: row offsets of the set F
-    float *Lw = stage + (KW <= 2 ? 32 * KW + LL : 256);
+    int *wrow = reinterpret_cast<int *>(stage + 32 * KW);   // row offsets of the list
+    int *foff = wrow + LL;                                  // KW = 4: row offsets of the set F
+    float *Lw = reinterpret_cast<float *>(foff + (KW == 4 ? 128 : 0));
     __syncthreads();
 
     bool usable[KW];
@@ -840,6 +836,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             rank[s] = r;
                             if (inS[s]) {
                                 widx[r] = 4 * lane + s;
+                                wrow[r] = (4 * lane + s) * RS;
                                 zbuf[r] = comp ? -u[s] : g[s];
                                 ++r;
                             }
@@ -862,8 +859,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                     if (lane < p4 - p) {
                         widx[p + lane] = 0;
                         zbuf[p + lane] = 0.0f;
-                        if constexpr (KW <= 2)
-                            wrow[p + lane] = 0;
+                        wrow[p + lane] = 0;
                     }
                     __syncwarp();
                     float inv[PT], rp = 0.0f;
@@ -914,7 +910,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                             return DEFERRED;
                     } else {
                         if (p > 32 ? !chol32<PT>(comp ? Ms : Gs, widx, p, Lw, inv, RS, lane)
-                                   : p > 0 && !ldl_cols(comp ? Ms : Gs, widx, p, Lw, rp, RS, lane))
+                                   : p > 0 && !ldl_cols(comp ? Ms : Gs, widx, wrow, p, Lw, rp, lane))
                             return DEFERRED;
                     }
                     // Pass 0 solves the system (zbuf = g_F, or -u_A in the
@@ -949,7 +945,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                         // The step: dx_F from the direct solution, or
                         // base_F + M_FA z_A from the complement one.
                         if (comp)
-                            mv_list<KW>(Ms, widx, zbuf, p4, base, k4, lane);
+                            mv_list<KW>(Ms, wrow, zbuf, p4, base, lane);
 #pragma unroll
                         for (int s = 0; s < KW; ++s) {
                             const float dx = inF[s] ? (comp ? base[s] : zbuf[rank[s]]) : 0.0f;
@@ -965,13 +961,13 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                                 if (inS[s])
                                     zbuf[rank[s]] = x[s];
                             __syncwarp();
-                            mv_list<KW>(Gs, widx, zbuf, p4, w, k4, lane);
+                            mv_list<KW>(Gs, wrow, zbuf, p4, w, lane);
                         } else if constexpr (KW == 4) {
                             if (pass == 0 || p > 32) {
                                 stage_set(x);
                                 mv_set(Gs, foff, stage, n2, w, lane);
                             } else if (p > 0) {   // y is all that is left to form
-                                const float t = mv_rows(Gs, widx, p, x, k4, lane);
+                                const float t = mv_rows(Gs, wrow, p, x, k4, lane);
                                 __syncwarp();
                                 if (lane < p)
                                     zbuf[lane] = t;
