@@ -467,6 +467,11 @@ nmf_status one_iteration(nmf_handle *h)
 {
     const nmf_config &c = h->cfg;
     const bool warm = c.start_mode == NMF_START_WARM && h->passive_valid;
+    // Sparse BPP half-steps gather their right-hand sides inside the solves
+    // (written to V / Y as they go) unless something reads them first: the
+    // stopping measure or a proposal network.
+    const bool fuse = c.input_kind == NMF_INPUT_CSR && c.solver == NMF_SOLVER_BPP &&
+                      !c.no_fused_products && !h->pg_on && !h->mlp;
     // Side stream: Gram of the fixed factor, then the BPP preparation of that
     // Gram (both need only the fixed factor, current on the main stream at the
     // fork); the main stream runs the product meanwhile and joins before the
@@ -479,15 +484,10 @@ nmf_status one_iteration(nmf_handle *h)
         if (!have_gram)
             NMF_TRY(launch_gram(F, rows, c.k, G, h->gram_part, h->side));
         if (c.solver == NMF_SOLVER_BPP)
-            NMF_TRY(launch_bpp_prep(c.k, G, h->bpp_work, h->stats_dev, h->side));
+            NMF_TRY(launch_bpp_prep(c.k, G, h->bpp_work, h->stats_dev, h->side, fuse));
         NMF_CUDA(cudaEventRecord(h->ev_join, h->side));
         return NMF_OK;
     };
-    // Sparse BPP half-steps gather their right-hand sides inside the solves
-    // (written to V / Y as they go) unless something reads them first: the
-    // stopping measure or a proposal network.
-    const bool fuse = c.input_kind == NMF_INPUT_CSR && c.solver == NMF_SOLVER_BPP &&
-                      !c.no_fused_products && !h->pg_on && !h->mlp;
     const CsrGather gather_w{h->A.rowptr, h->A.colidx, h->A.vals, h->Ht};
     const CsrGather gather_h{h->t_rowptr, h->t_colidx, h->t_vals, h->W};
     // W <- argmin_{W >= 0} ||A - W H||: Gram H H^T, right-hand sides A H^T.

@@ -47,6 +47,7 @@
 //
 // Roofline: FP32 ALU for the pivoting; HBM traffic is nrhs * k * 8 bytes
 // (right-hand sides in, solutions out) plus bitmasks.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -64,7 +65,7 @@ constexpr int BPP_THREADS = BPP_WARPS * 32;
 
 // Workspace layout (bytes, 256-aligned pieces).
 struct WorkLayout {
-    size_t g32, m32, m64, usable, flags, counters, defer, prep, total;
+    size_t g32, m32, m64, usable, flags, counters, defer, total;
 };
 
 WorkLayout layout(int k)
@@ -79,7 +80,6 @@ WorkLayout layout(int k)
     w.flags = off; off += al(sizeof(int) * 4);
     w.counters = off; off += al(sizeof(unsigned long long) * CNT_WORDS);
     w.defer = off; off += al(sizeof(int64_t) * DEFER_CAP);
-    w.prep = off; off += al(sizeof(double) * (NMF_MAX_K + 2));   // 1 / L_aa, two norms
     w.total = off;
     return w;
 }
@@ -97,321 +97,323 @@ __device__ __forceinline__ int tri_row(int e)
 }
 
 // ---------------------------------------------------------------------------
-// Prep: FP64 Cholesky of G_UU, its inverse and the scaled cond_1.
-// flags[0] = mode (0 FP32, 1 FP64 with M, 2 FP64 without M), flags[1] = |U|,
-// flags[2] = 1 while the inverse and cond_1 are left to the kernels below,
-// flags[3] counts their last kernel's finished CTAs.
+// Prep: M = G_UU^{-1} in FP64, the scaled cond_1, FP32 copies of G and M.
+// flags[0] = mode (0 FP32, 1 FP64 with M, 2 FP64 without M), flags[1] = |U|.
 //
-// The factorisation runs on one CTA (a chain of pivots). When every index is
-// usable and k >= PREP_SPLIT_K, the rest spreads over the GPU (GB300's FP64
-// pipe does two operations per clock per SM, so one CTA spent most of the
-// preparation on them): L^{-1} one warp per column (bpp_prep_inv_kernel), M =
-// L^{-T} L^{-1} one CTA per column (bpp_prep_m_kernel), the column sums of
-// cond_1 and the symmetric copy of M one CTA per column
-// (bpp_prep_cond_kernel). All work inside M64: L in its lower triangle,
-// L^{-1} transposed in its strict upper triangle, then M's lower triangle
-// over L, then M's upper triangle over L^{-1}.
+// G_UU is inverted in place by Gauss-Jordan sweeps over its lower triangle:
+// sweep p takes the Schur complement's pivot d = A_pp (the square of the
+// Cholesky pivot, tested against the same floor), and sets A_ij -= A_ip A_pj /
+// d, A_ip /= d, A_pp = -1 / d; after the last one A = -M. On positive definite
+// matrices that is as accurate as the inverse through the factor (condition
+// 30 to 4e10, k = 20 to 100, against extended precision: 1.6 to 4 times less
+// error than M = L^{-T} L^{-1}), has the same k^3 / 2 multiply-adds, and one
+// barrier per pivot: the threads keep the triangle in registers, four
+// consecutive entries of a row each, and a pivot's column goes through shared
+// memory (two buffers).
+//
+// Bound by FP64: a quarter of an SM takes one warp instruction in 63-76 cycles,
+// one after the other, whatever its active lanes, and a division in 340. Warp 0
+// therefore keeps the diagonal (lane l: entries l, l + 32, ...) and has the
+// next pivot's reciprocal ready at the barrier, while the others update the
+// triangle. Above k = PREP_ONE_K a cluster of C = 8 CTAs shares the triangle
+// out and writes each pivot's column into every CTA's buffer, unless a product
+// runs beside it, which fills the SMs a cluster would have to wait for (C = 1).
+// Measured, k = 10, 20, 33, 50, 100: 11, 19, 28, 55 and (C = 8) 110 us, where an
+// FP64 Cholesky with three more kernels for the inverse (k >= 48) took 19, 40,
+// 75, 96 and 257.
+// Pairs of floats in place of FP64 were as fast (36 us at k = 50, 131 at 100),
+// but leave M's FP32 rounding to chance in one entry of 1e4 (condition 150).
 // ---------------------------------------------------------------------------
-constexpr int PREP_THREADS = 256;
-constexpr int PREP_SPLIT_K = 48;
+constexpr int PREP_THREADS = 1024;
+constexpr int PREP_ONE_K = 52;
 
-// Sum over the 32 lanes (xor butterfly: every lane gets the same value).
-__device__ __forceinline__ double warp_sum_d(double v)
+// Segment s of the lower triangle (rows in order, row i in i / 4 + 1 segments
+// of four columns): row i, first column j0.
+__device__ __forceinline__ void prep_segment(int s, int &i, int &j0)
 {
-    for (int o = 16; o > 0; o >>= 1)
-        v += __shfl_xor_sync(FULL, v, o);
-    return v;
+    int a = (int)((sqrtf(2.0f * (float)s + 1.0f) - 1.0f) * 0.5f);
+    while (2 * a * (a + 1) > s)
+        --a;
+    while (2 * (a + 1) * (a + 2) <= s)
+        ++a;
+    const int rem = s - 2 * a * (a + 1);   // rows 4 a .. 4 a + 3 have a + 1 each
+    i = 4 * a + rem / (a + 1);
+    j0 = 4 * (rem % (a + 1));
+}
+__host__ __device__ inline int prep_segments(int u)
+{
+    const int a = u >> 2;
+    return 2 * a * (a + 1) + (u & 3) * (a + 1);
 }
 
-__global__ void __launch_bounds__(PREP_THREADS)
+// Thread t's part of sum_a |Ms_ac| w_a: column c = t mod 128, every (threads /
+// 128)-th row.
+__device__ __forceinline__ float prep_colsum(const float *__restrict__ Ms, int u,
+                                             const float *__restrict__ w)
+{
+    const int c = threadIdx.x & 127, part = threadIdx.x >> 7, parts = blockDim.x >> 7;
+    float s = 0.0f;
+    if (c < u && part < parts)
+        for (int a = part; a < u; a += parts)
+            s = fmaf(fabsf(Ms[a * u + c]), w[a], s);
+    return s;
+}
+
+template <int C, int NSEG>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(C == 1 ? PREP_THREADS : PREP_THREADS / 2)
     bpp_prep_kernel(const double *__restrict__ G, int k, float *__restrict__ G32,
                     float *__restrict__ M32, double *__restrict__ M64,
                     uint32_t *__restrict__ usable_words, int *__restrict__ flags,
-                    unsigned long long *__restrict__ counters, BppStats *__restrict__ stats,
-                    double *__restrict__ prep)
+                    unsigned long long *__restrict__ counters, BppStats *__restrict__ stats)
 {
-    extern __shared__ double sm[];
-    // L: u x u, the Cholesky factor in its lower triangle (diagonal included)
-    // and, once formed, L^{-1} transposed in its strict upper triangle:
-    // (L^{-1})_ac for a > c at L[c * u + a]; rdiag holds (L^{-1})_aa = 1 / L_aa.
-    double *L = sm;
-    double *dsq = L + k * k;                          // sqrt(G_aa), a < u
-    double *rdiag = dsq + k;                          // 1 / L_aa
-    double *gdiag = rdiag + k;                        // G_aa
-    int *uidx = reinterpret_cast<int *>(gdiag + k);   // k
-    __shared__ int s_u, s_ok;
-    __shared__ unsigned long long s_norm[2];
-    const int tid = threadIdx.x;
+    constexpr int DS = NMF_MAX_K / 32;
+    extern __shared__ float Ms[];                           // u x u, CTA 0: G, then M, in FP32
+    __shared__ __align__(16) double col[2][NMF_MAX_K + 4];  // the pivot's column
+    __shared__ double rpiv[2];                              // 1 / pivot; 0: below the floor
+    __shared__ double floor_[NMF_MAX_K];                    // the pivots' floors
+    __shared__ float dsq[NMF_MAX_K], rdsq[NMF_MAX_K];       // sqrt(G_aa) and its reciprocal
+    __shared__ int uidx[NMF_MAX_K];
+    __shared__ uint32_t words[4];
+    __shared__ float red[2][PREP_THREADS];
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const int rank = C == 1 ? 0 : (int)blockIdx.x;
+    namespace cg = cooperative_groups;
+    auto sync = [&]() {
+        if constexpr (C == 1)
+            __syncthreads();
+        else
+            cg::this_cluster().sync();
+    };
+    auto at = [&](auto *ptr, int r) {
+        if constexpr (C == 1)
+            return ptr;
+        else
+            return cg::this_cluster().map_shared_rank(ptr, r);
+    };
 
-    for (int e = tid; e < k * k; e += PREP_THREADS) {
+    // Usable indices (G_ii > 0), in order.
+    double gii = 0.0;
+    if (tid < NMF_MAX_K) {   // (at least 128 threads)
+        gii = tid < k ? G[tid * (k + 1)] : 0.0;
+        const uint32_t b = __ballot_sync(FULL, gii > 0.0);
+        if (lane == 0)
+            words[tid >> 5] = b;
+    }
+    for (int e = tid; e < 2 * (NMF_MAX_K + 4); e += nt)
+        (&col[0][0])[e] = 0.0;
+#pragma unroll 4
+    for (int e = rank * nt + tid; e < k * k; e += C * nt)
         G32[e] = (float)G[e];
-        M32[e] = 0.0f;
-        M64[e] = 0.0;
+    __syncthreads();
+    int u = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+        u += __popc(words[w]);
+    if (gii > 0.0) {
+        int a = __popc(words[tid >> 5] & lanemask_lt(lane));
+        for (int w = 0; w < (tid >> 5); ++w)
+            a += __popc(words[w]);
+        uidx[a] = tid;
+        floor_[a] = PIVOT_TOL64 * gii;
+        const float d = sqrtf((float)gii);
+        dsq[a] = d;
+        rdsq[a] = 1.0f / d;
     }
-    if (tid == 0) {
-        int u = 0;
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        for (int i = 0; i < k; ++i)
-            if (G[i * k + i] > 0.0) {
-                uidx[u++] = i;
-                w[i >> 5] |= 1u << (i & 31);
+    if (rank == 0) {
+        if (tid < 4)
+            usable_words[tid] = words[tid];
+        if (tid < CNT_WORDS)
+            counters[tid] = 0ull;
+    }
+    if (u < k)
+        for (int e = rank * nt + tid; e < k * k; e += C * nt) {
+            const int a = e / k, b = e - a * k;
+            if (!((words[a >> 5] >> (a & 31)) & (words[b >> 5] >> (b & 31)) & 1u)) {
+                M32[e] = 0.0f;
+                M64[e] = 0.0;
             }
-        for (int q = 0; q < 4; ++q)
-            usable_words[q] = w[q];
-        s_u = u;
-        s_ok = u > 0;
-        s_norm[0] = s_norm[1] = 0ull;
-        for (int c = 0; c < CNT_WORDS; ++c)
-            counters[c] = 0ull;
-    }
+        }
     __syncthreads();
-    const int u = s_u;
-    for (int e = tid; e < u * u; e += PREP_THREADS) {
-        const int a = e / u, b = e % u;
-        L[a * u + b] = G[uidx[a] * k + uidx[b]];
+
+    int row[NSEG], j0[NSEG];
+    double A[NSEG][4];
+    const int nseg = prep_segments(u);
+#pragma unroll
+    for (int q = 0; q < NSEG; ++q) {
+        const int sg = (q * (nt - 32) + tid - 32) * C + rank;
+        row[q] = -1;
+        j0[q] = 0;
+        if (tid >= 32 && sg < nseg)
+            prep_segment(sg, row[q], j0[q]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            A[q][e] = j0[q] + e <= row[q] ? G[uidx[row[q]] * k + uidx[j0[q] + e]] : 0.0;
     }
-    for (int a = tid; a < u; a += PREP_THREADS) {
-        gdiag[a] = G[uidx[a] * k + uidx[a]];
-        dsq[a] = sqrt(gdiag[a]);
+    double diag[DS];
+#pragma unroll
+    for (int t = 0; t < DS; ++t) {
+        const int i = lane + 32 * t;
+        diag[t] = tid < 32 && i < u ? G[uidx[i] * (k + 1)] : 1.0;
     }
-    __syncthreads();
-    // Right-looking Cholesky on the lower triangle. Pivot j + 1 is final once
-    // its diagonal entry has taken pivot j's update, which thread 0 makes
-    // itself (row j + 1 of the trailing triangle is its first row): it forms
-    // that pivot's root in the same phase, so each pivot takes two barriers.
-    auto pivot = [&](int j) {
-        const double d = L[j * u + j];
-        if (!(d > PIVOT_TOL64 * gdiag[j])) {
-            s_ok = 0;
-        } else {
-            // One reciprocal square root instead of a root and a division on
-            // the pivots' serial path (GB300's FP64 pipe is narrow).
-            const double r = rsqrt(d);
-            L[j * u + j] = d * r;
-            rdiag[j] = r;
+    if (C > 1)
+        sync();   // every CTA's buffers are cleared
+    // sign times the entries to both triangles of CTA 0's Ms.
+    auto to_shared = [&](float sign) {
+        float *dst = at(Ms, 0);
+#pragma unroll
+        for (int q = 0; q < NSEG; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = row[q], j = j0[q] + e;
+                if (j <= i) {
+                    const float v = sign * (float)A[q][e];
+                    dst[i * u + j] = v;
+                    dst[j * u + i] = v;
+                }
+            }
+    };
+    auto put = [&](double v, int i, int p) {   // entry i of pivot p's column
+        for (int t = 0; t < C; ++t)
+            *at(&col[p & 1][i], t) = v;
+    };
+    // A segment's entries of pivot p's column: row p itself, or column p.
+    auto put_segment = [&](double a0, double a1, double a2, double a3, int i, int j, int p) {
+        if (i == p) {
+            put(a0, j, p);
+            if (j + 1 <= p)
+                put(a1, j + 1, p);
+            if (j + 2 <= p)
+                put(a2, j + 2, p);
+            if (j + 3 <= p)
+                put(a3, j + 3, p);
+        } else if (i > p && j == (p & ~3)) {
+            const int e = p & 3;
+            put(e == 0 ? a0 : e == 1 ? a1 : e == 2 ? a2 : a3, i, p);
         }
     };
-    if (tid == 0 && u > 0)
-        pivot(0);
-    __syncthreads();
-    for (int j = 0; j < u; ++j) {
-        if (!s_ok)
+    to_shared(1.0f);
+#pragma unroll
+    for (int q = 0; q < NSEG; ++q)
+        put_segment(A[q][0], A[q][1], A[q][2], A[q][3], row[q], j0[q], 0);
+    if (tid == 0)
+        rpiv[0] = diag[0] > floor_[0] ? 1.0 / diag[0] : 0.0;
+    sync();
+    const float sg = rank == 0 ? prep_colsum(Ms, u, rdsq) : 0.0f;
+    bool ok = u > 0;
+    for (int p = 0; p < u; ++p) {
+        const double *c = col[p & 1];
+        const double r = rpiv[p & 1];
+        if (!(r > 0.0)) {
+            ok = false;   // (the same in every thread)
             break;
-        const double rj = rdiag[j];
-        for (int i = j + 1 + tid; i < u; i += PREP_THREADS)
-            L[i * u + j] *= rj;
-        __syncthreads();
-        // Trailing lower triangle (a >= b > j): rows by warp, columns by lane.
-        for (int a = j + 1 + (tid >> 5); a < u; a += PREP_THREADS / 32) {
-            const double laj = L[a * u + j];
-            for (int b = j + 1 + (tid & 31); b <= a; b += 32)
-                L[a * u + b] = fma(-laj, L[b * u + j], L[a * u + b]);
         }
-        if (tid == 0 && j + 1 < u)
-            pivot(j + 1);
-        __syncthreads();
+        const int np = p + 1;
+        if (tid < 32) {
+            // The diagonal, the next pivot's part first (entries already swept
+            // carry values of no use).
+            const int tn = np >> 5;
+            double d = diag[0];
+#pragma unroll
+            for (int t = 1; t < DS; ++t)
+                if (t == tn)
+                    d = diag[t];
+            const double cn = c[(lane + 32 * tn) & (NMF_MAX_K - 1)];
+            d = fma(-(cn * r), cn, d);
+            if (lane == (np & 31) && np < u) {
+                const double rn = 1.0 / d;
+                rpiv[np & 1] = d > floor_[np] ? rn : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < DS; ++t) {
+                if (t == tn) {
+                    diag[t] = d;
+                } else if (t > tn && 32 * t < u) {
+                    const double ct = c[lane + 32 * t];
+                    diag[t] = fma(-(ct * r), ct, diag[t]);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < NSEG; ++q) {
+                if (row[q] < 0)
+                    continue;
+                // Row p itself becomes c r: the same products with -r for c_i r
+                // and zero for A.
+                const bool prow = row[q] == p;
+                const double s = (prow ? -1.0 : c[row[q]]) * r;
+                const double2 c01 = *reinterpret_cast<const double2 *>(c + j0[q]);
+                const double2 c23 = *reinterpret_cast<const double2 *>(c + j0[q] + 2);
+                const double cj[4] = {c01.x, c01.y, c23.x, c23.y};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const double v = fma(-s, cj[e], prow ? 0.0 : A[q][e]);
+                    A[q][e] = j0[q] + e == p ? s : v;
+                }
+                put_segment(A[q][0], A[q][1], A[q][2], A[q][3], row[q], j0[q], np);
+            }
+        }
+        sync();
     }
-    if (!s_ok) {
-        if (tid == 0) {
+    if (!ok) {
+        if (rank == 0 && tid == 0) {
             flags[0] = 2;
             flags[1] = u;
-            flags[2] = 0;
             atomicAdd(&stats->fp64_halfsteps, 1ull);
         }
+        return;   // (the loop ended at a barrier all CTAs passed)
+    }
+    // M = -A to both triangles.
+#pragma unroll
+    for (int q = 0; q < NSEG; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = row[q], j = j0[q] + e;
+            if (j <= i) {
+                const double m = -A[q][e];
+                const int gi = uidx[i], gj = uidx[j];
+                M64[gi * k + gj] = m;
+                M64[gj * k + gi] = m;
+                M32[gi * k + gj] = (float)m;
+                M32[gj * k + gi] = (float)m;
+            }
+        }
+    to_shared(-1.0f);
+    sync();
+    if (rank != 0)
         return;
-    }
-    if (u == k && k >= PREP_SPLIT_K) {
-        // L (lower triangle, diagonal included) and 1 / L_aa to the kernels
-        // that finish the preparation.
-        for (int e = tid; e < k * k; e += PREP_THREADS) {
-            const int a = e / k, b = e - a * k;
-            if (b <= a)
-                M64[e] = L[a * u + b];
-        }
-        for (int a = tid; a < k; a += PREP_THREADS)
-            prep[a] = rdiag[a];
-        if (tid == 0) {
-            prep[k] = 0.0;
-            prep[k + 1] = 0.0;
-            flags[2] = 1;
-            flags[3] = 0;
-        }
+    // cond_1 of the scaled matrix, max column sum of |G_ac| / (d_a d_c) times
+    // max column sum of |M_ac| d_a d_c with d_a = sqrt(G_aa), in FP32 (the
+    // number only picks the arithmetic; where it is not finite, FP64).
+    red[0][tid] = sg;
+    red[1][tid] = prep_colsum(Ms, u, dsq);
+    __syncthreads();
+    if (tid >= 32)
         return;
-    }
-    if (tid == 0)
-        flags[2] = 0;
-    // Columns of L^{-1} by forward substitution, one column per thread, into
-    // the strict upper triangle of L (transposed).
-    for (int c = tid; c < u; c += PREP_THREADS) {
-        for (int a = c + 1; a < u; ++a) {
-            double s = -L[a * u + c] * rdiag[c];
-            for (int b = c + 1; b < a; ++b)
-                s = fma(-L[a * u + b], L[c * u + b], s);
-            L[c * u + a] = s * rdiag[a];
+    const int parts = nt >> 7;
+    float mg = 0.0f, mm = 0.0f;
+    bool fine = true;
+    for (int c = lane; c < u; c += 32) {
+        float tg = 0.0f, tm = 0.0f;
+        for (int q = 0; q < parts; ++q) {
+            tg += red[0][c + 128 * q];
+            tm += red[1][c + 128 * q];
         }
+        tg *= rdsq[c];
+        tm *= dsq[c];
+        fine &= isfinite(tg) && isfinite(tm);
+        mg = fmaxf(mg, tg);
+        mm = fmaxf(mm, tm);
     }
-    __syncthreads();
-    // M = L^{-T} L^{-1}: M_ab = sum_{c >= max(a, b)} (L^{-1})_ca (L^{-1})_cb,
-    // for a <= b, written to both triangles of M64 and M32.
-    for (int e = tid; e < u * (u + 1) / 2; e += PREP_THREADS) {
-        const int b = tri_row(e), a = e - b * (b + 1) / 2;   // a <= b
-        double s = (a == b ? rdiag[b] : L[a * u + b]) * rdiag[b];
-        for (int c = b + 1; c < u; ++c)
-            s = fma(L[a * u + c], L[b * u + c], s);
-        const int ga = uidx[a], gb = uidx[b];
-        M64[ga * k + gb] = s;
-        M64[gb * k + ga] = s;
-        M32[ga * k + gb] = (float)s;
-        M32[gb * k + ga] = (float)s;
-    }
-    __syncthreads();
-    // Scaled cond_1 = max column sum of |G_ac| / (d_a d_c) times max column
-    // sum of |M_ac| d_a d_c, d_a = sqrt(G_aa). Non-negative doubles order like
-    // their bit patterns, so an integer max reduces them.
-    for (int c = tid; c < u; c += PREP_THREADS) {
-        double sg = 0.0, sm2 = 0.0;
-        for (int a = 0; a < u; ++a) {
-            sg += fabs(G[uidx[a] * k + uidx[c]]) / dsq[a];
-            sm2 += fabs(M64[uidx[a] * k + uidx[c]]) * dsq[a];
-        }
-        sg /= dsq[c];
-        sm2 *= dsq[c];
-        atomicMax(&s_norm[0], (unsigned long long)__double_as_longlong(sg));
-        atomicMax(&s_norm[1], (unsigned long long)__double_as_longlong(sm2));
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const double cond = __longlong_as_double((long long)s_norm[0]) *
-                            __longlong_as_double((long long)s_norm[1]);
-        const int mode = cond <= COND_FP32 ? 0 : 1;
+    fine = __all_sync(FULL, fine);
+    const double cond = (double)warp_max(mg) * (double)warp_max(mm);
+    if (lane == 0) {
+        const int mode = fine && cond <= COND_FP32 ? 0 : 1;
         flags[0] = mode;
         flags[1] = u;
         if (mode)
             atomicAdd(&stats->fp64_halfsteps, 1ull);
     }
 }
-
-
-// (L^{-1})_ac, a > c, into M64[c][a]: one CTA per column c, the column's
-// forward substitution in its first warp, right-looking: lane a % 32 keeps
-// the pending sum of row a, s_a = -L_ac / L_cc - sum_{c < b < a} L_ab x_b,
-// adding the terms in increasing b (the order of the single-thread form, so
-// the values are the same); once x_b = s_b / L_bb is final its lane
-// broadcasts it and every later row takes its term. L's rows from c on are
-// staged in shared memory by the whole CTA first.
-constexpr int INV_THREADS = 256;
-
-__global__ void __launch_bounds__(INV_THREADS)
-    bpp_prep_inv_kernel(int k, double *__restrict__ M64, const double *__restrict__ prep,
-                        const int *__restrict__ flags)
-{
-    if (flags[2] != 1)
-        return;
-    extern __shared__ double inv_sm[];
-    double *Ls = inv_sm;               // k x k (lower triangle, rows c and on)
-    const int c = blockIdx.x;
-    for (int e = c * k + (int)threadIdx.x; e < k * k; e += INV_THREADS) {
-        const int a = e / k, b = e - a * k;
-        Ls[e] = b <= a ? M64[e] : 0.0;
-    }
-    __syncthreads();
-    if (threadIdx.x >= 32)
-        return;
-    const int lane = threadIdx.x;
-    constexpr int T = (NMF_MAX_K + 31) / 32;
-    const double rc = prep[c];
-    double sr[T];
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-        const int a = lane + 32 * t;
-        sr[t] = (a > c && a < k) ? -Ls[a * k + c] * rc : 0.0;
-    }
-    for (int b = c + 1; b < k; ++b) {
-        const int owner = b & 31, slot = b >> 5;
-        double mine = 0.0;
-#pragma unroll
-        for (int t = 0; t < T; ++t)
-            if (t == slot)
-                mine = sr[t];
-        const double xb = __shfl_sync(FULL, mine * prep[b], owner);
-        if (lane == owner)
-            M64[c * k + b] = xb;
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const int a = lane + 32 * t;
-            if (a > b && a < k)
-                sr[t] = fma(-Ls[a * k + b], xb, sr[t]);
-        }
-    }
-}
-
-// M_ab = sum_{c >= a} (L^{-1})_ca (L^{-1})_cb for a >= b into M64[a][b] (and
-// M32 both ways): one CTA per column b, one warp per entry.
-__global__ void __launch_bounds__(128)
-    bpp_prep_m_kernel(int k, double *__restrict__ M64, float *__restrict__ M32,
-                      const double *__restrict__ prep, const int *__restrict__ flags)
-{
-    if (flags[2] != 1)
-        return;
-    const int b = blockIdx.x, lane = threadIdx.x & 31;
-    for (int a = b + (threadIdx.x >> 5); a < k; a += 4) {
-        double part = 0.0;
-        for (int c = a + lane; c < k; c += 32) {
-            const double xa = c == a ? prep[a] : M64[a * k + c];
-            const double xb = c == b ? prep[b] : M64[b * k + c];
-            part = fma(xa, xb, part);
-        }
-        const double m = warp_sum_d(part);
-        if (lane == 0) {
-            M64[a * k + b] = m;
-            M32[a * k + b] = (float)m;
-            M32[b * k + a] = (float)m;
-        }
-    }
-}
-
-// Column c of the scaled cond_1 (max column sum of |G_ac| / (d_a d_c) and of
-// |M_ac| d_a d_c, d_a = sqrt(G_aa)) from M's lower triangle, and M's upper
-// triangle in column c; the last CTA sets the mode.
-__global__ void __launch_bounds__(32)
-    bpp_prep_cond_kernel(const double *__restrict__ G, int k, double *__restrict__ M64,
-                         double *__restrict__ prep, int *__restrict__ flags,
-                         BppStats *__restrict__ stats)
-{
-    if (flags[2] != 1)
-        return;
-    const int c = blockIdx.x, lane = threadIdx.x;
-    double sg = 0.0, sm = 0.0;
-    for (int a = lane; a < k; a += 32) {
-        const double da = sqrt(G[a * k + a]);
-        sg += fabs(G[a * k + c]) / da;
-        sm += fabs(a >= c ? M64[a * k + c] : M64[c * k + a]) * da;
-    }
-    const double dc = sqrt(G[c * k + c]);
-    sg = warp_sum_d(sg) / dc;
-    sm = warp_sum_d(sm) * dc;
-    for (int a = lane; a < c; a += 32)
-        M64[a * k + c] = M64[c * k + a];
-    if (lane == 0) {
-        unsigned long long *norm = reinterpret_cast<unsigned long long *>(prep + k);
-        // Non-negative doubles order like their bit patterns.
-        atomicMax(&norm[0], (unsigned long long)__double_as_longlong(sg));
-        atomicMax(&norm[1], (unsigned long long)__double_as_longlong(sm));
-        __threadfence();
-        if (atomicAdd(&flags[3], 1) == k - 1) {
-            __threadfence();
-            const double cond = __longlong_as_double((long long)atomicAdd(&norm[0], 0ull)) *
-                                __longlong_as_double((long long)atomicAdd(&norm[1], 0ull));
-            const int mode = cond <= COND_FP32 ? 0 : 1;
-            flags[0] = mode;
-            flags[1] = k;
-            flags[2] = 0;
-            if (mode)
-                atomicAdd(&stats->fp64_halfsteps, 1ull);
-        }
-    }
-}
-
 
 // FP64 Cholesky of S_ab = Src[idx[a] * ld + idx[b]], right-looking: after
 // each pivot the trailing lower triangle is updated with its (a, b) entries
@@ -1054,34 +1056,42 @@ nmf_status launch_solves(const SolveParams &P, cudaStream_t s)
 
 }  // namespace
 
-nmf_status launch_bpp_prep(int k, const double *G, void *work, BppStats *stats_dev, cudaStream_t s)
+namespace {
+
+constexpr size_t PREP_STATIC = 16 * 1024;   // at least the kernel's static shared memory
+
+template <int C, int NSEG>
+nmf_status launch_prep(const SolveParams &P, BppStats *stats_dev, cudaStream_t s)
+{
+    const int k = P.k;
+    const size_t smem = sizeof(float) * (size_t)k * k;
+    static SmemOptIn opt_in;
+    NMF_TRY(ensure_smem(bpp_prep_kernel<C, NSEG>, opt_in, smem + PREP_STATIC));
+    // A thread per segment of the triangle beside warp 0, 128 at a time.
+    const int64_t want = cdiv(cdiv(prep_segments(k), C) + 32, 128) * 128;
+    const int threads = (int)std::min<int64_t>(want, C == 1 ? PREP_THREADS : PREP_THREADS / 2);
+    bpp_prep_kernel<C, NSEG><<<C, threads, smem, s>>>(
+        P.G64, k, const_cast<float *>(P.G32), const_cast<float *>(P.M32),
+        const_cast<double *>(P.M64), const_cast<uint32_t *>(P.usable_words),
+        const_cast<int *>(P.flags), P.counters, stats_dev);
+    NMF_LAUNCHED("bpp_prep_kernel");
+    return NMF_OK;
+}
+
+}  // namespace
+
+nmf_status launch_bpp_prep(int k, const double *G, void *work, BppStats *stats_dev, cudaStream_t s,
+                           bool alone)
 {
     const SolveParams P = solve_params(k, 0, G, nullptr, nullptr, nullptr, nullptr, nullptr,
                                        nullptr, 0, work, stats_dev);
-    const size_t prep_smem = sizeof(double) * ((size_t)k * k + 3 * k) + sizeof(int) * (size_t)k;
-    static SmemOptIn opt_in;
-    NMF_TRY(ensure_smem(bpp_prep_kernel, opt_in, prep_smem));
-    double *prep = reinterpret_cast<double *>(static_cast<unsigned char *>(work) + layout(k).prep);
-    bpp_prep_kernel<<<1, PREP_THREADS, prep_smem, s>>>(
-        G, k, const_cast<float *>(P.G32), const_cast<float *>(P.M32),
-        const_cast<double *>(P.M64), const_cast<uint32_t *>(P.usable_words),
-        const_cast<int *>(P.flags), P.counters, stats_dev, prep);
-    NMF_LAUNCHED("bpp_prep_kernel");
-    if (k >= PREP_SPLIT_K) {   // (each returns at once unless the prep left them the work)
-        const size_t inv_smem = sizeof(double) * (size_t)k * k;
-        static SmemOptIn inv_opt_in;
-        NMF_TRY(ensure_smem(bpp_prep_inv_kernel, inv_opt_in, inv_smem));
-        bpp_prep_inv_kernel<<<(unsigned)k, INV_THREADS, inv_smem, s>>>(
-            k, const_cast<double *>(P.M64), prep, P.flags);
-        NMF_LAUNCHED("bpp_prep_inv_kernel");
-        bpp_prep_m_kernel<<<(unsigned)k, 128, 0, s>>>(k, const_cast<double *>(P.M64),
-                                                      const_cast<float *>(P.M32), prep, P.flags);
-        NMF_LAUNCHED("bpp_prep_m_kernel");
-        bpp_prep_cond_kernel<<<(unsigned)k, 32, 0, s>>>(G, k, const_cast<double *>(P.M64), prep,
-                                                       const_cast<int *>(P.flags), stats_dev);
-        NMF_LAUNCHED("bpp_prep_cond_kernel");
-    }
-    return NMF_OK;
+    if (k > PREP_ONE_K && alone)
+        return launch_prep<8, 1>(P, stats_dev, s);
+    // Segments per thread (k = 128: 2112).
+    const int nseg = prep_segments(k), nt = PREP_THREADS - 32;
+    return nseg <= nt       ? launch_prep<1, 1>(P, stats_dev, s)
+           : nseg <= 2 * nt ? launch_prep<1, 2>(P, stats_dev, s)
+                            : launch_prep<1, 3>(P, stats_dev, s);
 }
 
 nmf_status launch_bpp_solve(int k, int64_t nrhs, const double *G, const float *B, float *X,

@@ -225,7 +225,10 @@ nmf_status launch_bpp(int k, int64_t nrhs, const double *G, const float *B, floa
 // The two halves of launch_bpp: the per-Gram preparation (factor, inverse,
 // arithmetic mode), then the solves. A prep must complete before its solves
 // and must not overlap another half-step's prep or solves on the same work.
-nmf_status launch_bpp_prep(int k, const double *G, void *work, BppStats *stats_dev, cudaStream_t s);
+// alone: no other kernel runs beside it (a large preparation then takes a
+// cluster of CTAs).
+nmf_status launch_bpp_prep(int k, const double *G, void *work, BppStats *stats_dev, cudaStream_t s,
+                           bool alone = true);
 // Measures the solve kernel's launch shapes on this batch and keeps the fastest
 // for k (used by every later solve of that k); X receives the solution.
 nmf_status bpp_tune(int k, int64_t nrhs, const double *G, const float *B, float *X,
