@@ -100,9 +100,13 @@ extern "C" nmf_status nmf_mm_dense(const float *A, int64_t m, int64_t n, int64_t
         return launch_mm_tc(A, m, n, lda, F, k, trans, out, w.p, wb, s);
     }
     if (mm_f32_supported(A, lda)) {
-        const size_t wb = mm_f32_work_bytes(m, n, k, trans);
+        size_t wb = mm_f32_work_bytes(m, n, k, trans);
         TempBuf w(s);
-        NMF_CUDA(w.alloc(wb));
+        if (w.alloc(wb) != cudaSuccess) {   // not the memory for a shared last wave
+            cudaGetLastError();
+            wb = mm_f32_work_bytes(m, n, k, trans, false);
+            NMF_CUDA(w.alloc(wb));
+        }
         return launch_mm_f32(A, m, n, lda, F, k, trans, out, nullptr, nullptr, w.p, wb, s);
     }
     return launch_mm_simt(A, m, n, lda, F, k, trans, out, s);
@@ -676,9 +680,15 @@ extern "C" nmf_status nmf_init(nmf_handle **out, const nmf_config *cfg, const nm
     h->fused_obj = c.input_kind == NMF_INPUT_DENSE && c.k <= 64 &&
                    (c.precision == NMF_PREC_BF16X3 || h->f32);
     if (e == cudaSuccess && h->f32) {
-        h->tc_work_bytes = std::max(mm_f32_work_bytes(c.m, c.n, c.k, 0),
-                                    mm_f32_work_bytes(c.m, c.n, c.k, 1));
-        chk(cudaMalloc(&h->tc_work, h->tc_work_bytes));
+        for (const bool share : {true, false}) {   // (see mm_f32_work_bytes)
+            h->tc_work_bytes = std::max(mm_f32_work_bytes(c.m, c.n, c.k, 0, share),
+                                        mm_f32_work_bytes(c.m, c.n, c.k, 1));
+            if (!h->tc_work && cudaMalloc(&h->tc_work, h->tc_work_bytes) == cudaSuccess)
+                break;
+            cudaGetLastError();
+        }
+        if (!h->tc_work)
+            e = cudaErrorMemoryAllocation;
     }
     if (e == cudaSuccess && c.input_kind == NMF_INPUT_DENSE && c.precision == NMF_PREC_BF16X3) {
         h->tc_work_bytes = mm_tc_work_bytes(c.m, c.n, c.k, 0);

@@ -133,9 +133,11 @@ nmf_status launch_mm_simt(const float *A, int64_t m, int64_t n, int64_t lda, con
 // Dense products in plain FP32 with packed FP32x2 FMAs (mm_f32.cu): A 16-byte
 // aligned with lda a multiple of 4 (mm_f32_supported). trans = 0 with W and
 // f_dev non-null (k <= 64) also writes f(W, H) = ||A - W H||^2 to *f_dev.
-// `work` holds mm_f32_work_bytes(m, n, k, trans) bytes.
+// `work` holds mm_f32_work_bytes(m, n, k, trans) bytes, or, without the memory
+// for sharing out the last wave of A H^T, the fewer bytes of share = false
+// (same results).
 bool mm_f32_supported(const float *A, int64_t lda);
-size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans);
+size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans, bool share = true);
 nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, const float *F, int k,
                          int trans, float *out, const float *W, double *f_dev, void *work,
                          size_t work_bytes, cudaStream_t s);
@@ -147,8 +149,8 @@ nmf_status launch_mm_tc(const float *A, int64_t m, int64_t n, int64_t lda, const
                         int k, int trans, float *out, void *work, size_t work_bytes,
                         cudaStream_t s);
 size_t mm_tc_work_bytes(int64_t m, int64_t n, int k, int trans);
-// Contraction splits (CTAs along the contraction per output tile) the
-// tensor-core product of this shape uses, with or without the objective.
+// Contraction splits (CTAs along the contraction per output tile) the plain
+// tensor-core product of this shape uses.
 int mm_tc_splits(int64_t m, int64_t n, int trans);
 // Same, and with W, Ht, f_dev non-null (trans = 0, k <= 64) the objective
 // f(W, H) = ||A - W H||^2 fused into the pass, written to *f_dev.

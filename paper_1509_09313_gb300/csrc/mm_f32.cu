@@ -102,13 +102,21 @@ __device__ __forceinline__ void cp_async_wait()
 
 __device__ __forceinline__ int clamp16(int64_t v) { return v <= 0 ? 0 : v >= 16 ? 16 : (int)v; }
 
+// A H^T: tiles 0 .. full - 1 take one CTA each, the `tiles` after them `splits`
+// CTAs each, whose stage sums go to `part`.
+struct F32Tail {
+    int64_t full = 0, tiles = 0;
+    int splits = 1;
+    float *part = nullptr;
+};
+
 template <int TRANS, bool OBJ, int NCG, int RPT>
 __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t P, int64_t Q,
                                             int64_t lda, const float *__restrict__ Fc,
                                             int64_t ldf, int k, int64_t q_per_split,
                                             float *__restrict__ out,
                                             const float *__restrict__ W,
-                                            double *__restrict__ obj_part)
+                                            double *__restrict__ obj_part, const F32Tail tail)
 {
     using T = F32Tile<TRANS, NCG, RPT>;
     constexpr int NT = T::THREADS, BP = T::BP, KP = T::KP, BQ = T::BQ, NS = T::STAGES;
@@ -116,11 +124,28 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
     float *Wt = f32_smem + NS * T::STAGE;
     const int tid = threadIdx.x;
     const int pg = tid / NCG, cg = tid % NCG;
-    const int64_t p0 = (int64_t)blockIdx.x * BP;
-    const int c0 = blockIdx.y * KP;            // this CTA's column chunk
-    // Contraction range of this CTA (a split of it when gridDim.z > 1).
-    const int64_t qb = (int64_t)blockIdx.z * q_per_split;
-    const int64_t qe = min(Q, qb + q_per_split);
+    // Tile (rows and column chunk) and contraction range of this CTA. A^T W: a
+    // grid of tiles, chunks and contraction splits. A H^T: the tiles of whole
+    // waves first, then those left over, each shared by tail.splits CTAs.
+    int64_t tile = blockIdx.x;
+    int chunk = blockIdx.y;
+    int64_t qb = (int64_t)blockIdx.z * q_per_split, qe = min(Q, qb + q_per_split);
+    const bool shared_tile = TRANS == 0 && tile >= tail.full;
+    if (TRANS == 0) {
+        qb = 0;
+        qe = Q;
+        if (shared_tile) {
+            const int64_t e = tile - tail.full;
+            tile = tail.full + e / tail.splits;
+            qb = e % tail.splits * q_per_split;
+            qe = min(Q, qb + q_per_split);
+        }
+        const int64_t ptiles = (P + BP - 1) / BP;
+        chunk = (int)(tile / ptiles);
+        tile -= chunk * ptiles;
+    }
+    const int64_t p0 = tile * BP;
+    const int c0 = chunk * KP;
     const int64_t nst = qe > qb ? cdiv(qe - qb, BQ) : 0;
 
     auto load_stage = [&](int64_t st, int buf) {
@@ -320,6 +345,18 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
                 }
             continue;
         }
+        if (shared_tile) {
+            // The stage's sums for f32_stage_kernel, [stage][tile][entry].
+            float *dst = tail.part +
+                         ((qb / BQ + t) * tail.tiles +
+                          ((int64_t)blockIdx.x - tail.full) / tail.splits) * (BP * KP) + tid;
+#pragma unroll
+            for (int a = 0; a < RPT; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    dst[(a * 4 + b) * NT] = part[a][b];
+            continue;
+        }
         // Kahan: acc + cmp carries the running total to ~FP32 rounding.
 #pragma unroll
         for (int a = 0; a < RPT; ++a)
@@ -351,12 +388,12 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
 
     // Output: the compensated total rounded once, or (contraction split)
     // this split's total and compensation, for the sum over splits.
-    const bool split = gridDim.z > 1;
+    const bool split = TRANS == 1 && gridDim.z > 1;
     float *dst = out + (int64_t)blockIdx.z * 2 * P * k;
 #pragma unroll
     for (int a = 0; a < RPT; ++a) {
         const int64_t p = p0 + (TRANS == 0 ? pg + 16 * a : RPT * pg + a);
-        if (p < P) {
+        if (p < P && !shared_tile) {
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 const int c = c0 + (TRANS == 0 ? cg + NCG * b : 4 * cg + b);
@@ -385,7 +422,7 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
             double s = 0.0;
             for (int w = 0; w < NT / 32; ++w)
                 s += red[w];
-            obj_part[blockIdx.z * gridDim.x + blockIdx.x] = s;
+            obj_part[blockIdx.x] = s;
         }
     }
 }
@@ -398,9 +435,39 @@ __global__ void __launch_bounds__(16 * NCG, 1)
     mm_f32_kernel(const float *__restrict__ A, int64_t P, int64_t Q, int64_t lda,
                   const float *__restrict__ Fc, int64_t ldf, int k, int64_t q_per_split,
                   float *__restrict__ out, const float *__restrict__ W,
-                  double *__restrict__ obj_part)
+                  double *__restrict__ obj_part, const F32Tail tail)
 {
-    mm_f32_body<0, OBJ, NCG, RPT>(A, P, Q, lda, Fc, ldf, k, q_per_split, out, W, obj_part);
+    mm_f32_body<0, OBJ, NCG, RPT>(A, P, Q, lda, Fc, ldf, k, q_per_split, out, W, obj_part, tail);
+}
+
+// The shared tiles of A H^T: out from the stages' sums, added with the Kahan
+// steps of an unshared tile in its order (bitwise its result). Entry (a, b) of
+// thread tid of the product's CTA at (4 a + b) NT + tid. Reads 4 bytes per
+// entry and stage.
+template <int NCG, int RPT>
+__global__ void __launch_bounds__(256)
+    f32_stage_kernel(int64_t P, int64_t nst, int k, float *__restrict__ out, const F32Tail tail)
+{
+    using T = F32Tile<0, NCG, RPT>;
+    constexpr int E = T::BP * T::KP;
+    const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t stride = tail.tiles * E;
+    if (e >= stride)
+        return;
+    float acc = 0.0f, cmp = 0.0f;
+#pragma unroll 16
+    for (int64_t t = 0; t < nst; ++t) {
+        const float yk = tail.part[t * stride + e] - cmp;
+        const float tk = acc + yk;
+        cmp = (tk - acc) - yk;
+        acc = tk;
+    }
+    const int64_t tile = tail.full + e / E, ptiles = (P + T::BP - 1) / T::BP;
+    const int li = (int)(e % E), tid = li % T::THREADS, ab = li / T::THREADS;
+    const int64_t p = tile % ptiles * T::BP + tid / NCG + 16 * (ab >> 2);
+    const int c = (int)(tile / ptiles) * T::KP + tid % NCG + NCG * (ab & 3);
+    if (p < P && c < k)
+        out[p * k + c] = acc + -cmp;
 }
 
 template <int NCG, int RPT>
@@ -409,8 +476,8 @@ __global__ void __maxnreg__(128)
                     const float *__restrict__ Fc, int64_t ldf, int k, int64_t q_per_split,
                     float *__restrict__ out)
 {
-    mm_f32_body<1, false, NCG, RPT>(A, P, Q, lda, Fc, ldf, k, q_per_split, out, nullptr,
-                                    nullptr);
+    mm_f32_body<1, false, NCG, RPT>(A, P, Q, lda, Fc, ldf, k, q_per_split, out, nullptr, nullptr,
+                                    F32Tail{});
 }
 
 // out[p][c] = the sum over splits s of total[s][p][c] + compensation[s][p][c]
@@ -464,13 +531,17 @@ __global__ void f32_pad_kernel(const float *__restrict__ F, int64_t Q, int k, in
 int f32_ncg(int k) { return k <= 16 ? 4 : k <= 32 ? 8 : k <= 48 ? 12 : k <= 56 ? 14 : 16; }
 constexpr int RPT0 = 8, RPT1 = 8;   // rows per thread: A H^T, A^T W
 
+constexpr size_t F32_TAIL_BYTES = (size_t)512 << 20;   // most scratch for shared tiles
+
 struct F32Plan {
     int ncg, kp, nch, kpt, splits;
-    int64_t P, Q, ldf, bp, q_per_split;
+    int64_t P, Q, ldf, bp, bq, q_per_split;
+    F32Tail tail;
     size_t f_off, part_off, split_off, total;
 };
 
-F32Plan f32_plan(int64_t m, int64_t n, int k, int trans)
+// share: A H^T may share out the tiles of its last wave (needs scratch).
+F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool share = true)
 {
     F32Plan w;
     w.P = trans ? n : m;
@@ -481,18 +552,17 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans)
     w.kpt = w.kp * w.nch;
     w.bp = 16 * (trans ? RPT1 : RPT0);
     w.ldf = trans ? w.kpt : cdiv(w.Q > 0 ? w.Q : 1, 4) * 4;
-    // The contraction is split (up to 16 ways, each split keeping at least 8
-    // stages) so that the CTAs fill whole waves of the resident ones (A^T W two
-    // per SM, A H^T one): the fewest splits within 2% of the best wave
-    // efficiency. A H^T splits alike with and without the fused objective, so
-    // that its products are the same in both. (Unsplit, 24000 x 16000, k = 50
-    // ran 188 CTAs in two waves, 1.95 ms; 2000 x 1000, k = 10 ran 16 CTAs, 59
-    // us, and 101 us with the objective.)
+    const int64_t Q = w.Q > 0 ? w.Q : 1;
     const int64_t tiles = cdiv(w.P > 0 ? w.P : 1, w.bp) * w.nch;
     const int64_t bq = trans ? F32_BQ1 : 4 * w.ncg;
+    w.bq = bq;
     w.splits = 1;
-    {
-        const int64_t slots = (trans ? 2 : 1) * (int64_t)sm_count();
+    w.q_per_split = cdiv(Q, bq) * bq;
+    if (trans) {
+        // A^T W splits its contraction (up to 16 ways, each split keeping at
+        // least 8 stages) so that its CTAs fill whole waves of two per SM: the
+        // fewest splits within 2% of the best wave efficiency.
+        const int64_t slots = 2 * (int64_t)sm_count();
         auto eff = [&](int64_t sp) {
             const int64_t ctas = tiles * sp;
             return (double)ctas / (double)(cdiv(ctas, slots) * slots);
@@ -507,17 +577,38 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans)
                 w.splits = (int)sp;
                 break;
             }
+        w.q_per_split = cdiv(cdiv(Q, w.splits), bq) * bq;
+    } else {
+        // A H^T (one CTA per SM) shares out the contraction of the tiles its
+        // whole waves leave over, at least 8 stages to a CTA, and adds the
+        // stages' sums in the order of an unshared tile, so that the products
+        // do not depend on the grid (nor on the fused objective): an ANLS run's
+        // iterates follow every last bit of them. Unshared, 24000 x 16000, k =
+        // 50 ran 188 CTAs in two waves, 1.95 ms; 2000 x 1000, k = 10 ran 16,
+        // 59 us, and 101 us with the objective.
+        w.tail.full = tiles;
+        const int64_t sms = sm_count(), left = tiles % sms, nst = cdiv(Q, bq);
+        const int64_t splits = left ? std::min(sms / left, nst / 8) : 1;
+        const size_t bytes = sizeof(float) * (size_t)(left * nst * w.bp * w.kp);
+        if (share && splits >= 2 && bytes <= F32_TAIL_BYTES) {
+            w.q_per_split = cdiv(nst, splits) * bq;
+            w.tail.full = tiles - left;
+            w.tail.tiles = left;
+            w.tail.splits = (int)cdiv(Q, w.q_per_split);
+        }
     }
-    w.q_per_split = cdiv(cdiv(w.Q > 0 ? w.Q : 1, w.splits), bq) * bq;
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     w.f_off = 0;
-    const size_t fbytes = trans ? sizeof(float) * (size_t)(w.Q > 0 ? w.Q : 1) * w.kpt
+    const size_t fbytes = trans ? sizeof(float) * (size_t)Q * w.kpt
                                 : sizeof(float) * (size_t)w.kpt * w.ldf;
     w.part_off = al(fbytes);
     w.split_off = w.part_off +
-                  al(sizeof(double) * (size_t)(cdiv(w.P > 0 ? w.P : 1, w.bp) * w.splits));
-    w.total = w.split_off +
-              (w.splits > 1 ? al(sizeof(float) * 2 * (size_t)w.splits * (size_t)w.P * k) : 0);
+                  al(sizeof(double) * (size_t)(w.tail.full + w.tail.tiles * w.tail.splits + 1));
+    w.total = w.split_off;
+    if (w.splits > 1)
+        w.total += al(sizeof(float) * 2 * (size_t)w.splits * (size_t)w.P * k);
+    if (w.tail.tiles > 0)
+        w.total += al(sizeof(float) * (size_t)(w.tail.tiles * cdiv(Q, bq) * w.bp * w.kp));
     return w;
 }
 
@@ -529,13 +620,20 @@ nmf_status launch_tile(const float *A, const F32Plan &w, int64_t lda, const floa
     using T = F32Tile<TRANS, NCG, RPT>;
     const size_t smem = T::bytes(OBJ);
     static SmemOptIn opt_in;
-    const dim3 grid((unsigned)cdiv(w.P, T::BP), (unsigned)w.nch, (unsigned)w.splits);
     if constexpr (TRANS == 0) {
+        const dim3 grid((unsigned)(w.tail.full + w.tail.tiles * w.tail.splits));
         NMF_TRY(ensure_smem(mm_f32_kernel<OBJ, NCG, RPT>, opt_in, smem));
         mm_f32_kernel<OBJ, NCG, RPT><<<grid, T::THREADS, smem, s>>>(
-            A, w.P, w.Q, lda, Fc, w.ldf, k, w.q_per_split, out, W, part);
+            A, w.P, w.Q, lda, Fc, w.ldf, k, w.q_per_split, out, W, part, w.tail);
         NMF_LAUNCHED("mm_f32_kernel");
+        if (w.tail.tiles > 0) {
+            const int64_t len = w.tail.tiles * T::BP * T::KP;
+            f32_stage_kernel<NCG, RPT><<<(unsigned)cdiv(len, 256), 256, 0, s>>>(
+                w.P, cdiv(w.Q, w.bq), k, out, w.tail);
+            NMF_LAUNCHED("f32_stage_kernel");
+        }
     } else {
+        const dim3 grid((unsigned)cdiv(w.P, T::BP), (unsigned)w.nch, (unsigned)w.splits);
         NMF_TRY(ensure_smem(mm_f32_t_kernel<NCG, RPT>, opt_in, smem));
         static SmemOptIn carve;   // all of the SM's on-chip memory as shared memory
         int dev = 0;
@@ -572,9 +670,9 @@ bool mm_f32_supported(const float *A, int64_t lda)
     return (lda % 4) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
 }
 
-size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans)
+size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans, bool share)
 {
-    return f32_plan(m, n, k, trans).total;
+    return f32_plan(m, n, k, trans, share).total;
 }
 
 nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, const float *F, int k,
@@ -582,7 +680,9 @@ nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, cons
                          size_t work_bytes, cudaStream_t s)
 {
     const bool obj = W != nullptr;
-    const F32Plan w = f32_plan(m, n, k, trans);
+    F32Plan w = f32_plan(m, n, k, trans);
+    if (work_bytes < w.total)
+        w = f32_plan(m, n, k, trans, false);
     if (w.P == 0)
         return NMF_OK;
     if (!mm_f32_supported(A, lda) || work_bytes < w.total || (obj && (trans || k > 64 || !f_dev)))
@@ -590,6 +690,7 @@ nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, cons
     unsigned char *wb = static_cast<unsigned char *>(work);
     float *Fc = reinterpret_cast<float *>(wb + w.f_off);
     double *part = reinterpret_cast<double *>(wb + w.part_off);
+    w.tail.part = reinterpret_cast<float *>(wb + w.split_off);
     float *dst = w.splits > 1 ? reinterpret_cast<float *>(wb + w.split_off) : out;
     if (trans == 0) {
         const dim3 tg((unsigned)cdiv(w.ldf, 32), (unsigned)cdiv(w.kpt, 32));
@@ -616,7 +717,8 @@ nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, cons
         NMF_LAUNCHED("f32_reduce_kernel");
     }
     if (obj)
-        return launch_sum_partials(part, (int)(cdiv(w.P, w.bp) * w.splits), f_dev, s);
+        return launch_sum_partials(part, (int)(w.tail.full + w.tail.tiles * w.tail.splits), f_dev,
+                                   s);
     return NMF_OK;
 }
 

@@ -87,6 +87,8 @@
 
 #include <mutex>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -139,12 +141,18 @@ struct TcLayout {
 struct TcArgs {
     int64_t P, Q;
     int k, col0, kc;
-    int kb_per_split;       // K-blocks per CTA along the contraction (grid.y splits)
+    int kb_per_split;       // K-blocks per CTA along the contraction (grid.y splits; with the
+                            // objective, of the split tiles)
     float *out;             // grid.y == 1: the output; else partials [split][P][k]
     double *obj_partials;   // per-CTA sums of squared residuals (OBJ)
     int *err;
     // TRANS = 2: A^T pre-split, tile-major (see mm_tc_presplit_kernel).
     const unsigned char *at_hi, *at_lo;
+    // With the objective: CTAs 0 .. full - 1 take a whole tile each; the
+    // tiles from `full` on (`tail` of them) are shared by `tail_splits` CTAs,
+    // which write every fold's partial sums to fold_part (mm_tc_fold_kernel).
+    int full, tail, tail_splits;
+    float *fold_part;
     int64_t at_kbs;         // K-blocks per 128-row block of tiles
 };
 
@@ -211,10 +219,21 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    const int64_t p0 = (int64_t)blockIdx.x * TC_BM;
     const int nkb_all = (int)((Q + TC_BK - 1) / TC_BK);
-    const int kb0 = blockIdx.y * args.kb_per_split;   // first K-block of this CTA
-    const int nkb = min(args.kb_per_split, nkb_all - kb0);
+    int tile = blockIdx.x, nkb = nkb_all;
+    int kb0 = blockIdx.y * args.kb_per_split;   // first K-block of this CTA
+    const bool shared_tile = OBJ && tile >= args.full;
+    if (OBJ) {
+        kb0 = 0;
+        if (shared_tile) {
+            const int e = (int)blockIdx.x - args.full;
+            tile = args.full + e / args.tail_splits;
+            kb0 = (e % args.tail_splits) * args.kb_per_split;
+        }
+    }
+    if (!OBJ || shared_tile)
+        nkb = min(args.kb_per_split, nkb_all - kb0);
+    const int64_t p0 = (int64_t)tile * TC_BM;
     auto stage = [&](int s) { return sbase + (uint32_t)(s * L::STAGE_BYTES); };
     // Descriptors are formed once and advanced by constant adds: the start
     // address field holds addr >> 4 in its low 14 bits, and every shared
@@ -249,7 +268,7 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
                     // contiguous KB in global memory, already in the K-major
                     // swizzled operand layout the split warps would write.
                     const size_t toff =
-                        ((size_t)blockIdx.x * (size_t)args.at_kbs + (size_t)(kb0 + kb)) *
+                        ((size_t)tile * (size_t)args.at_kbs + (size_t)(kb0 + kb)) *
                         (size_t)L::A_BYTES;
                     bulk_load(dst, args.at_hi + toff, L::A_BYTES, full(s));
                     bulk_load(dst + L::A_BYTES, args.at_lo + toff, L::A_BYTES, full(s));
@@ -580,6 +599,16 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
             folded = true;
         };
         const int row = quarter * 32 + lane;    // row of the tile owned by this thread
+        // A shared tile's fold: the partial sums to fold_part, [fold][tile][column][row].
+        auto put_fold = [&](int f) {
+            float *o = args.fold_part +
+                       (((int64_t)f * args.tail + (tile - args.full)) * N + cbase) * TC_BM + row;
+#pragma unroll
+            for (int c = 0; c < NH; ++c) {
+                o[c * TC_BM] = part[c];
+                part[c] = 0.0f;
+            }
+        };
         bool ok = true;
         for (int kb = 0; kb < nkb; ++kb) {
             const int b = kb & 1, ub = kb >> 1;
@@ -593,19 +622,20 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(acc_empty(b));
-            if ((kb % TC_FOLD) == TC_FOLD - 1)
-                fold();
+            if ((kb % TC_FOLD) == TC_FOLD - 1) {
+                if (shared_tile)
+                    put_fold((kb0 + kb) / TC_FOLD);
+                else
+                    fold();
+            }
         }
-        if (ok) {
+        if (ok && shared_tile) {
+            if (kb0 + nkb == nkb_all)   // what is left, as the unsplit pass folds it
+                put_fold(nkb_all / TC_FOLD);
+        } else if (ok) {
             fold();
             const int64_t p = p0 + row;
-            const int64_t len = P * args.k;
-            // A split of the pass with the objective keeps its compensation too
-            // (two arrays per split), so that the sum over the splits rounds
-            // like the unsplit pass.
-            const bool pair = OBJ && gridDim.y > 1;
-            float *o = args.out + (int64_t)blockIdx.y * (pair ? 2 * len : len) + p * args.k +
-                       args.col0 + cbase;
+            float *o = args.out + (int64_t)blockIdx.y * P * args.k + p * args.k + args.col0 + cbase;
 #pragma unroll
             for (int c0 = 0; c0 < NH; c0 += CH) {
                 float sm[CH], cm[CH];
@@ -614,11 +644,8 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
                 if (p < P) {
 #pragma unroll
                     for (int i = 0; i < CH; ++i)
-                        if (cbase + c0 + i < args.kc) {
-                            o[c0 + i] = pair ? sm[i] : sm[i] - cm[i];
-                            if (pair)
-                                o[len + c0 + i] = -cm[i];
-                        }
+                        if (cbase + c0 + i < args.kc)
+                            o[c0 + i] = sm[i] - cm[i];
                 }
             }
         }
@@ -634,7 +661,7 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
             double s = 0.0;
             for (int w = 0; w < 4; ++w)
                 s += red[w];
-            args.obj_partials[blockIdx.y * gridDim.x + blockIdx.x] = s;
+            args.obj_partials[blockIdx.x] = s;
         }
     }
     if (warp == 1) {
@@ -784,6 +811,30 @@ __global__ void mm_tc_reduce_kernel(const float *__restrict__ part, int arrays, 
     out[e] = sum_strided(part + e, arrays, P * k);
 }
 
+// The shared tiles of the pass with the objective: out from the folds' partial
+// sums, added with the Kahan steps of the unsplit pass in its order (bitwise
+// its result). One thread per row and column; reads 4 bytes per fold.
+__global__ void mm_tc_fold_kernel(const float *__restrict__ part, int nfolds, int tail, int N,
+                                  int64_t p0, int64_t P, int k, float *__restrict__ out)
+{
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)tail * N * TC_BM;
+    if (e >= stride)
+        return;
+    float s = 0.0f, c = 0.0f;
+#pragma unroll 8
+    for (int f = 0; f < nfolds; ++f) {
+        const float y = part[f * stride + e] - c;
+        const float t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
+    const int64_t p = p0 + e / ((int64_t)N * TC_BM) * TC_BM + e % TC_BM;
+    const int col = (int)(e / TC_BM % N);
+    if (p < P && col < k)
+        out[p * k + col] = s - c;
+}
+
 __global__ void obj_sum_kernel(const double *__restrict__ parts, int n, double *__restrict__ f)
 {
     __shared__ double red[32];
@@ -814,7 +865,9 @@ nmf_status launch_tc(const CUtensorMap (&maps)[5], const TcArgs &a, cudaStream_t
     static SmemOptIn opt_in;
     NMF_TRY(ensure_smem(mm_tc_kernel<N, TRANS, OBJ>, opt_in, (size_t)smem));
     const int nkb = (int)cdiv(a.Q, TC_BK);
-    const dim3 grid((unsigned)cdiv(a.P, TC_BM), (unsigned)cdiv(nkb, a.kb_per_split));
+    const dim3 grid(OBJ ? (unsigned)(a.full + a.tail * a.tail_splits)
+                        : (unsigned)cdiv(a.P, TC_BM),
+                    OBJ ? 1u : (unsigned)cdiv(nkb, a.kb_per_split));
     mm_tc_kernel<N, TRANS, OBJ><<<grid, L::THREADS, smem, s>>>(maps[0], maps[1], maps[2], maps[3],
                                                                maps[4], a);
     NMF_LAUNCHED("mm_tc_kernel");
@@ -839,10 +892,7 @@ struct TcWork {
 
 constexpr int TC_MAX_SPLITS = 16;   // tall-skinny A: few output tiles, a long contraction
 
-// Contraction splits that fill the last wave of CTAs better (1 CTA per SM),
-// with and without the objective (each split sums its own columns' residuals:
-// 24000 x 16000, k = 50 with the objective took 392 us in 188 CTAs, against
-// 243 us for the product alone in 752).
+// Contraction splits that fill the last wave of CTAs better (1 CTA per SM).
 int choose_splits(int64_t P, int64_t Q)
 {
     const int64_t tiles = cdiv(P, TC_BM), nkb = cdiv(Q, TC_BK);
@@ -862,6 +912,35 @@ int choose_splits(int64_t P, int64_t Q)
     return best;
 }
 
+// The pass with the objective (1 CTA per SM) takes the tiles of its whole waves
+// unsplit and shares out the contraction of those left over, whose partial
+// sums are then added in the unsplit order: the products do not depend on the
+// grid (24000 x 16000, k = 50: 392 us in 188 unsplit CTAs, 258 + 11 us so).
+struct ObjPlan {
+    int full, tail, splits, kb_per_split, nfolds;
+};
+
+ObjPlan obj_plan(int64_t P, int64_t Q)
+{
+    const int tiles = (int)cdiv(P, TC_BM), nkb = (int)cdiv(Q, TC_BK), sms = sm_count();
+    ObjPlan o;
+    o.full = tiles;
+    o.tail = 0;
+    o.splits = 1;
+    o.kb_per_split = nkb;
+    o.nfolds = nkb / TC_FOLD + 1;
+    const int left = tiles % sms;
+    // At least two folds per CTA.
+    const int splits = left ? std::min(sms / left, nkb / (2 * TC_FOLD)) : 1;
+    if (splits >= 2) {
+        o.full = tiles - left;
+        o.tail = left;
+        o.kb_per_split = (int)cdiv(cdiv(nkb, splits), TC_FOLD) * TC_FOLD;
+        o.splits = (int)cdiv(nkb, o.kb_per_split);
+    }
+    return o;
+}
+
 TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj)
 {
     const int64_t P = trans ? n : m;
@@ -877,13 +956,18 @@ TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj)
     if (obj)
         off += al(2 * sizeof(__nv_bfloat16) * (size_t)Pp * 64);
     w.part_off = off;
-    const int splits = choose_splits(P, Q);
-    if (obj)
-        off += al(sizeof(double) * (size_t)(Pp / TC_BM) * (size_t)splits);
+    if (obj) {
+        const ObjPlan o = obj_plan(P > 0 ? P : 1, Q > 0 ? Q : 1);
+        off += al(sizeof(double) * (size_t)(o.full + o.tail * o.splits));
+        w.split_off = off;
+        off += al(sizeof(float) * (size_t)o.nfolds * (size_t)o.tail * (size_t)N * TC_BM);
+        w.total = off;
+        return w;
+    }
     w.split_off = off;
+    const int splits = choose_splits(P, Q);
     if (splits > 1)
-        off += al(sizeof(float) * (size_t)(obj ? 2 * splits : splits) *
-                  (size_t)(P > 0 ? P : 1) * (size_t)k);
+        off += al(sizeof(float) * (size_t)splits * (size_t)(P > 0 ? P : 1) * (size_t)k);
     w.total = off;
     return w;
 }
@@ -999,9 +1083,15 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
         const int splits = choose_splits(P, Q);
         const int nkb = (int)cdiv(Q, TC_BK);
         a.kb_per_split = (int)cdiv(nkb, splits);
-        if (fuse)   // whole folds: the partial sums of the unsplit pass
-            a.kb_per_split = (int)cdiv(a.kb_per_split, TC_FOLD) * TC_FOLD;
-        const int grid_y = (int)cdiv(nkb, a.kb_per_split);
+        const ObjPlan op = obj_plan(P, Q);
+        if (fuse) {
+            a.kb_per_split = op.kb_per_split;
+            a.full = op.full;
+            a.tail = op.tail;
+            a.tail_splits = op.splits;
+            a.fold_part = reinterpret_cast<float *>(wb + wl.split_off);
+        }
+        const int grid_y = fuse ? 1 : (int)cdiv(nkb, a.kb_per_split);
         float *partial = reinterpret_cast<float *>(wb + wl.split_off);
         a.out = grid_y > 1 ? partial : out;
         nmf_status st;
@@ -1013,12 +1103,18 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
             st = presplit ? launch_tc_n<3, 0>(N, maps, a, s) : launch_tc_n<0, 0>(N, maps, a, s);
         NMF_TRY(st);
         if (grid_y > 1) {
-            mm_tc_reduce_kernel<<<(unsigned)cdiv(P * kc, 256), 256, 0, s>>>(
-                partial, fuse ? 2 * grid_y : grid_y, P, k, col0, kc, out);
+            mm_tc_reduce_kernel<<<(unsigned)cdiv(P * kc, 256), 256, 0, s>>>(partial, grid_y, P, k,
+                                                                            col0, kc, out);
             NMF_LAUNCHED("mm_tc_reduce_kernel");
         }
         if (fuse) {
-            obj_sum_kernel<<<1, 256, 0, s>>>(a.obj_partials, (int)(Pp / TC_BM) * grid_y, f_dev);
+            if (op.tail > 0) {
+                const int64_t len = (int64_t)op.tail * N * TC_BM;
+                mm_tc_fold_kernel<<<(unsigned)cdiv(len, 256), 256, 0, s>>>(
+                    a.fold_part, op.nfolds, op.tail, N, (int64_t)op.full * TC_BM, P, k, out);
+                NMF_LAUNCHED("mm_tc_fold_kernel");
+            }
+            obj_sum_kernel<<<1, 256, 0, s>>>(a.obj_partials, op.full + op.tail * op.splits, f_dev);
             NMF_LAUNCHED("obj_sum_kernel");
         }
     }
