@@ -161,15 +161,29 @@ extern "C" nmf_status nmf_nls_bpp(const nmf_nls_desc *d, void *stream)
     if (ranges_overlap(d->B, d->X, sizeof(float) * (size_t)d->nrhs * d->k))
         return NMF_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    TempBuf w(s), st(s);
-    NMF_CUDA(w.alloc(bpp_work_bytes(d->k)));
-    NMF_CUDA(st.alloc(sizeof(BppStats)));
-    NMF_CUDA(cudaMemsetAsync(st.p, 0, sizeof(BppStats), s));
+    // One buffer: statistics, workspace, and scratch for predicted partitions
+    // where the caller asks for neither passive sets nor round counts (which
+    // an FP64 half-step counts from its start). Without the memory for the
+    // scratch the FP64 solves start from passive_in.
+    const size_t base = 256 + bpp_work_bytes(d->k);
+    const size_t words = (size_t)d->nrhs * ((d->k + 63) / 64);
+    bool scratch = !d->passive_out && !d->rounds_out;
+    TempBuf w(s);
+    if (scratch && w.alloc(base + sizeof(uint64_t) * words) != cudaSuccess) {
+        cudaGetLastError();
+        w.p = nullptr;
+        scratch = false;
+    }
+    if (!w.p)
+        NMF_CUDA(w.alloc(base));
+    unsigned char *wp = static_cast<unsigned char *>(w.p);
+    BppStats *st = reinterpret_cast<BppStats *>(wp);
+    NMF_CUDA(cudaMemsetAsync(st, 0, sizeof(BppStats), s));
     NMF_TRY(launch_bpp(d->k, d->nrhs, d->G, d->B, d->X, d->passive_in, d->passive_out,
-                       d->rounds_out, d->status_out, d->max_rounds, w.p,
-                       static_cast<BppStats *>(st.p), s));
+                       d->rounds_out, d->status_out, d->max_rounds, wp + 256, st, s,
+                       scratch ? reinterpret_cast<uint64_t *>(wp + base) : nullptr));
     BppStats host;
-    NMF_CUDA(cudaMemcpyAsync(&host, st.p, sizeof(BppStats), cudaMemcpyDeviceToHost, s));
+    NMF_CUDA(cudaMemcpyAsync(&host, st, sizeof(BppStats), cudaMemcpyDeviceToHost, s));
     NMF_CUDA(cudaStreamSynchronize(s));
     return worst_from_stats(host);
 }

@@ -892,7 +892,7 @@ __global__ void __launch_bounds__(BPP_THREADS, 2)
         nwork = use_list ? (int64_t)nd : P.nrhs;
         counter = &P.counters[CNT_DEFER_WORK];
     } else if (P.predict) {
-        pin = P.pout;
+        pin = P.predict;
     }
     solve64<KW, (KW + 1) / 2, 1>(P, sh1, pin, nwork, use_list, counter);
 }
@@ -966,13 +966,17 @@ nmf_status launch_modes(SolveParams P, cudaStream_t s)
     if (P.fused) {
         // FP64 half-step: the right-hand sides are formed here instead of
         // inside the FP32 solves.
-        NMF_TRY(launch_spmm_unless_fp32(P.gat.rowptr, P.gat.colidx, P.gat.vals, P.nrhs, P.gat.F,
-                                        P.k, const_cast<float *>(P.B), P.flags, s));
+        NMF_TRY(launch_spmm_unless_fp32(P.gat.rowptr, P.gat.colidx, P.gat.vals, P.nrhs,
+                                        P.gat.cols, P.gat.F, P.k, const_cast<float *>(P.B),
+                                        P.flags, s));
     }
     // Mode 1 (FP64): the FP32 kernel first predicts each right-hand side's
-    // partition into pout, and the FP64 solves start from it (their answer
-    // does not depend on the start; they need fewer rounds).
-    P.predict = P.pout && P.max_rounds >= 2 * PREDICT_ROUNDS;   // (a tight cap keeps its meaning)
+    // partition, and the FP64 solves start from it (their answer does not
+    // depend on the start; they need fewer rounds: 16000 right-hand sides, k =
+    // 50, from the signs of the unconstrained solution: 0.32 ms, 1.25 from that
+    // start itself). Not under a tight cap, which keeps its meaning.
+    if (P.max_rounds < 2 * PREDICT_ROUNDS)
+        P.predict = nullptr;
     NMF_TRY(launch_solve32(P, s));
     return launch_solve64<KW>(P, s);
 }
@@ -1031,9 +1035,9 @@ SolveParams solve_params(int k, int64_t nrhs, const double *G, const float *B, f
     P.rounds_out = rounds_out;
     P.status_out = status_out;
     P.counters = reinterpret_cast<unsigned long long *>(w + L.counters);
-    P.predict = 0;
+    P.predict = passive_out;
     P.fused = 0;
-    P.gat = CsrGather{nullptr, nullptr, nullptr, nullptr};
+    P.gat = CsrGather{nullptr, nullptr, nullptr, nullptr, 0};
     P.defer = reinterpret_cast<int64_t *>(w + L.defer);
     P.stats = stats_dev;
     const BppShape sh = shape_for(k);
@@ -1097,7 +1101,7 @@ nmf_status launch_bpp_prep(int k, const double *G, void *work, BppStats *stats_d
 nmf_status launch_bpp_solve(int k, int64_t nrhs, const double *G, const float *B, float *X,
                             const uint64_t *passive_in, uint64_t *passive_out, int32_t *rounds_out,
                             int8_t *status_out, int max_rounds, void *work, BppStats *stats_dev,
-                            cudaStream_t s, const CsrGather *gather)
+                            cudaStream_t s, const CsrGather *gather, uint64_t *predict)
 {
     if (nrhs == 0)
         return NMF_OK;
@@ -1107,6 +1111,8 @@ nmf_status launch_bpp_solve(int k, int64_t nrhs, const double *G, const float *B
         P.fused = 1;
         P.gat = *gather;
     }
+    if (!P.predict)
+        P.predict = predict;
     return launch_solves(P, s);
 }
 
@@ -1205,11 +1211,11 @@ nmf_status bpp_get_shape(int k, int *warps, int *chunk, int *group)
 nmf_status launch_bpp(int k, int64_t nrhs, const double *G, const float *B, float *X,
                       const uint64_t *passive_in, uint64_t *passive_out, int32_t *rounds_out,
                       int8_t *status_out, int max_rounds, void *work, BppStats *stats_dev,
-                      cudaStream_t s)
+                      cudaStream_t s, uint64_t *predict)
 {
     NMF_TRY(launch_bpp_prep(k, G, work, stats_dev, s));
     return launch_bpp_solve(k, nrhs, G, B, X, passive_in, passive_out, rounds_out, status_out,
-                            max_rounds, work, stats_dev, s);
+                            max_rounds, work, stats_dev, s, nullptr, predict);
 }
 
 }  // namespace nmf

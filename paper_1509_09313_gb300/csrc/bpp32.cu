@@ -1104,7 +1104,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
                                    ((P.pin[j * P.nwords + (i >> 6)] >> (i & 63)) & 1ull);
                         }
                     }
-                    write_words<KW>(f, P.pout + j * P.nwords, lane);
+                    write_words<KW>(f, P.predict + j * P.nwords, lane);
                 }
                 continue;
             }

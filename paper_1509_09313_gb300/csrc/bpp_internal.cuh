@@ -51,11 +51,11 @@ struct SolveParams {
     unsigned long long *counters;  // CNT_WORDS words
     int64_t *defer;                // DEFER_CAP indices
     BppStats *stats;
-    // predict = 1: in an FP64 (mode 1) half-step the FP32 kernel runs too, and
-    // only writes passive sets (pout) for the FP64 solves to start from; no X,
+    // Not null: in an FP64 (mode 1) half-step the FP32 kernel runs too, and
+    // only writes passive sets there for the FP64 solves to start from; no X,
     // rounds, status or statistics, at most PREDICT_ROUNDS rounds, its own
-    // counter.
-    int predict;
+    // counter. (pout, or scratch where the caller wants no passive sets.)
+    uint64_t *predict;
     // group = 1: the group-tile pass ran first; the per-warp kernel solves
     // only the right-hand sides it marked GROUP_PENDING.
     int group;

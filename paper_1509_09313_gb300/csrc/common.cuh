@@ -215,6 +215,8 @@ nmf_status launch_pgrad_sq(const double *G, int k, const float *R, const float *
                            double *partials, double *out, cudaStream_t s);
 
 // Batched BPP. Workspace layout is private to bpp.cu; size from bpp_work_bytes.
+// predict (nrhs rows of words, or null) is scratch for the FP64 half-steps'
+// predicted partitions of a caller without passive_out and rounds_out.
 size_t bpp_work_bytes(int k);
 struct BppStats {
     unsigned long long rhs, rounds, max_rounds, fp64_solves, not_converged, singular, nonfinite,
@@ -223,7 +225,7 @@ struct BppStats {
 nmf_status launch_bpp(int k, int64_t nrhs, const double *G, const float *B, float *X,
                       const uint64_t *passive_in, uint64_t *passive_out, int32_t *rounds_out,
                       int8_t *status_out, int max_rounds, void *work, BppStats *stats_dev,
-                      cudaStream_t s);
+                      cudaStream_t s, uint64_t *predict = nullptr);
 // The two halves of launch_bpp: the per-Gram preparation (factor, inverse,
 // arithmetic mode), then the solves. A prep must complete before its solves
 // and must not overlap another half-step's prep or solves on the same work.
@@ -242,7 +244,8 @@ nmf_status bpp_get_shape(int k, int *warps, int *chunk, int *group);
 nmf_status launch_bpp_solve(int k, int64_t nrhs, const double *G, const float *B, float *X,
                             const uint64_t *passive_in, uint64_t *passive_out, int32_t *rounds_out,
                             int8_t *status_out, int max_rounds, void *work, BppStats *stats_dev,
-                            cudaStream_t s, const CsrGather *gather = nullptr);
+                            cudaStream_t s, const CsrGather *gather = nullptr,
+                            uint64_t *predict = nullptr);
 
 // Learned passive-set proposal (mlp.cu).
 struct MlpNet;
