@@ -122,7 +122,7 @@ extern "C" nmf_status nmf_mm_csr(const int64_t *rowptr, const int32_t *colidx, c
         return NMF_OK;
     if (!rowptr || !out || !F || !colidx || !vals)
         return NMF_ERR_INVALID_ARG;
-    return launch_spmm(rowptr, colidx, vals, rows, F, k, out, as_stream(stream));
+    return launch_spmm(rowptr, colidx, vals, rows, cols, F, k, out, as_stream(stream));
 }
 
 extern "C" nmf_status nmf_csr_transpose(const int64_t *rowptr, const int32_t *colidx,
@@ -389,8 +389,9 @@ nmf_status mm(nmf_handle *h, int trans, const float *F, float *out)
     const nmf_config &c = h->cfg;
     if (c.input_kind == NMF_INPUT_CSR) {
         if (trans == 0)
-            return launch_spmm(h->A.rowptr, h->A.colidx, h->A.vals, c.m, F, c.k, out, h->stream);
-        return launch_spmm(h->t_rowptr, h->t_colidx, h->t_vals, c.n, F, c.k, out, h->stream);
+            return launch_spmm(h->A.rowptr, h->A.colidx, h->A.vals, c.m, c.n, F, c.k, out,
+                               h->stream);
+        return launch_spmm(h->t_rowptr, h->t_colidx, h->t_vals, c.n, c.m, F, c.k, out, h->stream);
     }
     if (c.precision == NMF_PREC_BF16X3) {
         h->mm_splits_max = std::max<int64_t>(h->mm_splits_max, mm_tc_splits(c.m, c.n, trans));
@@ -506,8 +507,8 @@ nmf_status one_iteration(nmf_handle *h)
         NMF_CUDA(cudaEventRecord(h->ev_join, h->side));
         return NMF_OK;
     };
-    const CsrGather gather_w{h->A.rowptr, h->A.colidx, h->A.vals, h->Ht};
-    const CsrGather gather_h{h->t_rowptr, h->t_colidx, h->t_vals, h->W};
+    const CsrGather gather_w{h->A.rowptr, h->A.colidx, h->A.vals, h->Ht, c.n};
+    const CsrGather gather_h{h->t_rowptr, h->t_colidx, h->t_vals, h->W, c.m};
     // W <- argmin_{W >= 0} ||A - W H||: Gram H H^T, right-hand sides A H^T.
     NMF_TRY(fork_prepare(h->Ht, c.n, h->GH, h->gh_current));
     if (!fuse) {

@@ -1093,7 +1093,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
             if (predict) {
                 // Only the partition reached seeds the FP64 solves; where the
                 // FP32 system was singular, the starting one (given or empty).
-                if (P.pout) {
+                {
                     bool f[KW];
 #pragma unroll
                     for (int s = 0; s < KW; ++s) {

@@ -170,14 +170,16 @@ nmf_status launch_mm_tc_presplit(const void *hi, const void *lo, int64_t m, int6
                                  const float *F, int k, int trans, float *out, const float *W,
                                  double *f_dev, void *work, size_t work_bytes, cudaStream_t s);
 
-// CSR SpMM: out (rows x k) = S F.
+// CSR SpMM: out (rows x k) = S F, F cols x k.
 nmf_status launch_spmm(const int64_t *rowptr, const int32_t *colidx, const float *vals,
-                       int64_t rows, const float *F, int k, float *out, cudaStream_t s);
+                       int64_t rows, int64_t cols, const float *F, int k, float *out,
+                       cudaStream_t s);
 // The same product, skipped on the device when *mode_flag == 0 (an FP32
 // half-step whose solves gather their right-hand sides themselves).
 nmf_status launch_spmm_unless_fp32(const int64_t *rowptr, const int32_t *colidx,
-                                   const float *vals, int64_t rows, const float *F, int k,
-                                   float *out, const int *mode_flag, cudaStream_t s);
+                                   const float *vals, int64_t rows, int64_t cols,
+                                   const float *F, int k, float *out, const int *mode_flag,
+                                   cudaStream_t s);
 
 // Right-hand sides formed inside the batched BPP as b_j = (S F)_j (rows of the
 // CSR matrix S times F, k columns), for the sparse ANLS half-steps.
@@ -186,6 +188,7 @@ struct CsrGather {
     const int32_t *colidx;
     const float *vals;
     const float *F;
+    int64_t cols;   // rows of F
 };
 
 // Objective pieces. Dense: per-block FP64 partial sums of squared residuals,

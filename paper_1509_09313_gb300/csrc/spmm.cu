@@ -11,7 +11,11 @@
 //
 // Roofline: HBM. Compulsory bytes per product: rowptr + colidx + vals +
 // F + out; the gathers of F rows add up to nnz * k * 4 bytes when F is not
-// L2-resident.
+// L2-resident. While it is, 64 warps per SM with one or two rows in flight
+// each are best (200000 x 10^6, 10^7 entries, k = 20: 237 us against 360 with
+// spmm_stream_kernel; 100000 x 50000, 10^6 entries, k = 50: 40 against 52);
+// beyond, fewer warps with eight in flight (10^6 x 10^6, 10^7 entries: k = 50
+// 609 us against 480, k = 33, 132 MB, 532 against 449).
 #include "common.cuh"
 
 namespace nmf {
@@ -59,6 +63,113 @@ __global__ void __launch_bounds__(SPMM_THREADS)
             if (r < k)
                 out[i * k + r] = acc[s];
         }
+    }
+}
+
+// Rows of F gathered from beyond the L2 cache: a warp takes up to STREAM_ROWS
+// consecutive rows, whose stored entries are one stretch, reads the entries 32
+// at a time, the next 32 while these are used, and keeps STREAM_BATCH gathered
+// rows in flight, in 24 to 32 warps per SM. The same sums in the same order as
+// spmm_kernel. VEC = 2: k even and F, out 8-byte aligned; lane l owns columns
+// 2 l + 64 s and the next (KW slots). VEC = 1: columns l + 32 s.
+constexpr int STREAM_ROWS = 16, STREAM_BATCH = 8;
+
+template <int KW, int VEC>
+__global__ void __launch_bounds__(SPMM_THREADS)
+    spmm_stream_kernel(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                       const float *__restrict__ vals, int64_t rows, const float *__restrict__ F,
+                       int k, float *__restrict__ out, const int *__restrict__ mode_flag,
+                       int chunk)
+{
+    if (mode_flag && *mode_flag == 0)
+        return;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp0 = ((int64_t)blockIdx.x * SPMM_THREADS + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * SPMM_THREADS) >> 5;
+    for (int64_t r0 = warp0 * chunk; r0 < rows; r0 += nw * chunk) {
+        const int nr = (int)min((int64_t)chunk, rows - r0);
+        const int64_t rp = rowptr[r0 + min(lane, nr)];   // lane l: the start of row r0 + l
+        const int64_t end = __shfl_sync(FULL, rp, nr);
+        float acc[KW][VEC];
+#pragma unroll
+        for (int s = 0; s < KW; ++s)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e)
+                acc[s][e] = 0.0f;
+        int r = 0;
+        int64_t p = __shfl_sync(FULL, rp, 0), rend = __shfl_sync(FULL, rp, 1);
+        auto put_row = [&]() {   // row r is complete
+#pragma unroll
+            for (int s = 0; s < KW; ++s) {
+                const int c = VEC * (lane + 32 * s);
+                if (c < k) {
+                    float *o = out + (r0 + r) * k + c;
+                    if constexpr (VEC == 2)
+                        *reinterpret_cast<float2 *>(o) = make_float2(acc[s][0], acc[s][1]);
+                    else
+                        *o = acc[s][0];
+                }
+#pragma unroll
+                for (int e = 0; e < VEC; ++e)
+                    acc[s][e] = 0.0f;
+            }
+            ++r;
+            rend = __shfl_sync(FULL, rp, min(r + 1, nr));
+        };
+        int c = 0, cn = 0;
+        float v = 0.0f, vn = 0.0f;
+        if (p + lane < end) {
+            cn = colidx[p + lane];
+            vn = vals[p + lane];
+        }
+        while (p < end) {
+            c = cn;
+            v = vn;
+            const int64_t pn = p + 32 + lane;
+            cn = pn < end ? colidx[pn] : 0;
+            vn = pn < end ? vals[pn] : 0.0f;
+            const int cnt = (int)min((int64_t)32, end - p);
+            for (int l = 0; l < cnt;) {
+                while (r < nr && rend <= p + l)
+                    put_row();
+                if (r == nr)
+                    break;
+                const int n = (int)min((int64_t)min(cnt - l, STREAM_BATCH), rend - (p + l));
+                float f[STREAM_BATCH][KW][VEC], w[STREAM_BATCH];
+#pragma unroll
+                for (int q = 0; q < STREAM_BATCH; ++q)
+                    if (q < n) {
+                        const int64_t cl = __shfl_sync(FULL, c, l + q);
+                        w[q] = __shfl_sync(FULL, v, l + q);
+                        const float *frow = F + cl * k;
+#pragma unroll
+                        for (int s = 0; s < KW; ++s) {
+                            const int cc = VEC * (lane + 32 * s);
+                            if constexpr (VEC == 2) {
+                                const float2 t = cc < k
+                                                     ? *reinterpret_cast<const float2 *>(frow + cc)
+                                                     : make_float2(0.0f, 0.0f);
+                                f[q][s][0] = t.x;
+                                f[q][s][1] = t.y;
+                            } else {
+                                f[q][s][0] = cc < k ? frow[cc] : 0.0f;
+                            }
+                        }
+                    }
+#pragma unroll
+                for (int q = 0; q < STREAM_BATCH; ++q)
+                    if (q < n)
+#pragma unroll
+                        for (int s = 0; s < KW; ++s)
+#pragma unroll
+                            for (int e = 0; e < VEC; ++e)
+                                acc[s][e] = fmaf(w[q], f[q][s][e], acc[s][e]);
+                l += n;
+            }
+            p += 32;
+        }
+        while (r < nr)
+            put_row();
     }
 }
 
@@ -136,12 +247,49 @@ __global__ void sort_rows_kernel(const int64_t *__restrict__ t_rowptr, int64_t n
 }  // namespace
 
 namespace {
+
+double l2_bytes()
+{
+    static double bytes = 0.0;
+    if (bytes == 0.0) {
+        int dev = 0, b = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&b, cudaDevAttrL2CacheSize, dev);
+        bytes = b > 0 ? b : 1.0;
+    }
+    return bytes;
+}
+
+// cols: the rows of F.
 nmf_status spmm_launch(const int64_t *rowptr, const int32_t *colidx, const float *vals,
-                       int64_t rows, const float *F, int k, float *out, const int *mode_flag,
-                       cudaStream_t s)
+                       int64_t rows, int64_t cols, const float *F, int k, float *out,
+                       const int *mode_flag, cudaStream_t s)
 {
     if (rows == 0)
         return NMF_OK;
+    const int64_t frows = cols < 0 ? 0 : cols;
+    if ((double)frows * k * sizeof(float) > 0.9 * l2_bytes()) {
+        const bool pairs = k % 2 == 0 && ((reinterpret_cast<uintptr_t>(F) |
+                                           reinterpret_cast<uintptr_t>(out)) & 7) == 0;
+        const int kw = (int)cdiv(k, pairs ? 64 : 32);
+        auto kernel = pairs ? (kw == 1 ? spmm_stream_kernel<1, 2> : spmm_stream_kernel<2, 2>)
+                      : kw == 1 ? spmm_stream_kernel<1, 1>
+                      : kw == 2 ? spmm_stream_kernel<2, 1>
+                      : kw == 3 ? spmm_stream_kernel<3, 1>
+                                : spmm_stream_kernel<4, 1>;
+        int per_sm = 0;
+        NMF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, SPMM_THREADS, 0));
+        const int64_t most = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();
+        // Chunks of STREAM_ROWS rows, shorter where that leaves warps without
+        // one.
+        const int64_t warps = most * (SPMM_THREADS / 32), share = rows / (2 * warps);
+        const int chunk = (int)(share < 1 ? 1 : share < STREAM_ROWS ? share : STREAM_ROWS);
+        const int64_t want = cdiv(cdiv(rows, chunk) * 32, SPMM_THREADS);
+        kernel<<<(unsigned)(want < most ? want : most), SPMM_THREADS, 0, s>>>(
+            rowptr, colidx, vals, rows, F, k, out, mode_flag, chunk);
+        NMF_LAUNCHED("spmm_stream_kernel");
+        return NMF_OK;
+    }
     int64_t blocks = cdiv(rows * 32, SPMM_THREADS);
     const int64_t cap = 16LL * sm_count();
     if (blocks > cap)
@@ -161,16 +309,18 @@ nmf_status spmm_launch(const int64_t *rowptr, const int32_t *colidx, const float
 }  // namespace
 
 nmf_status launch_spmm(const int64_t *rowptr, const int32_t *colidx, const float *vals,
-                       int64_t rows, const float *F, int k, float *out, cudaStream_t s)
+                       int64_t rows, int64_t cols, const float *F, int k, float *out,
+                       cudaStream_t s)
 {
-    return spmm_launch(rowptr, colidx, vals, rows, F, k, out, nullptr, s);
+    return spmm_launch(rowptr, colidx, vals, rows, cols, F, k, out, nullptr, s);
 }
 
 nmf_status launch_spmm_unless_fp32(const int64_t *rowptr, const int32_t *colidx,
-                                   const float *vals, int64_t rows, const float *F, int k,
-                                   float *out, const int *mode_flag, cudaStream_t s)
+                                   const float *vals, int64_t rows, int64_t cols,
+                                   const float *F, int k, float *out, const int *mode_flag,
+                                   cudaStream_t s)
 {
-    return spmm_launch(rowptr, colidx, vals, rows, F, k, out, mode_flag, s);
+    return spmm_launch(rowptr, colidx, vals, rows, cols, F, k, out, mode_flag, s);
 }
 
 nmf_status launch_csr_transpose(const int64_t *rowptr, const int32_t *colidx, const float *vals,

@@ -46,3 +46,30 @@ def test_bpp_batch_equals_its_parts(nmf, nrhs, k, warm):
                 assert torch.equal(part[name], whole[name][a:b]), (name, a, b)
     finally:
         nmf.nmf_nls_bpp_set_shape(k, *old)
+
+
+# F below and above the L2 cache (two kernels), even and odd k (pairs of columns
+# or single ones), empty rows, a row longer than a 32-entry block: each output
+# row against FP64, within the FP32 sum's error.
+@pytest.mark.parametrize("k", [2, 33, 50, 65, 128])
+@pytest.mark.parametrize("cols", [5000, 40_000_000])
+def test_spmm_small_and_streamed_factors(nmf, cols, k):
+    cols = 5000 if cols == 5000 else 150_000_000 // (4 * k) + 1
+    rng = np.random.default_rng(cols % 1000 + k)
+    count = rng.integers(0, 25, 3001)
+    count[[0, 7, 8, 3000]] = 0
+    count[100] = 333
+    rowptr = np.concatenate([[0], np.cumsum(count)])
+    colidx = np.sort(rng.integers(0, cols, rowptr[-1])).astype(np.int32)
+    rng.shuffle(colidx)
+    vals = rng.uniform(-1, 1, rowptr[-1]).astype(np.float32)
+    F = torch.rand((cols, k), device="cuda", generator=torch.Generator("cuda").manual_seed(k))
+    rp, ci, va = (torch.from_numpy(x).cuda() for x in (rowptr.astype(np.int64), colidx, vals))
+    out = nmf.nmf_mm_csr(rp, ci, va, cols, F)
+    row = torch.repeat_interleave(torch.arange(3001, device="cuda"), rp.diff())
+    terms = va.double()[:, None] * F[ci.long()].double()
+    ref = torch.zeros((3001, k), dtype=torch.float64, device="cuda").index_add_(0, row, terms)
+    size = torch.zeros_like(ref).index_add_(0, row, terms.abs())
+    # n sequential FMAs: at most n roundings of the running sum.
+    n = rp.diff().clamp_min(1).double()[:, None]
+    assert ((out.double() - ref).abs() <= n * 2.0 ** -24 * size).all()
