@@ -241,7 +241,7 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
                     pp[a][b] = make_float2(0.0f, 0.0f);
-#pragma unroll 2
+#pragma unroll   // (all: with 7 or 8 warps per SM the loads need the whole stage to hide in)
             for (int qq = 0; qq < BQ / 4; ++qq) {
                 float4 av[RPT], fv[4];
 #pragma unroll
@@ -314,7 +314,7 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
                     pp[ap][b] = make_float2(0.0f, 0.0f);
-#pragma unroll 1
+#pragma unroll   // (all: 24000 x 16000, k = 50 1367 us rolled, 1270 by 4, 1115 so)
             for (int q = 0; q < BQ; ++q) {
                 float2 av[RPT / 2];
 #pragma unroll
