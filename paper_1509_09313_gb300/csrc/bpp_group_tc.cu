@@ -8,10 +8,9 @@
 // empty start every usable y_i = -g_i infeasible); for the group F = U and the
 // factor is the inverse M = G_UU^{-1} the preparation holds, so
 //     x0 = M g,   r = g - G x0 (on U),   x1 = x0 + M r,
-// and x1 is kept where it passes the sign test. A member is marked
-// GROUP_PENDING before its tile is solved and the mark is overwritten only by
-// its solution, so anything this pass does not finish (including a wait that
-// timed out) goes to the per-warp kernel.
+// and x1 is kept where it passes the sign test. A member whose solution is not
+// kept (or not formed, when a wait timed out) is marked GROUP_PENDING and goes
+// to the per-warp kernel.
 //
 // The three products run as tcgen05 MMAs (M = 128 right-hand sides, N = k
 // padded to 16, K = 16) on BF16 splits, accumulated in FP32 in TMEM:
@@ -34,9 +33,18 @@
 //              (split in registers, stored in the canonical K-major
 //              128-byte-swizzled layout), the masks, the sign test and the
 //              outputs; per-row decisions combine the four threads' partial
-//              results through shared memory (named barrier 1).
-// M and G (split) stay in shared memory for the whole kernel. Every mbarrier
-// wait is bounded (~2 s).
+//              results through shared memory (a named barrier of the four
+//              warps that share 32 rows).
+// M and G (split) stay in shared memory for the whole kernel: with the A tiles
+// they fill it, so one tile is in flight per SM and its chain of phases bounds
+// the kernel. What shortens the chain: the next tile's right-hand sides are
+// loaded into registers while the last product runs; results leave through
+// the A tiles in bulk copies (rows of k floats: a warp's own stores touch 32
+// lines each); membership divides only where products cannot decide it; one
+// exchange per decision. 1e6 right-hand sides, k = 100: 33000 cycles per tile
+// without these (888 us for the kernel), 23000 with them (637 us); by memory traffic
+// it would be 120 us.
+// Every mbarrier wait is bounded (~2 s).
 #include <math.h>
 
 #include "bpp_internal.cuh"
@@ -66,9 +74,10 @@ struct GcLayout {
     static constexpr int OFF_TMEM = OFF_BAR + 16;
     static constexpr int OFF_ABORT = OFF_TMEM + 4;
     static constexpr int OFF_DSQ = OFF_BAR + 32;     // GC_MAX_K floats
-    static constexpr int OFF_USE = OFF_DSQ + 4 * GC_MAX_K;
-    static constexpr int OFF_XCH = (OFF_USE + GC_MAX_K + 15) & ~15;   // [part][row] int, float
-    static constexpr int BYTES = OFF_XCH + 8 * GC_PARTS * GC_BM;
+    static constexpr int OFF_RD = OFF_DSQ + 4 * GC_MAX_K;        // GC_MAX_K float2
+    static constexpr int OFF_XCH = OFF_RD + 8 * GC_MAX_K;        // twice [part][row] float2
+    static constexpr int BYTES = OFF_XCH + 2 * 8 * GC_PARTS * GC_BM;
+    static_assert(OFF_RD % 16 == 0 && OFF_XCH % 16 == 0, "alignment");
     static constexpr int TMEM_COLS = 3 * NP <= 64 ? 64 : 3 * NP <= 128 ? 128
                                    : 3 * NP <= 256 ? 256 : 512;
     static_assert(NP % 16 == 0 && NP <= GC_MAX_K, "MMA N");
@@ -86,6 +95,14 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[1
           "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
           "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 }
 
 // v = hi + mid + lo to 2^-24 |v| (each step's remainder is exact in FP32).
@@ -151,7 +168,7 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + L::OFF_TMEM);
     volatile int *abort = reinterpret_cast<volatile int *>(smem + L::OFF_ABORT);
     float *dsq = reinterpret_cast<float *>(smem + L::OFF_DSQ);
-    unsigned char *use = smem + L::OFF_USE;
+    float2 *rd = reinterpret_cast<float2 *>(smem + L::OFF_RD);
 
     int nU = 0;
     uint64_t umask[2] = {0ull, 0ull};
@@ -166,14 +183,18 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < k; i += GC_THREADS) {
-        const bool u = (P.usable_words[i >> 5] >> (i & 31)) & 1u;
-        use[i] = u;
-        dsq[i] = u ? sqrtf(P.G32[i * k + i]) : 1.0f;
+    // sqrt(G_ii); its reciprocal with, where the column is not usable, the
+    // infinity that takes the column out of a minimum. In range: the
+    // reciprocals' products decide the membership (below).
+    bool dr = true;
+    for (int i = tid; i < NP; i += GC_THREADS) {
+        const bool u = i < k && ((P.usable_words[i >> 5] >> (i & 31)) & 1u);
+        const float d = u ? sqrtf(P.G32[i * k + i]) : 1.0f;
+        dr = dr && d >= 0x1p-40f && d <= 0x1p40f;
+        dsq[i] = d;
+        rd[i] = make_float2(1.0f / d, u ? 0.0f : INFINITY);
     }
-    // A operand tiles: zero (the columns past NP stay zero).
-    for (int e = tid; e < 2 * NKB * L::A_TILE / 16; e += GC_THREADS)
-        reinterpret_cast<uint4 *>(smem + L::OFF_AHI)[e] = make_uint4(0, 0, 0, 0);
+    const bool scales_ok = __syncthreads_and(dr);
     // B operands: row n (the output index i), 16-byte chunk c along K (the
     // contraction index j): M[n][j] 2-way, G[n][j] 3-way, zero past k.
     for (int e = tid; e < NP * NKB * 8; e += GC_THREADS) {
@@ -233,6 +254,8 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
         for (int kb = 0; kb < NKB; ++kb)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
+                if (4 * kb + kk >= NP / 16)   // (columns past NP are zero)
+                    continue;
                 const uint64_t oa = kb * A16 + (uint64_t)(kk * 2);
                 const uint64_t ob = kb * B16 + (uint64_t)(kk * 2);
                 const uint32_t acc = (kb | kk) ? 1u : 0u;
@@ -264,8 +287,11 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
         const uint32_t tq = tmem + ((uint32_t)(quarter * 32) << 16);
         constexpr int NCH = NP / 16;                       // 16-column chunks
         constexpr int MYCH = (NCH + GC_PARTS - 1) / GC_PARTS;   // chunks per part (at most)
-        int *xok = reinterpret_cast<int *>(smem + L::OFF_XCH);        // [part][row]
-        float *xmx = reinterpret_cast<float *>(smem + L::OFF_XCH + 4 * GC_PARTS * GC_BM);
+        float2 *xch = reinterpret_cast<float2 *>(smem + L::OFF_XCH);
+        uint32_t xph = 0;
+        auto quarter_sync = [&] {
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + quarter), "n"(GC_PARTS * 32) : "memory");
+        };
         unsigned char *arow_hi = smem + L::OFF_AHI, *arow_lo = smem + L::OFF_ALO;
         auto put_a = [&](int c8, const uint4 &h, const uint4 &l) {
             const uint32_t off = (uint32_t)((c8 >> 3) * L::A_TILE) + sw128_off(rl, c8 & 7);
@@ -283,107 +309,145 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                 if (c < k && (((c < 64 ? umask[0] : umask[1]) >> (c & 63)) & 1ull))
                     mymask |= 1u << (16 * m + i);
             }
+        mymask = __reduce_or_sync(FULL, mymask);   // (the same in the whole warp)
         auto use_mi = [&](int m, int i) { return (mymask >> (16 * m + i)) & 1u; };
-        // The parts' partial results of one decision: AND of the flags, max of
-        // the values (every part gets the same combined result).
-        auto combine = [&](int okp, float vp, int &ok, float &v) {
-            xok[part * GC_BM + rl] = okp;
-            xmx[part * GC_BM + rl] = vp;
-            asm volatile("bar.sync 1, %0;" ::"r"(GC_PARTS * GC_BM) : "memory");
-            ok = 1;
-            v = 0.0f;
+        // The parts' partial results of one decision: max and min over the
+        // row, ok where no part gave the max a sign (every part gets the same
+        // result). A barrier of the four warps that share the rows; two sets
+        // of slots in turn, so that one barrier orders the reads and the
+        // writes after the next.
+        auto combine = [&](float mxp, float mnp, float &mx, float &mn) -> bool {
+            float2 *x = xch + (xph & 1u) * (GC_PARTS * GC_BM);
+            ++xph;
+            x[part * GC_BM + rl] = make_float2(mxp, mnp);
+            quarter_sync();
+            uint32_t sgn = 0;
+            mx = 0.0f;
+            mn = INFINITY;
 #pragma unroll
             for (int q = 0; q < GC_PARTS; ++q) {
-                ok &= xok[q * GC_BM + rl];
-                v = fmaxf(v, xmx[q * GC_BM + rl]);
+                const float2 v = x[q * GC_BM + rl];
+                sgn |= __float_as_uint(v.x);
+                mx = fmaxf(mx, fabsf(v.x));
+                mn = fminf(mn, v.y);
             }
-            asm volatile("bar.sync 1, %0;" ::"r"(GC_PARTS * GC_BM) : "memory");
+            return !(sgn >> 31);
         };
-        unsigned long long st_rhs = 0, st_rounds = 0, st_max = 0, st_nf = 0, pending = 0;
+        uint32_t st_rhs = 0, st_nf = 0, pending = 0;   // (at most one a tile and thread)
+        const int rounds = P.pin ? 0 : 1;
         uint32_t ph = 0;
         bool dead = false;   // a wait of this warp timed out: only mark from now on
         // Rows of B and X start on 16 bytes when k is a multiple of 4 (the
         // bases come from the allocator, 256-byte aligned, checked here).
         const bool vec4 = (k & 3) == 0 &&
                           ((reinterpret_cast<uintptr_t>(P.B) | reinterpret_cast<uintptr_t>(P.X)) & 15) == 0;
+        // This part's columns of a tile's right-hand sides, in registers
+        // (16-byte loads when the rows are 16-byte aligned: scalar loads flood
+        // the load queue).
+        float g[MYCH][16];
+        auto relu = [](float x) { return x > 0.0f ? x : 0.0f; };   // (a NaN gives 0)
+        auto load_g = [&](int64_t t) {
+            const int64_t j = t * GC_BM + rl;
+            const bool live = j < P.nrhs;
+            const float *row = P.B + (live ? j : 0) * k;
+#pragma unroll
+            for (int m = 0; m < MYCH; ++m)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int c = 16 * (part + GC_PARTS * m) + 4 * q;
+                    if (vec4) {
+                        const float4 v = live && c < k ? *reinterpret_cast<const float4 *>(row + c)
+                                                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        g[m][4 * q] = v.x;
+                        g[m][4 * q + 1] = v.y;
+                        g[m][4 * q + 2] = v.z;
+                        g[m][4 * q + 3] = v.w;
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            g[m][4 * q + i] = live && c + i < k ? row[c + i] : 0.0f;
+                    }
+                }
+        };
+        load_g(blockIdx.x);
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
             const int64_t j = t * GC_BM + rl;
             const bool live = j < P.nrhs;
-            // This part's columns of the right-hand side, in registers (16-byte
-            // loads when the rows are 16-byte aligned: scalar loads flood the
-            // load queue).
-            float g[MYCH][16];
-            {
-                const float *row = P.B + (live ? j : 0) * k;
-#pragma unroll
-                for (int m = 0; m < MYCH; ++m)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int c = 16 * (part + GC_PARTS * m) + 4 * q;
-                        if (vec4) {
-                            const float4 v = live && c < k
-                                                 ? *reinterpret_cast<const float4 *>(row + c)
-                                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                            g[m][4 * q] = v.x;
-                            g[m][4 * q + 1] = v.y;
-                            g[m][4 * q + 2] = v.z;
-                            g[m][4 * q + 3] = v.w;
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                g[m][4 * q + i] = live && c + i < k ? row[c + i] : 0.0f;
-                        }
-                    }
-            }
             // Membership: the first candidate partition is U (the test of the
-            // SIMT pass and of the per-warp kernel, from the combined max).
-            int member = 0;
+            // SIMT pass and of the per-warp kernel: every usable g_i above
+            // FEAS_TOL32 max_c |g_c| / d_c times d_i). The products g_i (1 /
+            // d_i) stand within 2^-22 of the quotients, and the test's own
+            // roundings within as much of its exact value, so where the
+            // least product is further than 2^-19 from the bound they decide
+            // alike; elsewhere, and where scales near the ends of the range
+            // could round further, the quotients decide. (28 divisions per
+            // thread and tile otherwise: a third of the instructions.)
+            int member;
             {
-                int okp = 1;
-                float gmp = 0.0f;
+                float fsum = 0.0f, mxp = 0.0f, mnp = INFINITY;
 #pragma unroll
-                for (int m = 0; m < MYCH; ++m)
+                for (int m = 0; m < MYCH; ++m) {
+                    const int c16 = part + GC_PARTS * m;
+                    if (c16 >= NCH)
+                        continue;   // warp-uniform
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int c = 16 * (part + GC_PARTS * m) + i;
-                        if (c < k) {
-                            okp &= isfinite(g[m][i]) ? 1 : 0;
-                            gmp = fmaxf(gmp, fabsf(g[m][i]) / dsq[c]);
-                        }
+                    for (int i = 0; i < 16; i += 2) {
+                        const float4 r = *reinterpret_cast<const float4 *>(rd + 16 * c16 + i);
+                        fsum = __fmaf_rn(g[m][i], 0.0f, fsum);   // NaN from any Inf or NaN
+                        fsum = __fmaf_rn(g[m][i + 1], 0.0f, fsum);
+                        mxp = fmaxf(mxp, fmaxf(fabsf(g[m][i] * r.x), fabsf(g[m][i + 1] * r.z)));
+                        mnp = fminf(mnp, fminf(__fmaf_rn(g[m][i], r.x, r.y),
+                                               __fmaf_rn(g[m][i + 1], r.z, r.w)));
                     }
-                int ok;
-                float gmax;
-                combine(okp, gmp, ok, gmax);
-                ok = ok && live && nU > 0;
-                int inp = 1;
-                if (ok) {
-                    if (P.pin) {
-                        if (part == 0)
-                            for (int w = 0; w < P.nwords; ++w)
-                                if ((P.pin[j * P.nwords + w] & umask[w]) != umask[w])
-                                    inp = 0;
-                    } else if (P.max_rounds >= 1) {
+                }
+                const bool okp = fsum == 0.0f;
+                // The last tile's results are out of the A tiles before the
+                // exchange lets this one's right-hand sides into them.
+                if (part == 0 && lane == 0)
+                    bulk_wait_read();
+                float mx, mn;
+                const bool ok = combine(okp ? mxp : -1.0f, mnp, mx, mn) && live && nU > 0;
+                if (P.pin) {
+                    bool inp = ok;
+                    if (ok)
+                        for (int w = 0; w < P.nwords; ++w)
+                            if ((P.pin[j * P.nwords + w] & umask[w]) != umask[w])
+                                inp = false;
+                    member = inp;
+                } else if (P.max_rounds < 1) {
+                    member = 0;
+                } else {
+                    const float bound = FEAS_TOL32 * mx;
+                    const bool far = scales_ok && mx >= 0x1p-60f && mx <= 0x1p60f &&
+                                     fabsf(mn - bound) > 0x1p-19f * bound;
+                    member = ok && mn > bound;
+                    if (__any_sync(FULL, ok && !far)) {   // (the same in the four warps)
+                        float gmp = 0.0f;
+#pragma unroll
+                        for (int m = 0; m < MYCH; ++m)
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                const int c = 16 * (part + GC_PARTS * m) + i;
+                                if (c < k)
+                                    gmp = fmaxf(gmp, fabsf(g[m][i]) / dsq[c]);
+                            }
+                        float gmax, unused;
+                        combine(gmp, 0.0f, gmax, unused);
                         const float ytol = FEAS_TOL32 * gmax;
+                        bool inp = true;
 #pragma unroll
                         for (int m = 0; m < MYCH; ++m)
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
                                 const int c = 16 * (part + GC_PARTS * m) + i;
                                 if (use_mi(m, i) && !(-g[m][i] < -ytol * dsq[c]))
-                                    inp = 0;
+                                    inp = false;
                             }
-                    } else {
-                        inp = 0;
+                        const bool all_in = combine(inp ? 0.0f : -1.0f, 0.0f, gmax, unused);
+                        member = ok && all_in;
                     }
                 }
-                int all_in;
-                float unused;
-                combine(inp, 0.0f, all_in, unused);
-                member = ok && all_in;
             }
-            if (member && part == 0)   // until its solution overwrites it
-                reinterpret_cast<uint32_t *>(P.X)[j * k] = GROUP_PENDING;
-            bool solved = false;
             if (!dead) {
                 // Step 1: A = g.
 #pragma unroll
@@ -426,7 +490,6 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                         float v[8], sm[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int c = 16 * c16 + 8 * h8 + i;
                             v[i] = use_mi(m, 8 * h8 + i) ? __uint_as_float(raw[8 * h8 + i]) + 0.0f
                                                          : 0.0f;
                         }
@@ -461,7 +524,6 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                         float v[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int c = 16 * c16 + 8 * h8 + i;
                             v[i] = member && use_mi(m, 8 * h8 + i)
                                        ? g[m][8 * h8 + i] - __uint_as_float(raw[8 * h8 + i])
                                        : 0.0f;
@@ -476,14 +538,18 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                 mbar_arrive(bar_a);
                 if (tid == 0)
                     issue(2);
+            }
+            // The next tile's right-hand sides, while the last product runs and
+            // this tile's results go out (g is not read again in this tile).
+            load_g(t + gridDim.x);
+            if (!dead) {
                 // Step 4: x1 = x0' + M r, the sign test, the outputs.
                 dead = !__all_sync(FULL, mbar_wait(bar_d, ph & 1u, abort));
                 ++ph;
             }
-            // The combines below are block-level (named barrier): every part
-            // takes part in them, dead or not.
+            // The exchanges below take every warp, dead or not.
             float x1[MYCH][16];
-            float xmp = 0.0f;
+            float xmp = 0.0f, xnp = 0.0f;
             if (!dead) {
                 tc_fence_after();
 #pragma unroll
@@ -495,19 +561,23 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                             x1[m][i] = 0.0f;
                         continue;
                     }
-                    uint32_t a0[16], a2[16];
-                    tmem_ld16_nowait(tq + (uint32_t)(16 * c16), a0);
-                    tmem_ld16_nowait(tq + (uint32_t)(2 * NP + 16 * c16), a2);
-                    tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int c = 16 * c16 + i;
-                        const float x = use_mi(m, i)
-                                            ? __uint_as_float(a0[i]) + (__uint_as_float(a2[i]) + 0.0f)
-                                            : 0.0f;
-                        x1[m][i] = x;
-                        if (use_mi(m, i))
-                            xmp = fmaxf(xmp, fabsf(x) * dsq[c]);
+                    for (int h8 = 0; h8 < 2; ++h8) {   // (16 columns at once spill)
+                        uint32_t a0[8], a2[8];
+                        tmem_ld8_nowait(tq + (uint32_t)(16 * c16 + 8 * h8), a0);
+                        tmem_ld8_nowait(tq + (uint32_t)(2 * NP + 16 * c16 + 8 * h8), a2);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int ci = 8 * h8 + i;
+                            const float x = use_mi(m, ci) ? __uint_as_float(a0[i]) +
+                                                                (__uint_as_float(a2[i]) + 0.0f)
+                                                          : 0.0f;
+                            x1[m][ci] = x;
+                            const float xd = x * dsq[16 * c16 + ci];   // (not usable: 0)
+                            xmp = fmaxf(xmp, fabsf(xd));
+                            xnp = fminf(xnp, xd);
+                        }
                     }
                 }
                 tc_fence_before();   // the accumulators are read before the next tile's MMAs
@@ -518,49 +588,68 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                     for (int i = 0; i < 16; ++i)
                         x1[m][i] = 0.0f;
             }
-            int okall;
-            float xm;
-            combine(dead ? 0 : 1, xmp, okall, xm);
-            const float xtol = FEAS_TOL32 * xm;
-            int feasp = 1, finp = 1;
+            float xm, xn;
+            const bool okall = combine(dead ? -1.0f : xmp, xnp, xm, xn);
+            const bool feasible = !(xn < -(FEAS_TOL32 * xm));
+            bool fin = true;
+            if (__any_sync(FULL, isinf(xm))) {   // (no x is infinite otherwise; the same in the four warps)
+                float big = 0.0f, unused;
 #pragma unroll
-            for (int m = 0; m < MYCH; ++m)
+                for (int m = 0; m < MYCH; ++m)
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int c = 16 * (part + GC_PARTS * m) + i;
-                    if (use_mi(m, i) && x1[m][i] * dsq[c] < -xtol)
-                        feasp = 0;
-                    if (c < k && !isfinite(x1[m][i] > 0.0f ? x1[m][i] : 0.0f))
-                        finp = 0;
-                }
-            int feasible;
-            float fin_f;
-            combine(feasp, finp ? 0.0f : 1.0f, feasible, fin_f);
+                    for (int i = 0; i < 16; ++i)
+                        big = fmaxf(big, x1[m][i]);
+                combine(big, 0.0f, big, unused);
+                fin = !isinf(big);
+            }
             const bool keep = okall && member && feasible;
-            if (keep) {
+            if (vec4 && __all_sync(FULL, keep)) {   // (the same in the four warps)
+                // The quarter's 32 rows are one piece of X: through the rows'
+                // part of the A tiles (every product of this tile has read
+                // them), 4 KB of each in turn, and out in bulk copies.
+#pragma unroll
+                for (int m = 0; m < MYCH; ++m)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int c = 16 * (part + GC_PARTS * m) + 4 * q;
+                        const uint32_t o = (uint32_t)(lane * k + c) * 4u;
+                        if (c < k)
+                            *reinterpret_cast<float4 *>(arow_hi + (o >> 12) * L::A_TILE +
+                                                        quarter * 4096 + (o & 4095u)) =
+                                make_float4(relu(x1[m][4 * q]), relu(x1[m][4 * q + 1]),
+                                            relu(x1[m][4 * q + 2]), relu(x1[m][4 * q + 3]));
+                    }
+                fence_proxy_async();
+                quarter_sync();
+                if (part == 0 && lane == 0) {
+                    float *x = P.X + (t * GC_BM + quarter * 32) * k;
+                    for (uint32_t o = 0; o < 128u * (uint32_t)k; o += 4096u)
+                        bulk_store(x + o / 4, sbase + L::OFF_AHI + (o >> 12) * L::A_TILE + quarter * 4096,
+                                   min(128u * (uint32_t)k - o, 4096u));
+                    bulk_commit();
+                }
+            } else if (keep) {
                 float *xr = P.X + j * k;
 #pragma unroll
                 for (int m = 0; m < MYCH; ++m)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const int c = 16 * (part + GC_PARTS * m) + 4 * q;
-                        float v[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            v[i] = x1[m][4 * q + i] > 0.0f ? x1[m][4 * q + i] : 0.0f;
                         if (vec4) {
                             if (c < k)
-                                *reinterpret_cast<float4 *>(xr + c) = make_float4(v[0], v[1], v[2], v[3]);
+                                *reinterpret_cast<float4 *>(xr + c) =
+                                    make_float4(relu(x1[m][4 * q]), relu(x1[m][4 * q + 1]),
+                                                relu(x1[m][4 * q + 2]), relu(x1[m][4 * q + 3]));
                         } else {
 #pragma unroll
                             for (int i = 0; i < 4; ++i)
                                 if (c + i < k)
-                                    xr[c + i] = v[i];
+                                    xr[c + i] = relu(x1[m][4 * q + i]);
                         }
                     }
+            }
+            if (keep) {
                 if (part == 0) {
-                    const bool fin = fin_f == 0.0f;
-                    const int rounds = P.pin ? 0 : 1;
                     if (P.pout)
                         for (int w = 0; w < P.nwords; ++w)
                             P.pout[j * P.nwords + w] = umask[w];
@@ -569,22 +658,21 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                     if (P.status_out)
                         P.status_out[j] = (int8_t)(fin ? NMF_OK : NMF_ERR_NONFINITE);
                     st_rhs += 1;
-                    st_rounds += rounds;
-                    if ((unsigned long long)rounds > st_max)
-                        st_max = (unsigned long long)rounds;
                     st_nf += fin ? 0 : 1;
                 }
-                solved = true;
             }
-            // Members not solved keep their mark.
-            if (part == 0 && live && !solved)
+            // The others go to the per-warp kernel, members with their mark.
+            if (part == 0 && live && !keep) {
+                if (member)
+                    reinterpret_cast<uint32_t *>(P.X)[j * k] = GROUP_PENDING;
                 pending += 1;
+            }
         }
+        if (part == 0 && lane == 0)
+            bulk_wait_all();
         for (int o = 16; o > 0; o >>= 1) {
             pending += __shfl_xor_sync(FULL, pending, o);
             st_rhs += __shfl_xor_sync(FULL, st_rhs, o);
-            st_rounds += __shfl_xor_sync(FULL, st_rounds, o);
-            st_max = max(st_max, __shfl_xor_sync(FULL, st_max, o));
             st_nf += __shfl_xor_sync(FULL, st_nf, o);
         }
         if (lane == 0) {
@@ -592,8 +680,8 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
                 atomicAdd(&P.counters[CNT_PENDING], pending);
             if (st_rhs) {
                 atomicAdd(&P.stats->rhs, st_rhs);
-                atomicAdd(&P.stats->rounds, st_rounds);
-                atomicMax(&P.stats->max_rounds, st_max);
+                atomicAdd(&P.stats->rounds, (unsigned long long)(rounds * st_rhs));
+                atomicMax(&P.stats->max_rounds, (unsigned long long)rounds);
                 if (st_nf)
                     atomicAdd(&P.stats->nonfinite, st_nf);
             }

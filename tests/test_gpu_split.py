@@ -73,3 +73,58 @@ def test_spmm_small_and_streamed_factors(nmf, cols, k):
     # n sequential FMAs: at most n roundings of the running sum.
     n = rp.diff().clamp_min(1).double()[:, None]
     assert ((out.double() - ref).abs() <= n * 2.0 ** -24 * size).all()
+
+
+# The tensor-core group pass against the per-warp solves: parts of a 32-row
+# quarter and a 128-row tile, more tiles than SMs, rows whose stores are not
+# 16-byte aligned (k = 65, 111), first tests at and next to their bound, zero,
+# non-finite and far-scaled rows, and scales at which quotients decide.
+@pytest.mark.parametrize("nrhs", [1, 33, 300, 152 * 128 + 97])
+@pytest.mark.parametrize("k,scale,warm", [(4, 0, False), (65, 0, False), (96, 45, False),
+                                          (111, 0, True), (112, 0, False)])
+def test_bpp_tensor_group_edges(nmf, nrhs, k, scale, warm):
+    rng = np.random.default_rng(nrhs + k)
+    f4 = np.float32
+    d = np.exp2(scale * (np.arange(k) % 2 * 2 - 1)).astype(f4)
+    # An M-matrix: a right-hand side >= 0 has a solution >= 0, whichever
+    # entries the first test takes; the rounds tell what it took.
+    G = (np.eye(k) - 0.25 * (np.eye(k, k=1) + np.eye(k, k=-1))) * d[:, None] * d
+    B = (rng.uniform(0.1, 1.0, (nrhs, k)) * d).astype(f4)
+    kind = np.where(np.arange(nrhs) // 32 % 2 == 1, rng.integers(0, 10, nrhs), 0)
+    kind[-1] = 1
+    at = rng.integers(0, k, nrhs)
+    for j in range(nrhs):
+        i = at[j]
+        if 1 <= kind[j] <= 3:
+            rest = (np.arange(k) != i)
+            gmax = (np.abs(B[j]) / d)[rest].max()
+            bound = f4(f4(2.0 ** -20) * gmax) * d[i]
+            B[j, i] = [bound, np.nextafter(bound, f4(np.inf)), np.nextafter(bound, f4(0))][kind[j] - 1]
+        elif kind[j] == 4:
+            B[j] = 0
+        elif kind[j] == 5:
+            B[j, i] = np.nan if j % 2 else np.inf
+        elif kind[j] in (6, 7):
+            B[j] *= f4(2.0 ** ((-70 if kind[j] == 6 else 70) if scale == 0 else 0))
+        elif kind[j] == 8:
+            B[j, i] = -B[j, i]
+    Gd, Bd = torch.from_numpy(G.astype(np.float64)).cuda(), torch.from_numpy(B).cuda()
+    pin = nmf.bool_to_passive(torch.ones(nrhs, k, dtype=torch.bool)).cuda() if warm else None
+    old = nmf.nmf_nls_bpp_get_shape(k)
+    out = []
+    try:
+        for group in (0, 2):
+            nmf.nmf_nls_bpp_set_shape(k, 8, 8, group)
+            out.append(nmf.nmf_nls_bpp(Gd, Bd, pin))
+    finally:
+        nmf.nmf_nls_bpp_set_shape(k, *old)
+    for name in ("passive", "rounds", "status"):
+        assert torch.equal(out[0][name], out[1][name]), name
+    ok = (out[0]["status"] == 0).cpu()
+    assert torch.equal(ok, torch.from_numpy(kind != 5))
+    x0, x2 = (o["X"].double().cpu()[ok] * torch.from_numpy(d).double() for o in out)
+    # Rows of |G| sum to 1.5 in these scales and rows of its inverse to 2 at
+    # most: the residual's accumulations (five per 16 columns, truncated to
+    # 2^-23, and a dozen roundings on either side) reach x three times over.
+    tol = 3 * (5 * -(-k // 16) + 16) * 2.0 ** -23
+    assert ((x0 - x2).abs() <= tol * x0.abs().amax(1, keepdim=True)).all()
