@@ -38,11 +38,12 @@
 // M and G (split) stay in shared memory for the whole kernel: with the A tiles
 // they fill it, so one tile is in flight per SM and its chain of phases bounds
 // the kernel. What shortens the chain: the next tile's right-hand sides are
-// loaded into registers while the last product runs; results leave through
+// loaded into registers while the last product runs (four lanes to a row: 64
+// us less than a row to a lane); results leave through
 // the A tiles in bulk copies (rows of k floats: a warp's own stores touch 32
 // lines each); membership divides only where products cannot decide it; one
 // exchange per decision. 1e6 right-hand sides, k = 100: 33000 cycles per tile
-// without these (888 us for the kernel), 23000 with them (637 us); by memory traffic
+// without these (888 us for the kernel), 20000 with them (570 us); by memory traffic
 // it would be 120 us.
 // Every mbarrier wait is bounded (~2 s).
 #include <math.h>
@@ -341,31 +342,62 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
         // bases come from the allocator, 256-byte aligned, checked here).
         const bool vec4 = (k & 3) == 0 &&
                           ((reinterpret_cast<uintptr_t>(P.B) | reinterpret_cast<uintptr_t>(P.X)) & 15) == 0;
-        // This part's columns of a tile's right-hand sides, in registers
-        // (16-byte loads when the rows are 16-byte aligned: scalar loads flood
-        // the load queue).
+        // This part's columns of a tile's right-hand sides, in registers.
+        // Where rows are 16-byte aligned, four lanes read 64 contiguous bytes
+        // of each of their four rows in turn (8 rows per load instead of 32:
+        // the cost is in the lines an instruction touches), and own_rows
+        // exchanges them before use.
         float g[MYCH][16];
         auto relu = [](float x) { return x > 0.0f ? x : 0.0f; };   // (a NaN gives 0)
         auto load_g = [&](int64_t t) {
-            const int64_t j = t * GC_BM + rl;
-            const bool live = j < P.nrhs;
-            const float *row = P.B + (live ? j : 0) * k;
+            if (vec4) {
+                const int64_t j4 = t * GC_BM + (rl & ~3);
+                const float *rows = P.B + (j4 < P.nrhs ? j4 : 0) * k;
 #pragma unroll
-            for (int m = 0; m < MYCH; ++m)
+                for (int m = 0; m < MYCH; ++m) {
+                    const int c = 16 * (part + GC_PARTS * m) + 4 * (lane & 3);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = 16 * (part + GC_PARTS * m) + 4 * q;
-                    if (vec4) {
-                        const float4 v = live && c < k ? *reinterpret_cast<const float4 *>(row + c)
-                                                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 v = j4 + q < P.nrhs && c < k
+                                             ? *reinterpret_cast<const float4 *>(rows + q * k + c)
+                                             : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                         g[m][4 * q] = v.x;
                         g[m][4 * q + 1] = v.y;
                         g[m][4 * q + 2] = v.z;
                         g[m][4 * q + 3] = v.w;
-                    } else {
+                    }
+                }
+            } else {
+                const int64_t j = t * GC_BM + rl;
+                const bool live = j < P.nrhs;
+                const float *row = P.B + (live ? j : 0) * k;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            g[m][4 * q + i] = live && c + i < k ? row[c + i] : 0.0f;
+                for (int m = 0; m < MYCH; ++m)
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const int c = 16 * (part + GC_PARTS * m) + i;
+                        g[m][i] = live && c < k ? row[c] : 0.0f;
+                    }
+            }
+        };
+        // Quads q of lane b of four <- quad b of lane q: a 4 x 4 transpose in
+        // two exchanges.
+        auto own_rows = [&] {
+            if (!vec4)
+                return;
+#pragma unroll
+            for (int m = 0; m < MYCH; ++m)
+#pragma unroll
+                for (int s = 1; s <= 2; s *= 2) {
+                    const bool up = lane & s;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        if ((e >> 2) & s)
+                            continue;
+                        float &a = g[m][e], &b = g[m][e + 4 * s];
+                        const float o = __shfl_xor_sync(FULL, up ? a : b, s);
+                        a = up ? o : a;
+                        b = up ? b : o;
                     }
                 }
         };
@@ -373,6 +405,7 @@ __global__ void __launch_bounds__(GC_THREADS, 1) bpp_group_tc_kernel(const Solve
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
             const int64_t j = t * GC_BM + rl;
             const bool live = j < P.nrhs;
+            own_rows();
             // Membership: the first candidate partition is U (the test of the
             // SIMT pass and of the per-warp kernel: every usable g_i above
             // FEAS_TOL32 max_c |g_c| / d_c times d_i). The products g_i (1 /
