@@ -10,9 +10,10 @@
 // indices (x_i < 0 on F, y_i < 0 off F) across until Eq. 4 holds.
 //
 // GPU design (differs from the paper's column grouping; same result):
-//  * bpp_prep_kernel (one CTA, FP64) factors the usable part of G once per
-//    half-step (G = L L^T; indices with G_ii <= 0 are never passive), forms
-//    M = G^{-1} and the condition number cond_1(S G S) = ||S G S||_1
+//  * bpp_prep_kernel (one CTA, or a cluster of eight where k is large and
+//    nothing runs beside it; FP64) turns the usable part of G into M = G^{-1}
+//    once per half-step by symmetric Gauss-Jordan sweeps in registers (indices
+//    with G_ii <= 0 are never passive), and forms the condition number cond_1(S G S) = ||S G S||_1
 //    ||S^-1 M S^-1||_1 of G with its diagonal scaled to one (S = diag(G)^-1/2),
 //    and picks the arithmetic of the solves: FP32 when it is <= 1e4 (mode 0),
 //    FP64 otherwise (mode 1), FP64 without M when G is numerically singular
@@ -28,7 +29,7 @@
 //      direct      G_FF x_F = g_F                          (|F| x |F|)
 //      complement  M_AA y_A = -u_A,  x_F = u_F + M_FA y_A  (|A| x |A|)
 //    (the second follows from G x = g + y with y supported on A and x_A = 0),
-//    by a warp-cooperative Cholesky in shared memory with shuffle-broadcast
+//    by a warp-cooperative factorisation with shuffle-broadcast
 //    substitutions. Cost per round O(min(|F|,|A|)^3 + k |F|) instead of
 //    O(|F|^3). bpp_solve32_kernel (bpp32.cu) runs mode 0: it refines once
 //    (residual g_F - G_FF x_F solved through the same factor: the explicit

@@ -229,7 +229,7 @@ nmf_status launch_bpp(int k, int64_t nrhs, const double *G, const float *B, floa
                       const uint64_t *passive_in, uint64_t *passive_out, int32_t *rounds_out,
                       int8_t *status_out, int max_rounds, void *work, BppStats *stats_dev,
                       cudaStream_t s, uint64_t *predict = nullptr);
-// The two halves of launch_bpp: the per-Gram preparation (factor, inverse,
+// The two halves of launch_bpp: the per-Gram preparation (inverse, condition,
 // arithmetic mode), then the solves. A prep must complete before its solves
 // and must not overlap another half-step's prep or solves on the same work.
 // alone: no other kernel runs beside it (a large preparation then takes a

@@ -14,8 +14,8 @@
 // owning rows 2 l and 2 l + 1; the coordinates are taken in blocks of 8. For
 // a block, the sums over the entries outside it, sum_l G_li x_l, are a small
 // matrix product (the lane's two rows are the halves of packed FP32x2 FMAs, G
-// is staged with every value twice as their other operand); HALS then takes the block's coordinates in
-// turn, adding each new value to the sums still open. Every sum consists of
+// is staged with every value twice as their other operand); HALS then takes the
+// block's coordinates in turn, adding each new value to the sums still open. Every sum consists of
 // the terms of its own definition: keeping x G and adding d times row i of G
 // after each change would save the products but loses digits. HALS often
 // drives whole columns to zero, and the large steps d = -x_i leave the updated
