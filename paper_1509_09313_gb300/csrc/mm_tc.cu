@@ -414,6 +414,11 @@ __global__ void __launch_bounds__(TcLayout<N, OBJ>::THREADS, 1)
                     fs = t;
                 }
                 tc_fence_before();
+                // These reads of the stage come before the bulk copies into it
+                // only through a proxy fence: where this warp is the last to
+                // release the stage, the next tile's bytes arrived in the
+                // values being read (one objective in 400 at 4000 x 2000).
+                fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(obj_empty(b1));

@@ -128,3 +128,21 @@ def test_bpp_tensor_group_edges(nmf, nrhs, k, scale, warm):
     # 2^-23, and a dozen roundings on either side) reach x three times over.
     tol = 3 * (5 * -(-k // 16) + 16) * 2.0 ** -23
     assert ((x0 - x2).abs() <= tol * x0.abs().amax(1, keepdim=True)).all()
+
+
+# The tensor-core pass with the objective, its last wave shared out: the
+# residual warps are the last to release a stage of the ring, which the next
+# copies overwrite at once. The same run must give the same bits every time.
+@pytest.mark.parametrize("m,n,k", [(4000, 2000, 50), (2500, 3100, 20)])
+def test_objective_pass_repeats_bitwise(nmf, m, n, k):
+    A = torch.from_numpy(synth.dense_planted(m, n, k, 0.05)).cuda()
+    W0, Ht0 = (torch.from_numpy(x).cuda() for x in synth.init_factors(m, n, k))
+    first = None
+    for _ in range(100):
+        h = nmf.nmf_init(A, W0.clone(), Ht0.clone(), precision="bf16x3", start="warm")
+        h.nmf_iterate(30)
+        assert h.nmf_sync() == nmf.NMF_OK
+        f = list(h.nmf_objective_history())
+        h.nmf_destroy()
+        first = first or f
+        assert f == first
