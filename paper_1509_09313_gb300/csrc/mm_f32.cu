@@ -103,9 +103,11 @@ __device__ __forceinline__ void cp_async_wait()
 __device__ __forceinline__ int clamp16(int64_t v) { return v <= 0 ? 0 : v >= 16 ? 16 : (int)v; }
 
 // A H^T: tiles 0 .. full - 1 take one CTA each, the `tiles` after them `splits`
-// CTAs each, whose stage sums go to `part`.
+// CTAs each. The first of a tile's CTAs (`first` stages) adds its stages up as
+// an unshared tile does and leaves total and compensation in `part`, the others
+// their stages' sums.
 struct F32Tail {
-    int64_t full = 0, tiles = 0;
+    int64_t full = 0, tiles = 0, first = 0;
     int splits = 1;
     float *part = nullptr;
 };
@@ -345,10 +347,10 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
                 }
             continue;
         }
-        if (shared_tile) {
-            // The stage's sums for f32_stage_kernel, [stage][tile][entry].
+        if (shared_tile && qb > 0) {
+            // The stage's sums for f32_stage_kernel, [2 + stage - first][tile][entry].
             float *dst = tail.part +
-                         ((qb / BQ + t) * tail.tiles +
+                         ((qb / BQ + t - tail.first + 2) * tail.tiles +
                           ((int64_t)blockIdx.x - tail.full) / tail.splits) * (BP * KP) + tid;
 #pragma unroll
             for (int a = 0; a < RPT; ++a)
@@ -384,6 +386,18 @@ __device__ __forceinline__ void mm_f32_body(const float *__restrict__ A, int64_t
 #pragma unroll
             for (int b = 0; b < 4; ++b)
                 cmp[a][b] = -cmp[a][b];
+    }
+
+    if (shared_tile && qb == 0) {
+        float *dst = tail.part +
+                     ((int64_t)blockIdx.x - tail.full) / tail.splits * (BP * KP) + tid;
+#pragma unroll
+        for (int a = 0; a < RPT; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                dst[(a * 4 + b) * NT] = acc[a][b];
+                dst[tail.tiles * (BP * KP) + (a * 4 + b) * NT] = cmp[a][b];
+            }
     }
 
     // Output: the compensated total rounded once, or (contraction split)
@@ -443,7 +457,7 @@ __global__ void __launch_bounds__(16 * NCG, 1)
 // The shared tiles of A H^T: out from the stages' sums, added with the Kahan
 // steps of an unshared tile in its order (bitwise its result). Entry (a, b) of
 // thread tid of the product's CTA at (4 a + b) NT + tid. Reads 4 bytes per
-// entry and stage.
+// entry and stage, but for the first CTA's.
 template <int NCG, int RPT>
 __global__ void __launch_bounds__(256)
     f32_stage_kernel(int64_t P, int64_t nst, int k, float *__restrict__ out, const F32Tail tail)
@@ -454,9 +468,9 @@ __global__ void __launch_bounds__(256)
     const int64_t stride = tail.tiles * E;
     if (e >= stride)
         return;
-    float acc = 0.0f, cmp = 0.0f;
+    float acc = tail.part[e], cmp = -tail.part[stride + e];
 #pragma unroll 16
-    for (int64_t t = 0; t < nst; ++t) {
+    for (int64_t t = 2; t < nst - tail.first + 2; ++t) {
         const float yk = tail.part[t * stride + e] - cmp;
         const float tk = acc + yk;
         cmp = (tk - acc) - yk;
@@ -589,11 +603,13 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool share = true)
         w.tail.full = tiles;
         const int64_t sms = sm_count(), left = tiles % sms, nst = cdiv(Q, bq);
         const int64_t splits = left ? std::min(sms / left, nst / 8) : 1;
-        const size_t bytes = sizeof(float) * (size_t)(left * nst * w.bp * w.kp);
+        const int64_t first = splits >= 2 ? cdiv(nst, splits) : nst;
+        const size_t bytes = sizeof(float) * (size_t)(left * (nst - first + 2) * w.bp * w.kp);
         if (share && splits >= 2 && bytes <= F32_TAIL_BYTES) {
-            w.q_per_split = cdiv(nst, splits) * bq;
+            w.q_per_split = first * bq;
             w.tail.full = tiles - left;
             w.tail.tiles = left;
+            w.tail.first = first;
             w.tail.splits = (int)cdiv(Q, w.q_per_split);
         }
     }
@@ -608,7 +624,8 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool share = true)
     if (w.splits > 1)
         w.total += al(sizeof(float) * 2 * (size_t)w.splits * (size_t)w.P * k);
     if (w.tail.tiles > 0)
-        w.total += al(sizeof(float) * (size_t)(w.tail.tiles * cdiv(Q, bq) * w.bp * w.kp));
+        w.total += al(sizeof(float) * (size_t)(w.tail.tiles * (cdiv(Q, bq) - w.tail.first + 2) *
+                                               w.bp * w.kp));
     return w;
 }
 
