@@ -61,14 +61,19 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool liv
                  : "memory");
 }
 
-// a / g rounded to nearest for finite a >= 0, g > 0 and rg = 1 / g rounded: the
-// quotient corrected by its exact remainder (Markstein 1990), with the plain
-// division where the quotient is so large or small that a step of it could
-// overflow or lose bits.
+// a / g rounded to nearest for a >= 0 (or infinite), g > 0 and rg = 1 / g rounded:
+// the quotient corrected by its exact remainder (Markstein 1990), with the plain
+// division where one of the three is so large or small that a step could
+// overflow or lose bits (1 / g is infinite up to g = 2^-128, and 0 times that a
+// NaN; the remainder of a < 1e-31 is not exact). Zero, the common numerator, is
+// its own quotient.
 __device__ __forceinline__ float quotient(float a, float g, float rg)
 {
+    constexpr float LO = 1e-30f, HI = 1e30f;
     const float q = a * rg;
-    if (a > 0.0f && !(q > 1e-30f && q < 1e30f && g > 1e-30f && g < 1e30f))
+    if (!(a > 0.0f))
+        return 0.0f;
+    if (!(a > LO && a < HI && g > LO && g < HI && q > LO && q < HI))
         return a / g;
     return fmaf(fmaf(-q, g, a), rg, q);
 }

@@ -156,3 +156,33 @@ def test_step_at_tile_edges(nmf, solver, k, rows):
     fn(dev(G, torch.float64), dev(R), Xd)
     ref = (oracle.mu if solver == "mu" else oracle.hals)(G, R, X)
     assert row_rel_err(Xd.double().cpu().numpy(), ref) <= 2e-5
+
+
+# The division of HALS's coordinate on both sides of the switch between its two
+# kernels (48 rows per SM; 152 SMs): k = 1 makes x = max(r, 0) / g of every row,
+# which the FP32 division rounds to nearest. Diagonals down to the smallest
+# subnormal (their reciprocals overflow) and up to 1e38, numerators of every size
+# and zero and negative ones; then k = 3, where a column of such a norm stands
+# beside ordinary ones and is clamped to zero.
+@pytest.mark.parametrize("rows", [7295, 7297])
+@pytest.mark.parametrize("g", [1e-45, 1e-41, 2.0 ** -129, 2.0 ** -128, 2.0 ** -126, 3e-38, 1.1e-30,
+                               7e-20, 0.3, 1.0, 3.7e8, 9e29, 1.1e30, 2.0 ** 126, 1e38, 3.4e38])
+def test_hals_quotient_is_the_rounded_one(nmf, g, rows):
+    rng = np.random.default_rng(rows)
+    r = (np.exp2(rng.uniform(-149, 127.9, rows)) * rng.choice([-1, 1, 1, 1], rows)).astype(np.float32)
+    r[::5] = 0.0
+    with np.errstate(over="ignore"):
+        r[1::7] = np.float32(g) * rng.uniform(0.5, 2.0, r[1::7].shape).astype(np.float32)
+    X = dev(rng.uniform(0, 1, (rows, 1)))
+    nmf.nmf_update_hals(dev([[g]], torch.float64), dev(r[:, None]), X)
+    with np.errstate(over="ignore"):
+        want = np.maximum(r, np.float32(0)) / np.float32(g)
+    assert np.array_equal(X.cpu().numpy()[:, 0], want)
+
+    G = np.diag([4.0, g, 2.0])
+    R = np.stack([rng.uniform(1, 2, rows), -rng.uniform(0, 1, rows), rng.uniform(1, 2, rows)], 1)
+    X = dev(rng.uniform(0, 1, (rows, 3)))
+    nmf.nmf_update_hals(dev(G, torch.float64), dev(R), X)
+    R = R.astype(np.float32)
+    want = np.stack([R[:, 0] / np.float32(4), np.zeros(rows, np.float32), R[:, 2] / np.float32(2)], 1)
+    assert np.array_equal(X.cpu().numpy(), want)
