@@ -542,6 +542,7 @@ __device__ __forceinline__ bool ldl_regs(const float *__restrict__ Src, const in
                 s[b - 1] = fmaf(-m, __shfl_sync(FULL, s[b], j), s[b]);
         }
     }
+    __syncwarp();   // ldl_solve reads the other lanes' rows (a shuffle orders no memory)
     return __all_sync(FULL, ok);
 }
 
@@ -672,6 +673,7 @@ __global__ void __launch_bounds__(S32_MAX_WARPS * 32, KW == 4 ? 1 : 2)
     __shared__ unsigned long long wst[S32_MAX_WARPS][6];   // rhs, rounds, max, fp64, nc, nf
     if (lane < 6)
         wst[warp][lane] = 0;
+    __syncwarp();
 
     for (;;) {
         unsigned long long j0 = 0;

@@ -146,3 +146,17 @@ def test_objective_pass_repeats_bitwise(nmf, m, n, k):
         h.nmf_destroy()
         first = first or f
         assert f == first
+
+
+# The lanes of a warp hand each other the factor and the statistics through
+# shared memory: the same batch must give the same bits and counts every time,
+# in systems of 1 to 32 rows.
+@pytest.mark.parametrize("k", [2, 20, 33, 48, 50, 56, 64])
+def test_bpp_warp_solves_repeat_bitwise(nmf, k):
+    G, B = synth.nls_batch(k, 20011, seed=k)
+    Gd, Bd = torch.from_numpy(G).cuda(), torch.from_numpy(B.astype(np.float32)).cuda()
+    first = nmf.nmf_nls_bpp(Gd, Bd)
+    for _ in range(30):
+        again = nmf.nmf_nls_bpp(Gd, Bd)
+        for name in ("X", "passive", "rounds", "status"):
+            assert torch.equal(first[name], again[name]), name
