@@ -241,10 +241,14 @@ extern "C" nmf_status nmf_objective_dense(const float *A, int64_t m, int64_t n, 
     if (precision == NMF_PREC_BF16X3 && k <= 64 && m > 0 && n > 0) {
         // Tensor cores: the objective rides on an A H^T pass whose product
         // goes to scratch.
-        const size_t wb = mm_tc_work_bytes(m, n, k, 0);
+        size_t wb = mm_tc_obj_work_bytes(m, n, k);
         TempBuf w(s), v(s);
-        NMF_CUDA(w.alloc(wb));
         NMF_CUDA(v.alloc(sizeof(float) * (size_t)m * k));
+        if (w.alloc(wb) != cudaSuccess) {   // not the memory for a shared last wave
+            cudaGetLastError();
+            wb = mm_tc_obj_work_bytes(m, n, k, false);
+            NMF_CUDA(w.alloc(wb));
+        }
         NMF_TRY(launch_mm_tc_obj(A, m, n, lda, Ht, k, 0, static_cast<float *>(v.p), W,
                                  static_cast<double *>(f.p), w.p, wb, s));
     } else {
@@ -706,14 +710,26 @@ extern "C" nmf_status nmf_init(nmf_handle **out, const nmf_config *cfg, const nm
             e = cudaErrorMemoryAllocation;
     }
     if (e == cudaSuccess && c.input_kind == NMF_INPUT_DENSE && c.precision == NMF_PREC_BF16X3) {
-        h->tc_work_bytes = mm_tc_work_bytes(c.m, c.n, c.k, 0);
-        const size_t b1 = mm_tc_work_bytes(c.m, c.n, c.k, 1);
-        if (b1 > h->tc_work_bytes)
-            h->tc_work_bytes = b1;
-        chk(cudaMalloc(&h->tc_work, h->tc_work_bytes ? h->tc_work_bytes : 16));
+        // Workspace of every pass; the objective's with its last wave shared
+        // out where there is the memory.
+        const size_t plain = std::max(mm_tc_work_bytes(c.m, c.n, c.k, 0),
+                                      mm_tc_work_bytes(c.m, c.n, c.k, 1));
+        auto alloc_work = [&](bool share) {
+            h->tc_work_bytes = plain;
+            if (c.k <= 64)
+                h->tc_work_bytes =
+                    std::max(plain, mm_tc_obj_work_bytes(c.m, c.n, c.k, share));
+            h->tc_work = nullptr;
+            return cudaMalloc(&h->tc_work, h->tc_work_bytes ? h->tc_work_bytes : 16);
+        };
+        if (alloc_work(true) != cudaSuccess) {
+            cudaGetLastError();
+            chk(alloc_work(false));
+        }
         // A and A^T split into BF16 hi / lo once (4 bytes per element of A
         // each): the products then need no per-call split (nor transpose).
-        // Without the memory the handle splits A on the fly in every pass.
+        // Without the memory the handle splits A on the fly in every pass; the
+        // scratch of a shared last wave is given up for them.
         auto alloc_pair = [&](void **hi, void **lo, size_t bytes) {
             if (cudaMalloc(hi, bytes) != cudaSuccess || cudaMalloc(lo, bytes) != cudaSuccess) {
                 cudaGetLastError();
@@ -722,10 +738,30 @@ extern "C" nmf_status nmf_init(nmf_handle **out, const nmf_config *cfg, const nm
                 *hi = *lo = nullptr;
             }
         };
-        if (e == cudaSuccess && !c.no_split_copies)
-            alloc_pair(&h->at_hi, &h->at_lo, mm_tc_presplit_bytes(c.n, c.m));
-        if (e == cudaSuccess && h->at_hi)
-            alloc_pair(&h->ar_hi, &h->ar_lo, mm_tc_presplit_bytes(c.m, c.n));
+        auto alloc_copies = [&]() {
+            if (!h->at_hi)
+                alloc_pair(&h->at_hi, &h->at_lo, mm_tc_presplit_bytes(c.n, c.m));
+            if (h->at_hi)
+                alloc_pair(&h->ar_hi, &h->ar_lo, mm_tc_presplit_bytes(c.m, c.n));
+        };
+        if (e == cudaSuccess && !c.no_split_copies) {
+            alloc_copies();
+            const void *at = h->at_hi;
+            if (!h->ar_hi && c.k <= 64 &&
+                h->tc_work_bytes > std::max(plain, mm_tc_obj_work_bytes(c.m, c.n, c.k, false))) {
+                cudaFree(h->tc_work);
+                chk(alloc_work(false));
+                if (e == cudaSuccess)
+                    alloc_copies();
+                if (e == cudaSuccess && !h->ar_hi && h->at_hi == at) {   // nothing gained
+                    cudaFree(h->tc_work);
+                    if (alloc_work(true) != cudaSuccess) {
+                        cudaGetLastError();
+                        chk(alloc_work(false));
+                    }
+                }
+            }
+        }
     }
     if (e == cudaSuccess && c.input_kind == NMF_INPUT_CSR) {
         chk(dalloc(&h->t_rowptr, (size_t)c.n + 1));

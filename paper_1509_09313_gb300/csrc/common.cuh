@@ -149,6 +149,10 @@ nmf_status launch_mm_tc(const float *A, int64_t m, int64_t n, int64_t lda, const
                         int k, int trans, float *out, void *work, size_t work_bytes,
                         cudaStream_t s);
 size_t mm_tc_work_bytes(int64_t m, int64_t n, int k, int trans);
+// Workspace of the pass with the objective (trans = 0, k <= 64); without the
+// memory for sharing out its last wave, the fewer bytes of share = false (same
+// results).
+size_t mm_tc_obj_work_bytes(int64_t m, int64_t n, int k, bool share = true);
 // Contraction splits (CTAs along the contraction per output tile) the plain
 // tensor-core product of this shape uses.
 int mm_tc_splits(int64_t m, int64_t n, int trans);

@@ -920,12 +920,18 @@ int choose_splits(int64_t P, int64_t Q)
 // The pass with the objective (1 CTA per SM) takes the tiles of its whole waves
 // unsplit and shares out the contraction of those left over, whose partial
 // sums are then added in the unsplit order: the products do not depend on the
-// grid (24000 x 16000, k = 50: 392 us in 188 unsplit CTAs, 258 + 11 us so).
+// grid (24000 x 16000, k = 50: 392 us in 188 unsplit CTAs, 258 + 11 us so). The
+// partial sums need scratch (4 N bytes per row and fold of a shared tile: 38 MB
+// there, an eighth of A's bytes where every tile is shared); without it (share =
+// false) or above TC_FOLD_BYTES no tile is shared, with the same results.
 struct ObjPlan {
     int full, tail, splits, kb_per_split, nfolds;
+    size_t fold_bytes;
 };
 
-ObjPlan obj_plan(int64_t P, int64_t Q)
+constexpr size_t TC_FOLD_BYTES = (size_t)512 << 20;   // most scratch for shared tiles
+
+ObjPlan obj_plan(int64_t P, int64_t Q, int N, bool share)
 {
     const int tiles = (int)cdiv(P, TC_BM), nkb = (int)cdiv(Q, TC_BK), sms = sm_count();
     ObjPlan o;
@@ -934,19 +940,22 @@ ObjPlan obj_plan(int64_t P, int64_t Q)
     o.splits = 1;
     o.kb_per_split = nkb;
     o.nfolds = nkb / TC_FOLD + 1;
+    o.fold_bytes = 0;
     const int left = tiles % sms;
     // At least two folds per CTA.
     const int splits = left ? std::min(sms / left, nkb / (2 * TC_FOLD)) : 1;
-    if (splits >= 2) {
+    const size_t bytes = sizeof(float) * (size_t)o.nfolds * left * N * TC_BM;
+    if (share && splits >= 2 && bytes <= TC_FOLD_BYTES) {
         o.full = tiles - left;
         o.tail = left;
         o.kb_per_split = (int)cdiv(cdiv(nkb, splits), TC_FOLD) * TC_FOLD;
         o.splits = (int)cdiv(nkb, o.kb_per_split);
+        o.fold_bytes = bytes;
     }
     return o;
 }
 
-TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj)
+TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj, bool share)
 {
     const int64_t P = trans ? n : m;
     const int64_t Q = trans ? m : n;
@@ -962,10 +971,10 @@ TcWork tc_work(int64_t m, int64_t n, int k, int trans, bool obj)
         off += al(2 * sizeof(__nv_bfloat16) * (size_t)Pp * 64);
     w.part_off = off;
     if (obj) {
-        const ObjPlan o = obj_plan(P > 0 ? P : 1, Q > 0 ? Q : 1);
+        const ObjPlan o = obj_plan(P > 0 ? P : 1, Q > 0 ? Q : 1, N, share);
         off += al(sizeof(double) * (size_t)(o.full + o.tail * o.splits));
         w.split_off = off;
-        off += al(sizeof(float) * (size_t)o.nfolds * (size_t)o.tail * (size_t)N * TC_BM);
+        off += al(o.fold_bytes);
         w.total = off;
         return w;
     }
@@ -986,9 +995,12 @@ int mm_tc_splits(int64_t m, int64_t n, int trans)
 
 size_t mm_tc_work_bytes(int64_t m, int64_t n, int k, int trans)
 {
-    const size_t a = tc_work(m, n, k, trans, false).total;
-    const size_t b = (trans == 0 && k <= 64) ? tc_work(m, n, k, trans, true).total : 0;
-    return a > b ? a : b;
+    return tc_work(m, n, k, trans, false, false).total;
+}
+
+size_t mm_tc_obj_work_bytes(int64_t m, int64_t n, int k, bool share)
+{
+    return tc_work(m, n, k, 0, true, share).total;
 }
 
 namespace {
@@ -1022,7 +1034,12 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
     if (presplit ? ((reinterpret_cast<uintptr_t>(at_hi) | reinterpret_cast<uintptr_t>(at_lo)) & 15)
                  : ((reinterpret_cast<uintptr_t>(A) & 15) || (lda % 4)))
         return NMF_ERR_INVALID_ARG;
-    const TcWork wl = tc_work(m, n, k, trans, obj);
+    bool share = obj;
+    TcWork wl = tc_work(m, n, k, trans, obj, share);
+    if (share && work_bytes < wl.total) {
+        share = false;
+        wl = tc_work(m, n, k, trans, obj, share);
+    }
     if (!work || work_bytes < wl.total)
         return NMF_ERR_INVALID_ARG;
     const int64_t Qp = cdiv(Q, TC_BK) * TC_BK;
@@ -1088,7 +1105,7 @@ nmf_status launch_mm_tc_impl(const float *A, int64_t m, int64_t n, int64_t lda, 
         const int splits = choose_splits(P, Q);
         const int nkb = (int)cdiv(Q, TC_BK);
         a.kb_per_split = (int)cdiv(nkb, splits);
-        const ObjPlan op = obj_plan(P, Q);
+        const ObjPlan op = obj_plan(P, Q, N, share);
         if (fuse) {
             a.kb_per_split = op.kb_per_split;
             a.full = op.full;

@@ -3,6 +3,8 @@ group-tile pass's tile width and span, and the right-hand sides a warp grabs at
 once, follow the number of right-hand sides. Every split does the same
 arithmetic per right-hand side, so a batch must give the bits its parts give.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -160,3 +162,36 @@ def test_bpp_warp_solves_repeat_bitwise(nmf, k):
         again = nmf.nmf_nls_bpp(Gd, Bd)
         for name in ("X", "passive", "rounds", "status"):
             assert torch.equal(first[name], again[name]), name
+
+
+# Device memory the tensor-core products take beside their operands. A handle's
+# scratch for a shared last wave is bounded (71 row tiles, all shared: an eighth of
+# A's bytes otherwise), and nmf_mm_dense, which forms no objective, has none of it.
+def test_shared_wave_scratch_is_bounded(nmf):
+    m, n, k = 9000, 320000, 33
+    A = torch.zeros((m, n), device="cuda")
+    W0, Ht0 = torch.rand((m, k), device="cuda"), torch.rand((n, k), device="cuda")
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    h = nmf.nmf_init(A, W0, Ht0, precision="bf16x3", split_copies=False)
+    used = before - torch.cuda.mem_get_info()[0]
+    h.nmf_destroy()
+    # Factors, right-hand sides and passive sets, both factors in BF16 halves
+    # (64 columns), the Gram's and the splits' partial sums, rounded up freely.
+    assert used <= 4 * (8 * (m + n) * k + 4 * (m + n) * 64) + (512 << 20), used
+
+
+def test_mm_dense_takes_no_objective_scratch(nmf):
+    m, n, k = 9728, 16000, 50
+    A, F = torch.rand((m, n), device="cuda"), torch.rand((n, k), device="cuda")
+    torch.cuda.synchronize()
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, high = ctypes.c_void_p(), ctypes.c_uint64(0)
+    USED_MEM_HIGH = 8
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert cu.cuMemPoolSetAttribute(pool, USED_MEM_HIGH, ctypes.byref(high)) == 0
+    nmf.nmf_mm_dense(A, F, False, "bf16x3")
+    torch.cuda.synchronize()
+    assert cu.cuMemPoolGetAttribute(pool, USED_MEM_HIGH, ctypes.byref(high)) == 0
+    # F in BF16 halves and at most four partial sums of the output.
+    assert 0 < high.value <= 4 * n * 64 + 4 * 4 * m * k + (1 << 20), high.value
