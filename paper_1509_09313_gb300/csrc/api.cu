@@ -100,7 +100,7 @@ extern "C" nmf_status nmf_mm_dense(const float *A, int64_t m, int64_t n, int64_t
         return launch_mm_tc(A, m, n, lda, F, k, trans, out, w.p, wb, s);
     }
     if (mm_f32_supported(A, lda)) {
-        size_t wb = mm_f32_work_bytes(m, n, k, trans);
+        size_t wb = mm_f32_work_bytes(m, n, k, trans, !trans && mm_f32_share_once(m, n, k));
         TempBuf w(s);
         if (w.alloc(wb) != cudaSuccess) {   // not the memory for a shared last wave
             cudaGetLastError();
@@ -241,7 +241,7 @@ extern "C" nmf_status nmf_objective_dense(const float *A, int64_t m, int64_t n, 
     if (precision == NMF_PREC_BF16X3 && k <= 64 && m > 0 && n > 0) {
         // Tensor cores: the objective rides on an A H^T pass whose product
         // goes to scratch.
-        size_t wb = mm_tc_obj_work_bytes(m, n, k);
+        size_t wb = mm_tc_obj_work_bytes(m, n, k, mm_tc_obj_share_once(m, n, k));
         TempBuf w(s), v(s);
         NMF_CUDA(v.alloc(sizeof(float) * (size_t)m * k));
         if (w.alloc(wb) != cudaSuccess) {   // not the memory for a shared last wave

@@ -138,6 +138,9 @@ nmf_status launch_mm_simt(const float *A, int64_t m, int64_t n, int64_t lda, con
 // (same results).
 bool mm_f32_supported(const float *A, int64_t lda);
 size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans, bool share = true);
+// Whether sharing pays for the mapping of its scratch within one call (A H^T);
+// a handle maps it once.
+bool mm_f32_share_once(int64_t m, int64_t n, int k);
 nmf_status launch_mm_f32(const float *A, int64_t m, int64_t n, int64_t lda, const float *F, int k,
                          int trans, float *out, const float *W, double *f_dev, void *work,
                          size_t work_bytes, cudaStream_t s);
@@ -153,6 +156,7 @@ size_t mm_tc_work_bytes(int64_t m, int64_t n, int k, int trans);
 // memory for sharing out its last wave, the fewer bytes of share = false (same
 // results).
 size_t mm_tc_obj_work_bytes(int64_t m, int64_t n, int k, bool share = true);
+bool mm_tc_obj_share_once(int64_t m, int64_t n, int k);   // (as mm_f32_share_once)
 // Contraction splits (CTAs along the contraction per output tile) the plain
 // tensor-core product of this shape uses.
 int mm_tc_splits(int64_t m, int64_t n, int trans);

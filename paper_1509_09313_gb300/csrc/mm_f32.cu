@@ -546,6 +546,7 @@ int f32_ncg(int k) { return k <= 16 ? 4 : k <= 32 ? 8 : k <= 48 ? 12 : k <= 56 ?
 constexpr int RPT0 = 8, RPT1 = 8;   // rows per thread: A H^T, A^T W
 
 constexpr size_t F32_TAIL_BYTES = (size_t)512 << 20;   // most scratch for shared tiles
+constexpr size_t F32_ONCE_BYTES = (size_t)24 << 20;    // scratch that costs one call nothing
 
 struct F32Plan {
     int ncg, kp, nch, kpt, splits;
@@ -601,8 +602,12 @@ F32Plan f32_plan(int64_t m, int64_t n, int k, int trans, bool share = true)
         // 50 ran 188 CTAs in two waves, 1.95 ms; 2000 x 1000, k = 10 ran 16,
         // 59 us, and 101 us with the objective.
         w.tail.full = tiles;
+        // Not where whole waves of narrow tiles (16 columns) run: their CTAs are
+        // small enough to share SMs, and the left-over ones run beside them
+        // (24000 x 16000, k = 10: 934 us unshared, 958 shared).
         const int64_t sms = sm_count(), left = tiles % sms, nst = cdiv(Q, bq);
-        const int64_t splits = left ? std::min(sms / left, nst / 8) : 1;
+        const int64_t splits =
+            left && (w.ncg > 4 || tiles < sms) ? std::min(sms / left, nst / 8) : 1;
         const int64_t first = splits >= 2 ? cdiv(nst, splits) : nst;
         const size_t bytes = sizeof(float) * (size_t)(left * (nst - first + 2) * w.bp * w.kp);
         if (share && splits >= 2 && bytes <= F32_TAIL_BYTES) {
@@ -685,6 +690,21 @@ nmf_status launch_ncg(const float *A, const F32Plan &w, int64_t lda, const float
 bool mm_f32_supported(const float *A, int64_t lda)
 {
     return (lda % 4) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+}
+
+// The scratch of shared tiles (128 kp floats per tile and stage) comes from the
+// stream's memory pool, which maps it afresh after every wait for the stream:
+// about 2.3 us per MB past its first 32 MB. A stage saves its own time once,
+// whatever the number of tiles, and each tile pays for its mapping: 3.4 us
+// against 0.066 us per tile at kp = 56, 1.3 against 0.038 at 32. Measured, a call
+// that is waited for, n = 16000, k = 50, shared against unshared: 38 tiles 1010 /
+// 1173 us, 50 tiles 1171 / 1188, 76 tiles 1420 / 1187; k = 24: 24 tiles 681 / 870,
+// 38 tiles 950 / 868; n = 1000, k = 50, 76 tiles (20 MB): 250 / 275.
+bool mm_f32_share_once(int64_t m, int64_t n, int k)
+{
+    const F32Plan w = f32_plan(m, n, k, 0);
+    return w.tail.tiles * (w.kp > 32 ? 3 : 6) <= sm_count() ||
+           w.total - w.split_off <= F32_ONCE_BYTES;
 }
 
 size_t mm_f32_work_bytes(int64_t m, int64_t n, int k, int trans, bool share)

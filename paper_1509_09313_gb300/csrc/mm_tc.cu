@@ -930,6 +930,7 @@ struct ObjPlan {
 };
 
 constexpr size_t TC_FOLD_BYTES = (size_t)512 << 20;   // most scratch for shared tiles
+constexpr size_t TC_ONCE_BYTES = (size_t)24 << 20;    // scratch that costs one call nothing
 
 ObjPlan obj_plan(int64_t P, int64_t Q, int N, bool share)
 {
@@ -996,6 +997,19 @@ int mm_tc_splits(int64_t m, int64_t n, int trans)
 size_t mm_tc_work_bytes(int64_t m, int64_t n, int k, int trans)
 {
     return tc_work(m, n, k, trans, false, false).total;
+}
+
+// The scratch of shared tiles (64 N bytes per tile and 64-wide K-block, mapped by
+// the stream's pool after every wait at about 2.3 us per MB past its first 32 MB)
+// against what sharing saves. Measured, a call of nmf_objective_dense, k = 50,
+// shared against unshared, n = 16000: 50 tiles 442 / 468 us, 55 tiles 488 / 470,
+// 76 tiles 580 / 456; n = 4000, 76 tiles (20 MB): 291 / 302; k = 20: 76 tiles 467 /
+// 462.
+bool mm_tc_obj_share_once(int64_t m, int64_t n, int k)
+{
+    const int N = k <= 16 ? 16 : k <= 32 ? 32 : 64;
+    const ObjPlan o = obj_plan(m, n, N, true);
+    return (int64_t)o.tail * N * 3 <= 64 * (int64_t)sm_count() || o.fold_bytes <= TC_ONCE_BYTES;
 }
 
 size_t mm_tc_obj_work_bytes(int64_t m, int64_t n, int k, bool share)

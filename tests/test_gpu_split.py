@@ -181,17 +181,57 @@ def test_shared_wave_scratch_is_bounded(nmf):
     assert used <= 4 * (8 * (m + n) * k + 4 * (m + n) * 64) + (512 << 20), used
 
 
-def test_mm_dense_takes_no_objective_scratch(nmf):
-    m, n, k = 9728, 16000, 50
-    A, F = torch.rand((m, n), device="cuda"), torch.rand((n, k), device="cuda")
+def used_memory(call):
+    """Most bytes the device's default stream-ordered pool gave out during the call."""
     torch.cuda.synchronize()
     cu = ctypes.CDLL("libcuda.so.1")
     pool, high = ctypes.c_void_p(), ctypes.c_uint64(0)
     USED_MEM_HIGH = 8
     assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
     assert cu.cuMemPoolSetAttribute(pool, USED_MEM_HIGH, ctypes.byref(high)) == 0
-    nmf.nmf_mm_dense(A, F, False, "bf16x3")
+    call()
     torch.cuda.synchronize()
     assert cu.cuMemPoolGetAttribute(pool, USED_MEM_HIGH, ctypes.byref(high)) == 0
+    assert high.value > 0
+    return high.value
+
+
+def test_mm_dense_takes_no_objective_scratch(nmf):
+    m, n, k = 9728, 16000, 50
+    A, F = torch.rand((m, n), device="cuda"), torch.rand((n, k), device="cuda")
+    used = used_memory(lambda: nmf.nmf_mm_dense(A, F, False, "bf16x3"))
     # F in BF16 halves and at most four partial sums of the output.
-    assert 0 < high.value <= 4 * n * 64 + 4 * 4 * m * k + (1 << 20), high.value
+    assert used <= 4 * n * 64 + 4 * 4 * m * k + (1 << 20), used
+
+
+# One call maps the scratch of a shared last wave afresh: it is taken only where
+# it pays (76 tiles are half a wave; 36 of 24 columns, 18 narrow ones beside a whole
+# wave). F^T, the output and, of the objective, both factors' halves remain.
+@pytest.mark.parametrize("m,k", [(9728, 50), (4608, 24), (21760, 10)])
+def test_one_call_takes_no_scratch_that_does_not_pay(nmf, m, k):
+    n = 16000
+    A, F = torch.rand((m, n), device="cuda"), torch.rand((n, k), device="cuda")
+    W = torch.rand((m, k), device="cuda")
+    few = 4 * n * 64 + 4 * m * k + (1 << 20)
+    used = used_memory(lambda: nmf.nmf_mm_dense(A, F, False, "fp32"))
+    assert used <= few, used
+    if k == 50:
+        used = used_memory(lambda: nmf.nmf_objective_dense(A, W, F, "bf16x3"))
+        assert used <= few + 4 * m * 64, used
+
+
+# A H^T in FP32 with the last wave's tiles shared out, alone or behind a whole wave
+# (152 tiles of 128 rows), against the same rows multiplied alone or unshared: a
+# row's sums do not depend on the grid, to the bit. Column chunks of every width,
+# two chunks (k = 100), a contraction that ends inside a stage; 38 tiles are shared
+# by four CTAs each, 18 by eight, 77 by none.
+@pytest.mark.parametrize("k", [10, 24, 40, 50, 64, 100])
+def test_mm_fp32_rows_do_not_depend_on_the_grid(nmf, k):
+    n = 2003 + 1
+    g = torch.Generator("cuda").manual_seed(k)
+    A = torch.rand((170 * 128 + 5, n), device="cuda", generator=g) - 0.3
+    F = torch.rand((2003, k), device="cuda", generator=g) - 0.3
+    A = A[:, :2003]
+    whole = nmf.nmf_mm_dense(A, F, False, "fp32")
+    for a, b in ((0, 38 * 128), (0, 18 * 128), (152 * 128, 170 * 128 + 5), (0, 77 * 128), (128, 129)):
+        assert torch.equal(nmf.nmf_mm_dense(A[a:b], F, False, "fp32"), whole[a:b]), (a, b)
