@@ -870,12 +870,16 @@ __device__ __forceinline__ void solve64(const SolveParams &P, const Solve64Shape
 // once instead of three (2.4 us each): mode 1 (from the predicted partitions
 // where the FP32 kernel made them), mode 2, and, in mode 0, the second pass
 // that re-solves, from their starting partitions, the right-hand sides the FP32
-// kernel deferred (all of them if more than DEFER_CAP were).
+// kernel deferred (all of them if more than DEFER_CAP were). For large k mode
+// 2 has a launch of its own; `modes` has a bit for each mode a launch serves.
 template <int KW>
 __global__ void __launch_bounds__(BPP_THREADS, 2)
-    bpp_solve_kernel(const SolveParams P, const Solve64Shape sh1, const Solve64Shape sh2)
+    bpp_solve_kernel(const SolveParams P, const Solve64Shape sh1, const Solve64Shape sh2,
+                     int modes)
 {
     const int mode = P.flags[0];
+    if (!((modes >> mode) & 1))
+        return;
     if (mode == 2) {
         solve64<KW, KW, 2>(P, sh2, P.pin, P.nrhs, false, &P.counters[CNT_WORK]);
         return;
@@ -917,40 +921,48 @@ nmf_status launch_solve64(const SolveParams &P, cudaStream_t s)
     sh1.staged = mats_bytes(k, 1) + 2 * pw1 <= SMEM_LIMIT;
     sh2.staged = 0;
     const size_t mats = sh1.staged ? mats_bytes(k, 1) : 0;
-    sh1.warps = warps;
-    while (sh1.warps > 1 && mats + sh1.warps * pw1 > SMEM_LIMIT)
-        --sh1.warps;
-    size_t smem = mats + sh1.warps * pw1;
-    // Mode 2 (larger systems per warp) takes the warps that fit beside it, in
-    // at least half an SM's shared memory.
-    const size_t want2 = warps * pw2 < SMEM_HALF ? warps * pw2 : SMEM_HALF;
-    if (smem < want2)
-        smem = want2;
-    if (smem < pw2)
-        smem = pw2;
-    if (smem > SMEM_LIMIT)
+    auto fit = [&](size_t base, size_t pw, size_t limit) {   // warps of pw bytes beside base
+        return (int)std::min<size_t>(warps, limit > base ? (limit - base) / pw : 0);
+    };
+    sh1.warps = fit(mats, pw1, SMEM_LIMIT);
+    sh2.warps = fit(0, pw2, SMEM_LIMIT);
+    if (sh1.warps < 1 || sh2.warps < 1)
         return NMF_ERR_INVALID_ARG;
-    sh2.warps = (int)(smem / pw2) < warps ? (int)(smem / pw2) : warps;
-    const int nwarps = sh1.warps > sh2.warps ? sh1.warps : sh2.warps;
-    static SmemOptIn opt_in;
-    NMF_TRY(ensure_smem(bpp_solve_kernel<KW>, opt_in, smem));
-    int per_sm = 0;
-    NMF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bpp_solve_kernel<KW>,
-                                                           nwarps * 32, smem));
-    if (per_sm < 1)
-        return NMF_ERR_INVALID_ARG;
-    int64_t blocks = (int64_t)per_sm * sm_count();
-    SolveParams Q = P;
-    Q.chunk = grab_size(P, blocks * nwarps);
-    // As many CTAs as the batch has grabs for (the second pass's size is known
-    // only on the device).
-    const int64_t need =
-        cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), std::min(sh1.warps, sh2.warps));
-    if (need < blocks)
-        blocks = need < 1 ? 1 : need;
-    bpp_solve_kernel<KW><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, sh1, sh2);
-    NMF_LAUNCHED("bpp_solve_kernel");
-    return NMF_OK;
+    const size_t smem1 = mats + sh1.warps * pw1, smem2 = sh2.warps * pw2;
+    auto launch = [&](int modes, int nwarps, int least, size_t smem) -> nmf_status {
+        static SmemOptIn opt_in;
+        NMF_TRY(ensure_smem(bpp_solve_kernel<KW>, opt_in, smem));
+        int per_sm = 0;
+        NMF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bpp_solve_kernel<KW>,
+                                                               nwarps * 32, smem));
+        if (per_sm < 1)
+            return NMF_ERR_INVALID_ARG;
+        int64_t blocks = (int64_t)per_sm * sm_count();
+        SolveParams Q = P;
+        Q.chunk = grab_size(P, blocks * nwarps);
+        // As many CTAs as the batch has grabs for (the second pass's size is
+        // known only on the device).
+        const int64_t need = cdiv(cdiv(P.nrhs, (int64_t)Q.chunk), least);
+        if (need < blocks)
+            blocks = need < 1 ? 1 : need;
+        bpp_solve_kernel<KW><<<(unsigned)blocks, nwarps * 32, smem, s>>>(Q, sh1, sh2, modes);
+        NMF_LAUNCHED("bpp_solve_kernel");
+        return NMF_OK;
+    };
+    // Mode 2 reads G through the L1 cache, which has what the CTA's shared memory
+    // leaves: where its own shape takes less than mode 1's (k >= 83: three warps
+    // and fewer), it has a launch of its own (30000 right-hand sides, k = 88, 100,
+    // 128: 4.2, 7.5, 22.9 ms in a common launch, 3.3, 6.1, 16.5 so).
+    if (smem1 > smem2 && smem1 > SMEM_HALF) {
+        NMF_TRY(launch(1 << 2, sh2.warps, sh2.warps, smem2));
+        return launch(1 << 0 | 1 << 1, sh1.warps, sh1.warps, smem1);
+    }
+    // A common launch: where mode 1 leaves room for two CTAs per SM, mode 2
+    // takes what half an SM holds, else all it can use.
+    const size_t most = smem1 <= SMEM_HALF ? SMEM_HALF : SMEM_LIMIT;
+    sh2.warps = std::max(1, fit(0, pw2, std::max(most, smem1)));
+    const size_t smem = std::max(smem1, sh2.warps * pw2);
+    return launch(7, std::max(sh1.warps, sh2.warps), std::min(sh1.warps, sh2.warps), smem);
 }
 
 template <int KW>

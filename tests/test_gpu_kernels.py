@@ -346,6 +346,34 @@ def test_bpp_singular_gram(nmf):
     assert (comp <= 1e-9 * (scale[good] * np.abs(X[good]).max(axis=1) + 1e-30)).all()
 
 
+# The same at the sizes where the launch for these Grams changes: beside the other
+# FP64 solves in two CTAs per SM or one, or alone (k >= 83), with eight warps down to
+# one. Same bounds; a right-hand side's answer does not depend on the batch.
+@pytest.mark.parametrize("k", [51, 52, 53, 64, 65, 82, 83, 96, 112, 128])
+def test_bpp_singular_gram_launches(nmf, k):
+    rng = np.random.default_rng(k)
+    C = rng.uniform(0, 1, (4 * k, k))
+    C[:, 5] = C[:, 9]
+    G = C.T @ C
+    B32 = (rng.uniform(-0.5, 1.0, (1500, 4 * k)) @ C).astype(np.float32)
+    B32[::3, [5, 9]] = -1.0   # these two stay out: never singular
+    X, P, R, S, worst = run_bpp(nmf, G, B32)
+    assert set(np.unique(S)) <= {0, nmf.NMF_ERR_SINGULAR_GRAM}
+    good = S == 0
+    assert good[::3].all()
+    Bd = B32.astype(np.float64)
+    Y = X @ G - Bd
+    scale = np.abs(Bd).max(axis=1)
+    assert (X[good] >= 0).all()
+    # (X is rounded to FP32: G X - b moves by 2^-24 |G| |X|.)
+    slack = 2.0 ** -23 * (X @ G)[good]
+    assert (Y[good] >= -1e-9 * scale[good, None] - slack).all()
+    assert (np.abs(Y[good]) * (X[good] > 0) <= 1e-9 * scale[good, None] + slack).all()
+    X2, P2, R2, S2, _ = run_bpp(nmf, G, B32[200:207])
+    for a, b in ((X, X2), (P, P2), (R, R2), (S, S2)):
+        assert np.array_equal(a[200:207], b)
+
+
 class shape_of:
     """Sets the launch shape of solves of k inside a with-block, then restores it."""
 
