@@ -72,7 +72,87 @@ __global__ void __launch_bounds__(SPMM_THREADS)
 // rows in flight, in 24 to 32 warps per SM. The same sums in the same order as
 // spmm_kernel. VEC = 2: k even and F, out 8-byte aligned; lane l owns columns
 // 2 l + 64 s and the next (KW slots). VEC = 1: columns l + 32 s.
-constexpr int STREAM_ROWS = 16, STREAM_BATCH = 8;
+//
+// Stretches of more than STREAM_HEAVY entries a row are left for the end and
+// dealt out row by row, neighbouring ones to different warps: the long rows of a
+// matrix often lie together (sorted by degree), and a warp with 16 of them kept
+// the whole GPU waiting (1000 rows of 9000 entries side by side among 10^6 rows of
+// one, k = 50: 18.4 ms, 1.3 so, 3.9 with spmm_kernel; without such rows the search
+// for them costs 2 us of 480). As a function of its own, a heavy row takes no
+// registers from the stretches (inlined: 483 to 950 us at k = 50 to 100).
+constexpr int STREAM_ROWS = 16, STREAM_BATCH = 8, STREAM_HEAVY = 128;
+
+// One row of the product, a warp to it.
+template <int KW, int VEC>
+__device__ __noinline__ void stream_row(const int64_t *__restrict__ rowptr,
+                                        const int32_t *__restrict__ colidx,
+                                        const float *__restrict__ vals, int64_t row,
+                                        const float *__restrict__ F, int k, float *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    float acc[KW][VEC];
+#pragma unroll
+    for (int s = 0; s < KW; ++s)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e)
+            acc[s][e] = 0.0f;
+    int64_t p = rowptr[row];
+    const int64_t end = rowptr[row + 1];
+    int cn = p + lane < end ? colidx[p + lane] : 0;
+    float vn = p + lane < end ? vals[p + lane] : 0.0f;
+    for (; p < end; p += 32) {
+        const int c = cn;
+        const float v = vn;
+        const int64_t pn = p + 32 + lane;
+        cn = pn < end ? colidx[pn] : 0;
+        vn = pn < end ? vals[pn] : 0.0f;
+        const int cnt = (int)min((int64_t)32, end - p);
+        for (int l = 0; l < cnt;) {
+            const int n = min(cnt - l, STREAM_BATCH);
+            float f[STREAM_BATCH][KW][VEC], w[STREAM_BATCH];
+#pragma unroll
+            for (int q = 0; q < STREAM_BATCH; ++q)
+                if (q < n) {
+                    const int64_t cl = __shfl_sync(FULL, c, l + q);
+                    w[q] = __shfl_sync(FULL, v, l + q);
+                    const float *frow = F + cl * k;
+#pragma unroll
+                    for (int s = 0; s < KW; ++s) {
+                        const int cc = VEC * (lane + 32 * s);
+                        if constexpr (VEC == 2) {
+                            const float2 t =
+                                cc < k ? *reinterpret_cast<const float2 *>(frow + cc)
+                                       : make_float2(0.0f, 0.0f);
+                            f[q][s][0] = t.x;
+                            f[q][s][1] = t.y;
+                        } else {
+                            f[q][s][0] = cc < k ? frow[cc] : 0.0f;
+                        }
+                    }
+                }
+#pragma unroll
+            for (int q = 0; q < STREAM_BATCH; ++q)
+                if (q < n)
+#pragma unroll
+                    for (int s = 0; s < KW; ++s)
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e)
+                            acc[s][e] = fmaf(w[q], f[q][s][e], acc[s][e]);
+            l += n;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < KW; ++s) {
+        const int c = VEC * (lane + 32 * s);
+        if (c < k) {
+            float *o = out + row * k + c;
+            if constexpr (VEC == 2)
+                *reinterpret_cast<float2 *>(o) = make_float2(acc[s][0], acc[s][1]);
+            else
+                *o = acc[s][0];
+        }
+    }
+}
 
 template <int KW, int VEC>
 __global__ void __launch_bounds__(SPMM_THREADS)
@@ -90,6 +170,8 @@ __global__ void __launch_bounds__(SPMM_THREADS)
         const int nr = (int)min((int64_t)chunk, rows - r0);
         const int64_t rp = rowptr[r0 + min(lane, nr)];   // lane l: the start of row r0 + l
         const int64_t end = __shfl_sync(FULL, rp, nr);
+        if (chunk > 1 && end - __shfl_sync(FULL, rp, 0) > STREAM_HEAVY * chunk)
+            continue;   // (dealt out below)
         float acc[KW][VEC];
 #pragma unroll
         for (int s = 0; s < KW; ++s)
@@ -170,6 +252,25 @@ __global__ void __launch_bounds__(SPMM_THREADS)
         }
         while (r < nr)
             put_row();
+    }
+    if (chunk == 1)
+        return;
+    // The heavy stretches: warp j of a group of `chunk` warps takes row j of each
+    // of them among the group's (every groups-th).
+    const int64_t group = warp0 / chunk, groups = nw / chunk;
+    const int j = (int)(warp0 - group * chunk);
+    if (group >= groups)
+        return;
+    for (int64_t c0 = group; c0 * chunk < rows; c0 += 32 * groups) {
+        const int64_t a = min((c0 + lane * groups) * chunk, rows);
+        unsigned todo = __ballot_sync(
+            FULL, rowptr[min(a + chunk, rows)] - rowptr[a] > STREAM_HEAVY * chunk);
+        for (; todo; todo &= todo - 1) {
+            const int64_t row = (c0 + (__ffs(todo) - 1) * groups) * chunk + j;
+            if (row >= rows)
+                continue;
+            stream_row<KW, VEC>(rowptr, colidx, vals, row, F, k, out);
+        }
     }
 }
 

@@ -235,3 +235,39 @@ def test_mm_fp32_rows_do_not_depend_on_the_grid(nmf, k):
     whole = nmf.nmf_mm_dense(A, F, False, "fp32")
     for a, b in ((0, 38 * 128), (0, 18 * 128), (152 * 128, 170 * 128 + 5), (0, 77 * 128), (128, 129)):
         assert torch.equal(nmf.nmf_mm_dense(A[a:b], F, False, "fp32"), whole[a:b]), (a, b)
+
+
+# Long rows side by side (a matrix sorted by degree) in the streamed product: they
+# are dealt out to the warps row by row, at the edges of stretches of 16 rows and
+# of 2, and at the last, cut-off stretch. A row's sum does not depend on where the
+# row stands, to the bit, and lies within the FP32 sum's error of the FP64 one.
+@pytest.mark.parametrize("rows", [19463, 160001])
+@pytest.mark.parametrize("k", [33, 50, 100])
+def test_spmm_long_rows_side_by_side(nmf, rows, k):
+    cols = 150_000_000 // (4 * k) + 1
+    rng = np.random.default_rng(rows + k)
+    count = rng.integers(0, 4, rows)
+    count[4001:4107] = 3000
+    count[8007] = 40001
+    count[rows - 3:] = [2500, 0, 2500]
+    count[0], count[16] = 2049, 2047
+    ptr = np.concatenate([[0], np.cumsum(count)]).astype(np.int64)
+    col = rng.integers(0, cols, ptr[-1]).astype(np.int32)
+    val = rng.uniform(-1, 1, ptr[-1]).astype(np.float32)
+    F = torch.rand((cols, k), device="cuda", generator=torch.Generator("cuda").manual_seed(k))
+
+    def product(order):
+        at = np.concatenate([np.arange(ptr[r], ptr[r + 1]) for r in order])
+        p = np.concatenate([[0], np.cumsum(count[order])]).astype(np.int64)
+        return nmf.nmf_mm_csr(*(torch.from_numpy(x).cuda() for x in (p, col[at], val[at])), cols, F)
+
+    out = product(np.arange(rows))
+    order = rng.permutation(rows)
+    assert torch.equal(product(order), out[torch.from_numpy(order).cuda()])
+    for r in (0, 16, 4001, 4106, 8007, rows - 3, rows - 2, rows - 1, 5000):
+        e = slice(int(ptr[r]), int(ptr[r + 1]))
+        terms = (torch.from_numpy(val[e]).cuda().double()[:, None]
+                 * F[torch.from_numpy(col[e]).cuda().long()].double())
+        # n sequential FMAs: at most n roundings of the running sum.
+        assert ((out[r].double() - terms.sum(0)).abs()
+                <= max(count[r], 1) * 2.0 ** -24 * terms.abs().sum(0)).all(), r
