@@ -40,6 +40,8 @@
 // HALS 45 us, MU 37 us (one warp per row: 272 and 51 us; HBM alone 8.5 us);
 // 1000000 x 50: HALS 411 us (2785), MU 356 us (478). 128-row tiles, four rows
 // per lane, were slower at 96000 rows (50 and 46 us) and 1000000 (457, 421).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace nmf {
@@ -415,20 +417,22 @@ __global__ void lu_sum_kernel(const double *__restrict__ partials, int n, double
     }
 }
 
+// Warps per CTA (one CTA per SM) of the tile kernel that the shared memory holds.
+int ru_warps(int k, bool dup)
+{
+    const size_t g = sizeof(float) * ru_g_floats(k, dup), w = sizeof(float) * ru_warp_floats(k);
+    return (int)std::min<size_t>(RU_WARPS, (LU_SMEM - g) / w);
+}
+
 template <bool HALS, bool DUP>
 nmf_status launch_rows(const double *G, int k, const float *R, float *X, int64_t rows,
                        cudaStream_t s)
 {
     const int64_t tiles = cdiv(rows, RU_ROWS);
-    // One CTA per SM, with the warps that share the tiles out evenly (as many
-    // as the shared memory holds), so that G is staged once per SM.
-    const size_t g = sizeof(float) * ru_g_floats(k, DUP), w = sizeof(float) * ru_warp_floats(k);
-    int64_t nw = cdiv(tiles, sm_count());
-    if (nw > RU_WARPS)
-        nw = RU_WARPS;
-    while (nw > 1 && g + nw * w > LU_SMEM)
-        --nw;
-    const size_t smem = g + nw * w;
+    // As many warps as share the tiles out evenly, so that G is staged once per
+    // SM.
+    const int64_t nw = std::min<int64_t>(cdiv(tiles, sm_count()), ru_warps(k, DUP));
+    const size_t smem = sizeof(float) * (ru_g_floats(k, DUP) + nw * ru_warp_floats(k));
     static SmemOptIn opt_in;
     NMF_TRY(ensure_smem(row_update_kernel<HALS, DUP>, opt_in, smem));
     int64_t blocks = cdiv(tiles, nw);
@@ -480,13 +484,40 @@ nmf_status launch_lu_k(const double *G, int k, const float *R, float *X, int64_t
     return launch_lu<4, OP>(G, k, R, X, rows, partials, max_parts, nparts, s);
 }
 
+// Whether the tile kernel is the faster one. HALS: from the row count on where a
+// wave of tiles (20-25 us at k = 50, whatever the batch) passes that of single
+// rows (17); no k up to 128 and no partial wave after it is slower (k = 128, 7297
+// rows 94 / 115 us, 38913 rows, one tile past a wave, 178 / 405; k = 50, 96000
+// rows 45 / 264).
+// MU: single rows cost little more than the tiles' terms, so the last wave of
+// tiles has to be full enough: the time of full waves stands against that of
+// their rows, done singly, like 1 to 1.4 for 25 to 32 coordinates (one slot per
+// lane there), 1.6-1.8 up to 48, 1.5 up to 56 and 1.2-1.4 up to 64 (two slots, 12
+// and 10 warps of tiles), 1.65 and more with at least 7 warps (four slots), 1.65
+// (to k = 104) and 1.5 with 6, 1.25 with 5 and 1.05 with 4. Measured, tiles / single rows: k = 32,
+// 175200 rows 40.9 / 40.9 us, 117000 rows (half of the second wave) 40.9 / 30.5; k
+// = 64, 90000 rows 51 / 59, 97300 rows 86 / 63; k = 100, 80000 rows 121 / 141,
+// 58369 rows 125 / 108; k = 128, 77900 rows 213 / 168.
+bool rows_in_tiles(bool hals, int k, int64_t rows)
+{
+    if (rows < (hals ? 48 : 384) * (int64_t)sm_count())
+        return false;
+    if (hals || k <= 24)
+        return true;
+    const int nw = ru_warps(k, k <= RU_DUP_K);
+    const int64_t tiles = cdiv(rows, RU_ROWS), slots = (int64_t)nw * sm_count();
+    const double fill = (double)tiles / (double)(cdiv(tiles, slots) * slots);
+    return fill >= (k <= 32   ? 0.75
+                    : k <= 48 ? 0.6
+                    : k <= 64 ? (nw == RU_WARPS ? 0.67 : 0.82)
+                    : nw >= 7 ? 0.0
+                    : nw == 6 ? (k <= 104 ? 0.66 : 0.75)
+                    : nw == 5 ? 0.83
+                              : 0.95);
+}
+
 }  // namespace
 
-// The tile kernel from the row count where its tiles keep the GPU busy: a tile
-// of 64 rows takes 20-25 us whatever the batch, a wave of single rows 10 (MU)
-// or 17 (HALS) us. Measured, k = 50, tiles against single rows: HALS 5000 rows
-// 29 / 25 us, 20000 29 / 70, 96000 45 / 278; MU 20000 rows 33 / 19, 50000
-// 33 / 31, 77824 33 / 44.
 nmf_status launch_local_update(int solver, const double *G, int k, const float *R, float *X,
                                int64_t rows, cudaStream_t s)
 {
@@ -495,7 +526,7 @@ nmf_status launch_local_update(int solver, const double *G, int k, const float *
     if (solver != NMF_SOLVER_MU && solver != NMF_SOLVER_HALS)
         return NMF_ERR_INVALID_ARG;
     const bool hals = solver == NMF_SOLVER_HALS;
-    if (rows < (hals ? 48 : 384) * (int64_t)sm_count()) {
+    if (!rows_in_tiles(hals, k, rows)) {
         int np = 0;
         if (hals)
             return launch_lu_k<LU_HALS>(G, k, R, X, rows, nullptr, 0, &np, s);

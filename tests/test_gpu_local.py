@@ -158,6 +158,20 @@ def test_step_at_tile_edges(nmf, solver, k, rows):
     assert row_rel_err(Xd.double().cpu().numpy(), ref) <= 2e-5
 
 
+# MU takes tiles only where their last wave is full enough, by k and the warps that
+# fit (k = 25, 40, 56, 64, 100, 112, 128 on 152 SMs): both sides of each line. Same
+# bound.
+@pytest.mark.parametrize("k,rows", [(25, 87488), (25, 87616), (40, 69952), (40, 70080),
+                                    (56, 78144), (56, 78272), (64, 79744), (64, 79808),
+                                    (100, 76992), (100, 77056), (112, 80704), (112, 80768),
+                                    (128, 73920), (128, 73984), (96, 58369)])
+def test_mu_at_the_lines_of_partial_waves(nmf, k, rows):
+    G, R, X = problem(rows, k, seed=rows + k)
+    Xd = dev(X)
+    nmf.nmf_update_mu(dev(G, torch.float64), dev(R), Xd)
+    assert row_rel_err(Xd.double().cpu().numpy(), oracle.mu(G, R, X)) <= 2e-5
+
+
 # The division of HALS's coordinate on both sides of the switch between its two
 # kernels (48 rows per SM; 152 SMs): k = 1 makes x = max(r, 0) / g of every row,
 # which the FP32 division rounds to nearest. Diagonals down to the smallest
