@@ -383,8 +383,12 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(C == 1 ? PREP_THREAD
     if (rank != 0)
         return;
     // cond_1 of the scaled matrix, max column sum of |G_ac| / (d_a d_c) times
-    // max column sum of |M_ac| d_a d_c with d_a = sqrt(G_aa), in FP32 (the
-    // number only picks the arithmetic; where it is not finite, FP64).
+    // max column sum of |M_ac| d_a d_c with d_a = sqrt(G_aa). In FP32 first: with
+    // the diagonal far from the ends of the range that estimate is within 150 x
+    // 2^-24 per factor of the FP64 number (one rounding of G or M, two of each
+    // scale, at most 128 additions), so that 2^-13 away from the line it decides
+    // alike. Nearer, or with such a diagonal, the FP64 number does. Where FP32
+    // cannot hold G or M, FP64 solves.
     red[0][tid] = sg;
     red[1][tid] = prep_colsum(Ms, u, dsq);
     __syncthreads();
@@ -392,7 +396,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(C == 1 ? PREP_THREAD
         return;
     const int parts = nt >> 7;
     float mg = 0.0f, mm = 0.0f;
-    bool fine = true;
+    bool fine = true, in_range = true;
     for (int c = lane; c < u; c += 32) {
         float tg = 0.0f, tm = 0.0f;
         for (int q = 0; q < parts; ++q) {
@@ -402,11 +406,31 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(C == 1 ? PREP_THREAD
         tg *= rdsq[c];
         tm *= dsq[c];
         fine &= isfinite(tg) && isfinite(tm);
+        in_range &= dsq[c] >= 0x1p-50f && dsq[c] <= 0x1p50f;
         mg = fmaxf(mg, tg);
         mm = fmaxf(mm, tm);
     }
     fine = __all_sync(FULL, fine);
-    const double cond = (double)warp_max(mg) * (double)warp_max(mm);
+    in_range = __all_sync(FULL, in_range);
+    double cond = (double)warp_max(mg) * (double)warp_max(mm);
+    if (fine && (!in_range || fabs(cond - COND_FP32) <= 0x1p-13 * COND_FP32)) {
+        double *d = floor_;   // (the floors are done with)
+        for (int a = lane; a < u; a += 32)
+            d[a] = sqrt(G[uidx[a] * (k + 1)]);
+        __syncwarp();
+        double dg = 0.0, dm = 0.0;
+        for (int c = lane; c < u; c += 32) {
+            double tg = 0.0, tm = 0.0;
+            for (int a = 0; a < u; ++a) {
+                const int e = uidx[a] * k + uidx[c];
+                tg += fabs(G[e]) / d[a];
+                tm += fabs(M64[e]) * d[a];
+            }
+            dg = fmax(dg, tg / d[c]);
+            dm = fmax(dm, tm * d[c]);
+        }
+        cond = warp_max(dg) * warp_max(dm);
+    }
     if (lane == 0) {
         const int mode = fine && cond <= COND_FP32 ? 0 : 1;
         flags[0] = mode;

@@ -346,6 +346,26 @@ def test_bpp_singular_gram(nmf):
     assert (comp <= 1e-9 * (scale[good] * np.abs(X[good]).max(axis=1) + 1e-30)).all()
 
 
+# The arithmetic of a half-step follows the scaled cond_1 in FP64 on either side of
+# its line, 1e4 (1 + c) / (1 - c) for a pair of columns with cosine c, whatever the
+# columns' scales. A right-hand side entry of 1e-8 shows which one ran: positive in
+# FP64, within the sign tolerance (2^-20) of FP32 a zero.
+@pytest.mark.parametrize("k", [3, 20, 33, 50, 53, 100, 128])
+def test_bpp_mode_at_the_condition_line(nmf, k):
+    for seed in range(8):
+        rng = np.random.default_rng(1000 * k + seed)
+        d = rng.uniform(0.1, 10.0, k)
+        i, j, t = rng.permutation(k)[:3]
+        for side in (-1, 1):
+            R = 1e4 * (1 + side * 1e-9)
+            G = np.eye(k)
+            G[i, j] = G[j, i] = (R - 1) / (R + 1)
+            b = d * rng.uniform(0.5, 1.0, k)
+            b[t] = 1e-8 * d[t]
+            X = run_bpp(nmf, G * d[:, None] * d, b[None].astype(np.float32))[0]
+            assert (X[0, t] > 0) == (side > 0), (seed, side, X[0, t])
+
+
 # The same at the sizes where the launch for these Grams changes: beside the other
 # FP64 solves in two CTAs per SM or one, or alone (k >= 83), with eight warps down to
 # one. Same bounds; a right-hand side's answer does not depend on the batch.
