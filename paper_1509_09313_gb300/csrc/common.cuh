@@ -78,29 +78,50 @@ inline nmf_status ensure_smem(Kernel kernel, SmemOptIn &cache, size_t bytes)
     return NMF_OK;
 }
 
-// Sum of `n` floats `stride` apart, correct to about 2^-46 of their absolute
-// sum and rounded once: a pair of floats (Knuth's two-sum), since the FP64 pipe
-// does two additions per clock per SM (the sum of four 24000 x 50 partials
-// took 23 us in FP64, most of it additions and conversions). Where the FP32
-// sum is not finite (an infinity or NaN among the terms, or an overflow on the
-// way), the terms are added in FP64.
+// Sum of `n` floats `stride` apart, rounded once, as good as the rounding of their
+// FP64 sum (in order, `group` at a time). The FP64 pipe does two additions per
+// clock per SM (the sum of four 24000 x 50 partials took 23 us on it, most of it
+// additions and conversions), so a pair of floats (Knuth's two-sum) goes first.
+// Where no addition of the errors c rounded (few terms of one size: nearly
+// always), s + c is the true sum and its rounding the result. Else s + c is within
+// n^2 2^-49 of the terms' absolute sum `a` of the true sum, the FP64 sum within n
+// 2^-53, and where every number within four times that of s + c rounds to one
+// float, that is the FP64 sum's. In what remains (one sum in 10^4 or fewer: close
+// to the middle of two floats; infinities, NaN, overflow on the way) the terms are
+// added in FP64.
+template <int group>
 __device__ __forceinline__ float sum_strided(const float *__restrict__ v, int n, int64_t stride)
 {
-    float s = 0.0f, c = 0.0f;
+    float s = 0.0f, c = 0.0f, a = 0.0f;
+    bool exact = true;
 #pragma unroll 4
     for (int i = 0; i < n; ++i) {
         const float x = v[i * stride];
         const float t = s + x;
         const float b = t - s;
-        c += (s - (t - b)) + (x - b);
+        const float q = (s - (t - b)) + (x - b);
+        const float m = c + q;
+        exact = exact && m - c == q && m - q == c;
+        a += fabsf(x);
+        c = m;
         s = t;
     }
-    if (isfinite(s))
-        return s + c;
-    double d = 0.0;
-    for (int i = 0; i < n; ++i)
-        d += (double)v[i * stride];
-    return (float)d;
+    const float r = s + c;
+    if (exact && isfinite(a))
+        return r;
+    const float b = r - s;
+    const float e = (s - (r - b)) + (c - b);   // r + e = s + c exactly
+    const float d = (float)(n * n) * 0x1p-46f * a;
+    if (r + (e - d) == r && r + (e + d) == r)
+        return r;
+    double sum = 0.0;
+    for (int i = 0; i < n; i += group) {
+        double g = (double)v[i * stride];
+        for (int q = 1; q < group; ++q)
+            g += (double)v[(i + q) * stride];
+        sum += g;
+    }
+    return (float)sum;
 }
 
 // True when [a, a + bytes) and [b, b + bytes) share a byte.

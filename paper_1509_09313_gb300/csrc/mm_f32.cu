@@ -501,7 +501,7 @@ __global__ void f32_reduce_kernel(const float *__restrict__ part, int splits, in
 {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len;
          e += (int64_t)gridDim.x * blockDim.x)
-        out[e] = sum_strided(part + e, 2 * splits, len);
+        out[e] = sum_strided<2>(part + e, 2 * splits, len);
 }
 
 // F^T (trans = 0): Ft[c][q] = F[q][c] for c < k, 0 for k <= c < kpt, rows of

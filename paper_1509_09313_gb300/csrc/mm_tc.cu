@@ -813,7 +813,7 @@ __global__ void mm_tc_reduce_kernel(const float *__restrict__ part, int arrays, 
         const int64_t p = e / kc;
         e = p * k + col0 + (e - p * kc);
     }
-    out[e] = sum_strided(part + e, arrays, P * k);
+    out[e] = sum_strided<1>(part + e, arrays, P * k);
 }
 
 // The shared tiles of the pass with the objective: out from the folds' partial

@@ -271,3 +271,29 @@ def test_spmm_long_rows_side_by_side(nmf, rows, k):
         # n sequential FMAs: at most n roundings of the running sum.
         assert ((out[r].double() - terms.sum(0)).abs()
                 <= max(count[r], 1) * 2.0 ** -24 * terms.abs().sum(0)).all(), r
+
+
+# Partial sums of a split contraction are added in FP64 and rounded once (A H^T in
+# FP32 has one chain and none). Three terms in three splits: 1 + 2^-24 lies in the
+# middle of two floats, and 2^-50 decides; further on sums that cancel, that overflow
+# FP32 on the way and that end subnormal.
+@pytest.mark.parametrize("precision,trans", [("fp32", True), ("bf16x3", True), ("bf16x3", False)])
+def test_split_sums_round_once(nmf, precision, trans):
+    Q, P, k = 16000, 128, 8
+    h = 2.0 ** -24
+    terms = [(1, h, 2.0 ** -50), (1, h, -(2.0 ** -50)), (1, 2 * h, -(2.0 ** -50)),
+             (1, 0, -(2.0 ** -50)), (-1, -h, -(2.0 ** -50)), (h, 2.0 ** -50, 1),
+             (2.0 ** -50, 1, h), (3 * h, 1, 2.0 ** -60), (1 + 2.0 ** -6, -1, 2.0 ** -70), (0, 0, 0)]
+    if precision == "fp32":
+        terms += [(2.0 ** 127, 2.0 ** 127, -(2.0 ** 127)),
+                  (1.5 * 2.0 ** -130, 2.0 ** -140, -(2.0 ** -133))]
+    A = torch.zeros((P, Q))
+    at = [0, Q // 2, Q - 1]
+    for r, t in enumerate(terms):
+        A[r, at] = torch.tensor(t, dtype=torch.float32)
+    want = [np.float32(np.float64(np.float64(a) + np.float64(b)) + np.float64(c))
+            for a, b, c in terms]
+    Ad = (A.T.contiguous() if trans else A).cuda()
+    out = nmf.nmf_mm_dense(Ad, torch.ones((Q, k), device="cuda"), trans, precision).cpu().numpy()
+    for r, w in enumerate(want):
+        assert np.array_equal(out[r], np.full(k, w, np.float32)), (r, out[r], w)
