@@ -236,10 +236,13 @@ __global__ void __launch_bounds__(RU_WARPS * 32, 1)
                 float2 x;
                 if (HALS) {
                     add(i);
-                    const float n0 = (r.x - tot[i].x) - err[i].x;
-                    const float n1 = (r.y - tot[i].y) - err[i].y;
-                    x.x = gii > 0.0f ? quotient(n0 > 0.0f ? n0 : 0.0f, gii, rg) : 0.0f;
-                    x.y = gii > 0.0f ? quotient(n1 > 0.0f ? n1 : 0.0f, gii, rg) : 0.0f;
+                    // max(n, 0), where the error of a sum that overflowed, a NaN,
+                    // does not take an infinite n for zero.
+                    const float d0 = r.x - tot[i].x, d1 = r.y - tot[i].y;
+                    const float n0 = fmaxf(d0 - err[i].x, d0 == INFINITY ? d0 : 0.0f);
+                    const float n1 = fmaxf(d1 - err[i].y, d1 == INFINITY ? d1 : 0.0f);
+                    x.x = gii > 0.0f ? quotient(n0, gii, rg) : 0.0f;
+                    x.y = gii > 0.0f ? quotient(n1, gii, rg) : 0.0f;
                     *reinterpret_cast<float2 *>(Xs + (i0 + i) * RS + 2 * lane) = x;
                 } else {
                     const float2 t = tot[i];

@@ -200,3 +200,30 @@ def test_hals_quotient_is_the_rounded_one(nmf, g, rows):
     R = R.astype(np.float32)
     want = np.stack([R[:, 0] / np.float32(4), np.zeros(rows, np.float32), R[:, 2] / np.float32(2)], 1)
     assert np.array_equal(X.cpu().numpy(), want)
+
+
+# Infinities, NaN and sums that overflow, on both sides of the switch between the
+# kernels: the same answer. A negative sum beyond the range (only a Gram with
+# negative entries has one) makes the coordinate infinite, not zero.
+def test_hals_special_values_in_both_kernels(nmf):
+    k, rows = 5, 7297
+    G = np.eye(k) * 3 + 0.5
+    G[0, 3] = G[3, 0] = -2.0
+    G[1, 2] = G[2, 1] = 0.0
+    X = np.full((rows, k), 0.5, np.float32)
+    R = np.full((rows, k), 2.0, np.float32)
+    X[0::8, [0, 3]] = 3e38
+    R[1::8, 1] = np.inf
+    R[2::8, 1] = -np.inf
+    R[3::8, 1] = np.nan
+    R[4::8] = 3e38
+    whole, part = dev(X), dev(X[:1000])
+    nmf.nmf_update_hals(dev(G, torch.float64), dev(R), whole)
+    nmf.nmf_update_hals(dev(G, torch.float64), dev(R[:1000]), part)
+    a, b = whole[:1000].cpu().numpy(), part.cpu().numpy()
+    assert np.isposinf(a[0::8, 0]).all() and np.isposinf(a[1::8, 1]).all()
+    assert np.array_equal(np.isfinite(a), np.isfinite(b))
+    assert np.array_equal(a[~np.isfinite(b)], b[~np.isfinite(b)], equal_nan=True)
+    # Finite ones: the kernels' sums round differently, a few units of 2^-24.
+    fin = np.isfinite(b)
+    assert (np.abs(a[fin].astype(np.float64) - b[fin]) <= 16 * 2.0 ** -24 * np.abs(b[fin])).all()
