@@ -351,13 +351,12 @@ namespace {
 
 double l2_bytes()
 {
-    static double bytes = 0.0;
-    if (bytes == 0.0) {
+    static const double bytes = [] {   // (initialised once, whatever the threads)
         int dev = 0, b = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&b, cudaDevAttrL2CacheSize, dev);
-        bytes = b > 0 ? b : 1.0;
-    }
+        return b > 0 ? (double)b : 1.0;
+    }();
     return bytes;
 }
 
