@@ -52,6 +52,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <iterator>
 #include <mutex>
 
 #include "bpp_internal.cuh"
@@ -1180,6 +1181,11 @@ nmf_status bpp_tune(int k, int64_t nrhs, const double *G, const float *B, float 
     float best_ms = -1.0f;
     nmf_status st = NMF_OK;
     for (const BppShape &c : cand) {
+        // The same launch as another candidate: above k = 64 the FP32 solves
+        // take twice the shape's warps, at most 16, and the FP64 ones at most 8;
+        // the last one differs only in its group pass.
+        if ((c.warps == 16 && k > 64) || (&c == std::end(cand) - 1 && c.group == gm))
+            continue;
         P.warps = c.warps;
         P.chunk = c.chunk;
         P.group = c.group;
