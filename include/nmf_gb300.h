@@ -178,7 +178,7 @@ nmf_status nmf_nls_bpp_set_shape(int32_t k, int32_t warps, int32_t chunk, int32_
 nmf_status nmf_nls_bpp_get_shape(int32_t k, int32_t *warps, int32_t *chunk, int32_t *group);
 
 /* Allocation-free variant of nmf_nls_bpp (no counterpart in the paper; an
- * interface of this library). Same arguments, computation and results as
+ * interface of this library). Same arguments, kernels and results as
  * nmf_nls_bpp, but it never allocates device memory, for callers that cannot
  * call cudaMalloc: code under a memory manager that owns all device memory
  * (a framework's caching allocator or a fixed pool), latency-critical loops
@@ -197,6 +197,11 @@ nmf_status nmf_nls_bpp_get_shape(int32_t k, int32_t *warps, int32_t *chunk, int3
  *   - All calls share the one array and it keeps the last call's contents:
  *     calls that overlap on the GPU (for example on two streams at once)
  *     race and corrupt each other's results. Keep them ordered.
+ *   - Without passive_out and rounds_out, nmf_nls_bpp takes scratch to start
+ *     FP64 half-steps from predicted partitions; here they start from
+ *     passive_in, which takes about four times as long. The minimiser is the
+ *     same; an index with x_i = y_i = 0 may come out at rounding noise in one
+ *     call and at 0 in the other.
  *   - Waits for `stream` and returns the worst per-RHS status. */
 #define NMF_NOALLOC_MAX_K 128
 #define NMF_NOALLOC_SCRATCH_BYTES (272 * 1024)
@@ -206,13 +211,16 @@ nmf_status nmf_nls_bpp_noalloc(const nmf_nls_desc *d, void *stream);
  * in place), with G (k x k float64, the Gram of the fixed factor) and R (rows x k
  * float32, its right-hand sides: A H^T for W, (W^T A)^T for H^T):
  *   x_ij <- x_ij R_ij / (X G)_ij,  every (X G)_ij from the X before the step;
- * x_ij is left unchanged where (X G)_ij <= 0. Asynchronous on `stream`. */
+ * x_ij is left unchanged where (X G)_ij <= 0. Rows are independent, but large
+ * batches take another kernel, whose sums round differently: a row's last bits
+ * depend on how many rows the call has. Asynchronous on `stream`. */
 nmf_status nmf_update_mu(int32_t k, int64_t rows, const double *G, const float *R, float *X,
                          void *stream);
 
 /* One HALS sweep (Eq. 6) of the rows of X with the same arguments: for
  * i = 0..k-1 in order, x_i <- [R_i - sum_{l != i} G_li x_l]_+ / G_ii using the
- * newest x_l; x_i = 0 where G_ii <= 0. Asynchronous on `stream`. */
+ * newest x_l; x_i = 0 where G_ii <= 0. A row's last bits depend on the number of
+ * rows as in nmf_update_mu. Asynchronous on `stream`. */
 nmf_status nmf_update_hals(int32_t k, int64_t rows, const double *G, const float *R, float *X,
                            void *stream);
 

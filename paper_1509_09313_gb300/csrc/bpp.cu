@@ -1009,10 +1009,13 @@ nmf_status launch_modes(SolveParams P, cudaStream_t s)
                                         P.flags, s));
     }
     // Mode 1 (FP64): the FP32 kernel first predicts each right-hand side's
-    // partition, and the FP64 solves start from it (their answer does not
-    // depend on the start; they need fewer rounds: 16000 right-hand sides, k =
-    // 50, from the signs of the unconstrained solution: 0.32 ms, 1.25 from that
-    // start itself). Not under a tight cap, which keeps its meaning.
+    // partition, and the FP64 solves start from it: they need fewer rounds (16000
+    // right-hand sides, k = 50, from the signs of the unconstrained solution: 0.32
+    // ms, 1.25 from that start itself). Each NLS has one minimiser, but a
+    // degenerate index (x_i = y_i = 0) may come out at rounding noise or at zero,
+    // passive or not, by the start, and a batch that the cap on rounds stopped
+    // short of an answer may now reach it. Not under a tight cap, which keeps its
+    // meaning.
     if (P.max_rounds < 2 * PREDICT_ROUNDS)
         P.predict = nullptr;
     NMF_TRY(launch_solve32(P, s));

@@ -4,10 +4,14 @@
 // that owns all device memory (a framework's caching allocator, a fixed
 // pool), latency-critical loops where cudaMalloc / cudaFree may synchronise
 // the device, and programs that must not grow their device footprint after
-// start-up. For them this entry point runs exactly the kernels of
-// nmf_nls_bpp, but its workspace is a fixed array compiled into the library
-// instead of a stream-ordered allocation; the caller still supplies every
-// input and output buffer.
+// start-up. For them this entry point runs the kernels of nmf_nls_bpp, but its
+// workspace is a fixed array compiled into the library instead of a
+// stream-ordered allocation; the caller still supplies every input and output
+// buffer. One difference: nmf_nls_bpp without passive_out and rounds_out takes
+// scratch for the partitions that FP64 solves start from, which the array does
+// not hold; here such a call starts them from passive_in, as it does with
+// rounds_out, and an FP64 batch takes about four times as long. With passive_out
+// both predict there.
 //
 // The array is a file-scope __device__ variable, so every GPU that loads the
 // library holds it until the process exits. Host code cannot pass the
