@@ -220,6 +220,25 @@ def test_one_call_takes_no_scratch_that_does_not_pay(nmf, m, k):
         assert used <= few + 4 * m * 64, used
 
 
+# The same shapes unshared against their parts shared: the products to the bit; the
+# objective, whose residuals are the same but summed in other groups (compensated FP32
+# sums per thread, FP64 across), to the rounding of those sums.
+@pytest.mark.parametrize("m,k", [(9728, 50), (4608, 24), (21760, 10)])
+def test_unshared_and_shared_waves_agree(nmf, m, k):
+    n = 16000
+    g = torch.Generator("cuda").manual_seed(m)
+    A, F = (torch.rand(s, device="cuda", generator=g) for s in ((m, n), (n, k)))
+    W = torch.rand((m, k), device="cuda", generator=g)
+    whole = nmf.nmf_mm_dense(A, F, False, "fp32")
+    f = nmf.nmf_objective_dense(A, W, F, "bf16x3")
+    parts = 0.0
+    for a in range(0, m, 2304):   # 18 tiles and what is left
+        b = min(m, a + 2304)
+        assert torch.equal(nmf.nmf_mm_dense(A[a:b], F, False, "fp32"), whole[a:b]), a
+        parts += nmf.nmf_objective_dense(A[a:b], W[a:b], F, "bf16x3")
+    assert abs(parts - f) <= 2.0 ** -22 * f
+
+
 # A H^T in FP32 with the last wave's tiles shared out, alone or behind a whole wave
 # (152 tiles of 128 rows), against the same rows multiplied alone or unshared: a
 # row's sums do not depend on the grid, to the bit. Column chunks of every width,
