@@ -29,6 +29,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -607,38 +608,37 @@ struct Acts {
     size_t bytes;
 };
 
-size_t acts_bytes(const MlpNet &net, int64_t n, bool train)
-{
-    const size_t nh = (size_t)n * net.h, nk = (size_t)n * net.k;
-    size_t b = sizeof(float) * (2 * nh + nk);
-    if (train)
-        b += sizeof(float) * (nk + 2 * nh + n) +
-             sizeof(float) * (size_t)MLP_MAX_SPLITS * net.h * std::max(3 * net.k, net.h) +
-             sizeof(double) * 1025;
-    return b + 256 * 8;
-}
-
+// The buffers in `mem`, each on 256 bytes; bytes is what they take (mem may be
+// null, for that alone).
 Acts carve(const MlpNet &net, int64_t n, bool train, void *mem)
 {
-    auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-    char *p = static_cast<char *>(mem);
+    size_t off = 0;
+    auto take = [&](auto *&ptr, size_t count) {
+        ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(
+            reinterpret_cast<uintptr_t>(mem) + off);
+        off += (sizeof(*ptr) * count + 255) & ~size_t(255);
+    };
     const size_t nh = (size_t)n * net.h, nk = (size_t)n * net.k;
     Acts a{};
-    a.z1 = reinterpret_cast<float *>(p); p += al(sizeof(float) * nh);
-    a.z2 = reinterpret_cast<float *>(p); p += al(sizeof(float) * nh);
-    a.logit = reinterpret_cast<float *>(p); p += al(sizeof(float) * nk);
+    take(a.z1, nh);
+    take(a.z2, nh);
+    take(a.logit, nk);
     if (train) {
-        a.dz3 = reinterpret_cast<float *>(p); p += al(sizeof(float) * nk);
-        a.dz2 = reinterpret_cast<float *>(p); p += al(sizeof(float) * nh);
-        a.dz1 = reinterpret_cast<float *>(p); p += al(sizeof(float) * nh);
-        a.done = reinterpret_cast<unsigned int *>(p); p += al(sizeof(unsigned int) * 256);
-        a.split = reinterpret_cast<float *>(p);
-        p += al(sizeof(float) * (size_t)MLP_MAX_SPLITS * net.h * std::max(3 * net.k, net.h));
-        a.loss_part = reinterpret_cast<double *>(p); p += al(sizeof(double) * 1024);
-        a.loss = reinterpret_cast<double *>(p); p += al(sizeof(double));
+        take(a.dz3, nk);
+        take(a.dz2, nh);
+        take(a.dz1, nh);
+        take(a.done, 256);
+        take(a.split, (size_t)MLP_MAX_SPLITS * net.h * std::max(3 * net.k, net.h));
+        take(a.loss_part, 1024);
+        take(a.loss, 1);
     }
-    a.bytes = (size_t)(p - static_cast<char *>(mem));
+    a.bytes = off;
     return a;
+}
+
+size_t acts_bytes(const MlpNet &net, int64_t n, bool train)
+{
+    return carve(net, n, train, nullptr).bytes;
 }
 
 nmf_status forward(const MlpNet &net, const float *F, int64_t n, const Acts &a, cudaStream_t s)

@@ -78,6 +78,27 @@ def test_gradient_matches_oracle(nmf, k, h, n):
         assert np.linalg.norm(a - b) <= 2e-4 * np.linalg.norm(b) + 1e-9
 
 
+# Small batches, where the counters of the bias gradients take more of the workspace
+# than the activations do, and widths whose buffers end just past 256 bytes; then one
+# training step of the same batch. Same bounds.
+@pytest.mark.parametrize("k,h", [(1, 1), (8, 16), (5, 33), (50, 100), (20, 300), (128, 1024)])
+@pytest.mark.parametrize("n", [1, 2, 17, 65, 129, 255])
+def test_gradient_of_small_batches(nmf, k, h, n):
+    net, p = _net(nmf, k, h, seed=k + h)
+    rng = np.random.default_rng(n)
+    F = rng.standard_normal((n, 3 * k)).astype(np.float32)
+    y = rng.random((n, k)) < 0.4
+    lab = nmf.bool_to_passive(torch.from_numpy(y).cuda())
+    g, loss = net.nmf_mlp_gradient(dev(F), lab)
+    lo, go = omlp.loss_and_grad(p, F, y, k, h)
+    assert loss.item() == pytest.approx(lo, rel=1e-5)
+    g = g.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(g - go) <= 1e-4 * np.linalg.norm(go)
+    for a, b in zip(omlp.unpack(g, k, h), omlp.unpack(go, k, h)):
+        assert np.linalg.norm(a - b) <= 2e-4 * np.linalg.norm(b) + 1e-9
+    assert net.nmf_mlp_train(dev(F), lab, batch=n, lr=1e-3).item() == pytest.approx(lo, rel=1e-5)
+
+
 def test_adam_steps_match_oracle(nmf):
     k, h, n, lr = 20, 64, 512, 1e-3
     net, p = _net(nmf, k, h, seed=3)
