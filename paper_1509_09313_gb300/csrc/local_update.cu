@@ -24,8 +24,8 @@
 // for the direct form). Eight terms at a time are summed apart and then added
 // to the total.
 //
-// local_update_kernel (one warp per row) serves batches too small for tiles:
-// lane l holds entries l, l + 32, ... (KW slots), G in FP32 in shared memory
+// local_update_kernel (one warp per row) serves batches too small for tiles, and
+// MU where the last wave of tiles would be too empty: lane l holds entries l, l + 32, ... (KW slots), G in FP32 in shared memory
 // lane-interleaved (entry (r, c) at r * 32 KW + (c % 32) * KW + c / 32) so
 // that a lane reads its KW entries of a row as one vector; MU forms X G with
 // one product, HALS each coordinate's sum with a butterfly. It also forms the
