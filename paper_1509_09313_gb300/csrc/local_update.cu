@@ -25,14 +25,15 @@
 // to the total.
 //
 // local_update_kernel (one warp per row) serves batches too small for tiles, and
-// MU where the last wave of tiles would be too empty: lane l holds entries l, l + 32, ... (KW slots), G in FP32 in shared memory
-// lane-interleaved (entry (r, c) at r * 32 KW + (c % 32) * KW + c / 32) so
-// that a lane reads its KW entries of a row as one vector; MU forms X G with
-// one product, HALS each coordinate's sum with a butterfly. It also forms the
-// projected-gradient norm of the stopping rule (Lin 2007): grad = X G - R, an
-// entry counting where x_ij > 0 and, where x_ij = 0, only if negative; squares
-// summed in FP32 per row, FP64 across rows, per-CTA partials added in a fixed
-// order.
+// MU where the last wave of tiles would be too empty: lane l holds entries l, l +
+// 32, ... (KW slots), G in FP32 in shared memory lane-interleaved (entry (r, c) at
+// r * 32 KW + (c % 32) * KW + c / 32) so that a lane reads its KW entries of a row
+// as one vector; MU forms X G with one product, HALS each coordinate's sum with a
+// butterfly. It also forms the projected-gradient norm of the stopping rule (Lin
+// 2007): grad = X G - R, an entry counting where x_ij > 0 and, where x_ij = 0, only
+// if negative; squares summed in FP32 per row, FP64 across rows, per-CTA partials
+// added in a fixed order. The two kernels' sums round differently: a row's last
+// bits depend on how many rows the call has.
 //
 // Roofline: HBM (12 k bytes per row: R and X in, X out); 2 k^2 FLOPs per row.
 // The tile kernel is bound by the latency of its instruction stream (some ten
